@@ -133,6 +133,8 @@ void fill_consts(Consts &k)
     for (int i = 1; i < 192; ++i) k.inv_int[i] = (double)(1.0L / (long double)i);
     k.inv_int_lo[0] = 0.0;
     for (int i = 1; i < 64; ++i) k.inv_int_lo[i] = (double)(1.0L / (long double)i - (long double)k.inv_int[i]);
+    for (int l = 1; l < 16; ++l)
+        for (int m = 0; m <= l; ++m) k.kappa[l][m] = (double)((long double)(l * l - m * m) / (4 * l * l - 1));
     long double df = 1;
     for (int n = 0; n < 32; ++n) {
         k.dfact[n] = (double)df;                 // (2n-1)!!
@@ -300,6 +302,65 @@ static void gauss_legendre(int n, std::vector<long double> &x, std::vector<long 
         x[i] = t;
         w[i] = 2 / ((1 - t * t) * dp * dp);
     }
+}
+
+// Coefficients of the expanded angular part (layout at CGTab).  With S_{l,+-m} = nu_{l,m} p_{l,m}(z, r^2) {C_m, S_m},
+// nu_{l,m} = sqrt((2 - delta_{m0}) (l-m)!/(l+m)!) (2l-1)!!/(l-m)!, the product of the two theta functions is
+// expanded in those of (L, M) by Gauss-Legendre quadrature exact for the degrees (<= 2 (kLmaxAabA + kLmax2c)).
+static void make_cg(std::vector<double> &g, std::vector<int> &gbase, std::vector<double> &fc)
+{
+    const int lmax = kLmaxAabA + kLmax2c, nq = 24;
+    std::vector<long double> x, w;
+    gauss_legendre(nq, x, w);
+    // theta functions nu p sin^m at the nodes, and nu
+    std::vector<long double> th((size_t)(lmax + 1) * (lmax + 1) * nq, 0), nu((size_t)(lmax + 1) * (lmax + 1), 0);
+    for (int l = 0; l <= lmax; ++l)
+        for (int m = 0; m <= l; ++m) {
+            long double odd = 1;
+            for (int i = 2 * l - 1; i > 1; i -= 2) odd *= i;
+            nu[l * (lmax + 1) + m] = std::sqrt((m ? 2 : 1) * lfact(l - m) / lfact(l + m)) * odd / lfact(l - m);
+        }
+    for (int q = 0; q < nq; ++q)
+        for (int m = 0; m <= lmax; ++m) {
+            long double p0 = 0, p1 = 1, sm = 1;
+            const long double s = std::sqrt(1 - x[q] * x[q]);
+            for (int i = 0; i < m; ++i) sm *= s;
+            for (int l = m; l <= lmax; ++l) {
+                th[((size_t)l * (lmax + 1) + m) * nq + q] = nu[l * (lmax + 1) + m] * p1 * sm;
+                const long double n = x[q] * p1 - (long double)(l * l - m * m) / (4 * l * l - 1) * p0;
+                p0 = p1;
+                p1 = n;
+            }
+        }
+    auto theta = [&](int l, int m) { return &th[((size_t)l * (lmax + 1) + m) * nq]; };
+    gbase.assign(kNClassCG, 0);
+    fc.assign((size_t)kNClassCG * 28, 0.0);
+    g.clear();
+    for (int la = 0; la <= kLmaxAabA; ++la)
+        for (int lb = 0; lb <= kLmax2c; ++lb) {
+            const int J = std::min(la, lb) + 1, c = la * (kLmax2c + 1) + lb;
+            gbase[c] = (int)g.size();
+            for (int a = 0; a <= la; ++a)
+                for (int b = 0; b <= lb; ++b)
+                    for (int s = 0; s < 2; ++s)
+                        for (int p = 0; p < J; ++p) {
+                            const int L = la + lb - 2 * p, M = s ? a + b : std::abs(a - b);
+                            long double v = 0;
+                            if (M <= L && !(s && (!a || !b))) {
+                                const long double *ta = theta(la, a), *tb = theta(lb, b), *tL = theta(L, M);
+                                for (int q = 0; q < nq; ++q) v += w[q] * ta[q] * tb[q] * tL[q];
+                                v *= (2 * L + 1) / (M ? 4.0L : 2.0L) * nu[L * (lmax + 1) + M] * (a && b ? 0.5L : 1.0L);
+                            }
+                            g.push_back((double)v);
+                        }
+            for (int p = 0; p < J; ++p)
+                for (int j = 0; j <= p; ++j) {
+                    const int L = la + lb - 2 * p, i = p - j;
+                    long double v = lfact(p) / (lfact(i) * lfact(p - i)) * std::ldexp((lb & 1) ? -1.0L : 1.0L, la + lb);
+                    for (int q = i; q < p; ++q) v *= L + 1.5L + q;
+                    fc[(size_t)c * 28 + p * (p + 1) / 2 + j] = (double)v;
+                }
+        }
 }
 
 // Real Gaunt coefficients G = int Y_{L,M} Y_{l,m} Y_{l~,m~} dOmega for
@@ -522,11 +583,25 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
                  cudaMemcpy(d_gr, gr.data(), gr.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
                  cudaMemcpy(d_ge, ge.data(), ge.size() * sizeof(GauntEnt), cudaMemcpyHostToDevice) == cudaSuccess;
         }
+        double *d_cg = nullptr, *d_fc = nullptr;
+        int *d_cgb = nullptr;
+        if (ok) {
+            std::vector<double> cg, fc;
+            std::vector<int> cgb;
+            make_cg(cg, cgb, fc);
+            ok = cudaMalloc(&d_cg, cg.size() * sizeof(double)) == cudaSuccess &&
+                 cudaMalloc(&d_fc, fc.size() * sizeof(double)) == cudaSuccess &&
+                 cudaMalloc(&d_cgb, cgb.size() * sizeof(int)) == cudaSuccess &&
+                 cudaMemcpy(d_cg, cg.data(), cg.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+                 cudaMemcpy(d_fc, fc.data(), fc.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
+                 cudaMemcpy(d_cgb, cgb.data(), cgb.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
+        }
         if (!ok) {
             fail(SHG_ECUDA, "device tables: upload failed");
             return nullptr;
         }
         st.bin_rank3 = d_r3;
+        st.t.cg = CGTab{d_cg, d_cgb, d_fc};
         st.t.gaunt_base = d_gb;
         st.t.gaunt_row = d_gr;
         st.t.gaunt = d_ge;
@@ -1253,6 +1328,7 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     a.boys = t->boys;
     a.boys_e = t->boys_e;
     a.o_pre = o_pre;
+    a.cg = t->cg;
     a.k = consts();
     if (p->d.schedule == SHG_SCHED_PERSISTENT) {
         a.tile_begin = 0;
@@ -1299,6 +1375,7 @@ static int exec_fp64_static_range(shg_plan_t *p, int op, double omega, double sc
     a.boys = t->boys;
     a.boys_e = t->boys_e;
     a.o_pre = nullptr;
+    a.cg = t->cg;
     a.k = consts();
     a.tile_begin = tile_begin;
     a.tile_end = tile_end;
@@ -1361,6 +1438,7 @@ int shg_plan_2c_exec_fused(shg_plan_t *p, int n_ops, const int *ops, const doubl
     a.boys = t->boys;
     a.boys_e = t->boys_e;
     a.cprims = p->d.basis->cprims;
+    a.cg = t->cg;
     a.k = consts();
     const bool mixed = precision == SHG_PREC_MIXED;
     const bool persistent = p->d.schedule == SHG_SCHED_PERSISTENT;

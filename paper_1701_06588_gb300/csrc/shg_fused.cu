@@ -16,7 +16,7 @@
 //
 // Work mapping as the single-operator kernel: one thread per shell pair, a
 // warp per class-pure tile of up to 32 pairs, tiles from the same plan.
-#include "shg_device.cuh"
+#include "shg_cg.cuh"
 
 namespace shg {
 namespace {
@@ -170,67 +170,20 @@ __device__ void pair_2c_fused(const ArgsFused &g, int p)
             t *= -0.5 * ir2 * g.k.dint[2 * (kmax - j) + 1];
         }
     }
-    // erfc = coulomb - attenuated; then every operator's orders scaled by 2^{kmax-j}
+    // erfc = coulomb - attenuated
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const double p2 = g.k.pow2[kmax - j];
-        Ox[j] = (Oco[j] - (f_x ? Ox[j] : Oer[j])) * p2;
-        Oov[j] *= p2;
-        Oco[j] *= p2;
-        Oer[j] *= p2;
-        Oga[j] *= p2;
-    }
+    for (int j = 0; j < J; ++j) Ox[j] = Oco[j] - (f_x ? Ox[j] : Oer[j]);
 
-    double Rc[(kLmax2c + 1) * (kLmax2c + 2) / 2], Rs[(kLmax2c + 1) * (kLmax2c + 2) / 2];
-    scaled_harmonics(vx, vy, vz, la > lb ? la : lb, g.k, Rc, Rs);
-    const int nb = 2 * lb + 1;
-    double Wb[2 * kLmax2c + 1][J * J];
-    for (int mb = -lb; mb <= lb; ++mb) {
-        double w[J * J];
-        w_row<J>(Rc, Rs, lb, mb, w);
-#pragma unroll
-        for (int e = 0; e < J * J; ++e) Wb[mb + lb][e] = w[e];
-    }
-    const double sgn_b = (lb & 1) ? -1.0 : 1.0;
+    double P[cg::kNP2], PF[cg::kNP2], C[2 * kLmax2c + 1], S[2 * kLmax2c + 1];
+    cg::harmonics(vx, vy, vz, R2, kmax, J, g.k, P, C, S);
     const long long o = g.out_off[p];
-    for (int ma = -la; ma <= la; ++ma) {
-        double ua[J * J];
-        w_row<J>(Rc, Rs, la, ma, ua);
+    for (int op = 0; op < 5; ++op) {
+        if (!g.out[op]) continue;
+        double O[J];
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-#pragma unroll
-            for (int kp = 0; kp <= j; ++kp) {
-                const int e0 = j * j + (kp == 0 ? 0 : 2 * kp - 1);
-                ua[e0] *= g.k.jB[j][kp];
-                if (kp) ua[e0 + 1] *= g.k.jB[j][kp];
-            }
-        }
-        const double Aa = g.k.A[la][ma < 0 ? -ma : ma] * sgn_b;
-        for (int mb = -lb; mb <= lb; ++mb) {
-            // Q_j[ma][mb] for j = 0..J-1 (block j holds the 2j+1 entries e = j^2 .. j^2+2j)
-            double Q[J];
-#pragma unroll
-            for (int j = 0; j < J; ++j) {
-                double s = 0.0;
-#pragma unroll
-                for (int e = j * j; e < (j + 1) * (j + 1); ++e) s = fma(ua[e], Wb[mb + lb][e], s);
-                Q[j] = s;
-            }
-            const double aa = Aa * g.k.A[lb][mb < 0 ? -mb : mb];
-            const long long idx = o + (ma + la) * nb + (mb + lb);
-#define SHG_FUSED_STORE(OPID, ARR)                                          \
-    if (g.out[OPID]) {                                                      \
-        double s = 0.0;                                                     \
-        _Pragma("unroll") for (int j = 0; j < J; ++j) s = fma(ARR[j], Q[j], s); \
-        g.out[OPID][idx] = aa * s;                                          \
-    }
-            SHG_FUSED_STORE(OP_OVERLAP, Oov)
-            SHG_FUSED_STORE(OP_COULOMB, Oco)
-            SHG_FUSED_STORE(OP_ERFC, Ox)
-            SHG_FUSED_STORE(OP_ERF, Oer)
-            SHG_FUSED_STORE(OP_GAUSS, Oga)
-#undef SHG_FUSED_STORE
-        }
+        for (int j = 0; j < J; ++j)
+            O[j] = op == OP_OVERLAP ? Oov[j] : op == OP_COULOMB ? Oco[j] : op == OP_ERFC ? Ox[j] : op == OP_ERF ? Oer[j] : Oga[j];
+        cg::block_from_orders<J>(g.cg, la, lb, R2, O, P, C, S, PF, g.out[op] + o);
     }
 }
 

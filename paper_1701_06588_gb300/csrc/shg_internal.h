@@ -99,6 +99,7 @@ struct Consts {
     // the double-double (a|r_a^{2n}|b) path
     double jB_lo[kJmax][kJmax];
     double inv_int_lo[64];
+    double kappa[16][16];                  // (l^2 - m^2) / (4 l^2 - 1): recursion of the monic Legendre functions
 };
 
 void fill_consts(Consts &k);
@@ -116,6 +117,18 @@ struct ConstsMix {
 
 void fill_consts_mix(ConstsMix &k);
 
+// Coefficients of the expanded angular part (shg_cg.cuh), per class (la, lb) with la <= kLmaxAabA, lb <= kLmax2c, class
+// index c = la (kLmax2c + 1) + lb, J = min(la, lb) + 1:
+//   g + gbase[c]: for every (|ma|, |mb|), row-major, J coefficients g1 of |M| = ||ma| - |mb|| and J of |M| = |ma| + |mb|
+//   (p = 0..J-1, L = la + lb - 2p; 0 where L < |M|), with the norm nu_{L,M} of p_{L,M} in them
+//   fc + 28 c: coefficient of R^{2(p-j)} O^{(la+lb-j)} in F_p at p (p + 1) / 2 + j, with (-1)^lb 2^{la+lb} in it
+constexpr int kNClassCG = (kLmaxAabA + 1) * (kLmax2c + 1);
+struct CGTab {
+    const double *g;
+    const int *gbase;
+    const double *fc;
+};
+
 // Device-resident tables owned by the library, one set per device.
 struct DeviceTables {
     const double *boys;   // [kBoysGrid][kBoysN][kBoysStride] (layout above)
@@ -127,6 +140,7 @@ struct DeviceTables {
     const GauntEnt *gaunt;     // entries
     const float4 *boys_mix;    // [kBoysGrid][kBoysN][3] (layout above)
     const float2 *boys_e_mix;  // [kBoysGrid] exp(-T_i) as hi/lo
+    CGTab cg;
 };
 
 // Extra constants of the three-index kernels (by value).
@@ -246,6 +260,7 @@ struct Args2c {
     // family path: contracted radial terms O[j] of pair p precomputed at
     // o_pre[p * kJmax + j] (read by the OP_PRE instantiation only)
     const double *o_pre = nullptr;
+    CGTab cg;
     Consts k;
 };
 
@@ -267,6 +282,7 @@ struct ArgsFused {
     int share_att;                // erf and erfc requested with the same omega
     const double *boys, *boys_e;
     const CoulPrim *cprims;       // Coulomb-type weights per primitive
+    CGTab cg;
     Consts k;
 };
 

@@ -14,7 +14,7 @@
 // tile of up to 32 pairs of one (la, lb) class with similar Ka*Kb, so the
 // lanes run the same loop trip counts.
 
-#include "shg_device.cuh"
+#include "shg_cg.cuh"
 
 #include <cstdio>
 
@@ -62,46 +62,9 @@ __device__ void pair_2c_fp64(const Args2c &g, int p)
         radial_finish_fp64<OP, J>(R2, kmax, g.k, O, E);
     }
 
-    // g_e = 2^{kmax-j} (2j-1)!! B_{j,kappa} O^{(kmax-j)}, shared by z = c, s
-    double ge[J * J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const double oj = O[j] * g.k.pow2[kmax - j];
-#pragma unroll
-        for (int kp = 0; kp <= j; ++kp) {
-            const double v = oj * g.k.jB[j][kp];
-            const int e0 = j * j + (kp == 0 ? 0 : 2 * kp - 1);
-            ge[e0] = v;
-            if (kp) ge[e0 + 1] = v;
-        }
-    }
-
-    double Rc[(kLmax2c + 1) * (kLmax2c + 2) / 2], Rs[(kLmax2c + 1) * (kLmax2c + 2) / 2];
-    scaled_harmonics(vx, vy, vz, la > lb ? la : lb, g.k, Rc, Rs);
-
-    const int nb = 2 * lb + 1;
-    double Ub[2 * kLmax2c + 1][J * J];
-    for (int mb = -lb; mb <= lb; ++mb) {
-        double w[J * J];
-        w_row<J>(Rc, Rs, lb, mb, w);
-#pragma unroll
-        for (int e = 0; e < J * J; ++e) Ub[mb + lb][e] = w[e];
-    }
-    const double sgn_b = (lb & 1) ? -1.0 : 1.0;
-    double *out = g.out + g.out_off[p];
-    for (int ma = -la; ma <= la; ++ma) {
-        double ua[J * J];
-        w_row<J>(Rc, Rs, la, ma, ua);
-#pragma unroll
-        for (int e = 0; e < J * J; ++e) ua[e] *= ge[e];
-        const double Aa = g.k.A[la][ma < 0 ? -ma : ma] * sgn_b;
-        for (int mb = -lb; mb <= lb; ++mb) {
-            double s = 0.0;
-#pragma unroll
-            for (int e = 0; e < J * J; ++e) s = fma(ua[e], Ub[mb + lb][e], s);
-            out[(ma + la) * nb + (mb + lb)] = Aa * (g.k.A[lb][mb < 0 ? -mb : mb] * s);
-        }
-    }
+    double P[cg::kNP2], PF[cg::kNP2], C[2 * kLmax2c + 1], S[2 * kLmax2c + 1];
+    cg::harmonics(vx, vy, vz, R2, kmax, J, g.k, P, C, S);
+    cg::block_from_orders<J>(g.cg, la, lb, R2, O, P, C, S, PF, g.out + g.out_off[p]);
 }
 
 // ------------------------------------------------------------------------- //

@@ -137,6 +137,7 @@ extern "C" int shg_eval_2c_noalloc(const shg_basis_t *basis, int64_t n_pairs, co
     a.screen = b.screen;
     a.boys = t->boys;
     a.boys_e = t->boys_e;
+    a.cg = t->cg;
     a.k = consts();
     e = cudaMemsetAsync(plan.counter, 0, sizeof(int), s);
     if (e == cudaSuccess) e = launch_2c(a, op, precision, persistent_grid_2c(op, precision), true, s);
