@@ -190,17 +190,17 @@ int shg_plan_2c_exec(shg_plan_t *plan, int op, double omega, double screen_thres
                      const int64_t *d_out_offsets, double *d_out, void *stream);
 
 /*
- * shg_plan_2c_set_variant - compiled variant of the persistent fused kernel
- * used by later fused executions of the plan (an autotuner knob).
- *   FP64:  0 = registers as the compiler allocates them (253 per thread),
- *          1 = at most 170 (three 128-thread CTAs per SM), 2 = at most 128
- *          (four); the capped variants spill some values to local memory.
- *   mixed: 0 = registers as the compiler allocates them (about 124),
- *          1 = at most 96 (five 128-thread CTAs per SM), 2 = at most 85 (six).
- * A new plan uses variant 1 (the fastest of the three on GB300 for both
- * precisions on the 2M-pair workload).  The variants run the same operations
- * in the same order, so the results are bitwise equal.  SHG_EINVAL for a
- * value outside 0..2.
+ * shg_plan_2c_set_variant - register cap of the two-center kernels used by
+ * later executions of the plan (an autotuner knob), as 128-thread CTAs that
+ * must fit on an SM; capped kernels spill some values to local memory.
+ *   1/r and erfc, alone or together:   0 = four CTAs, 1 = eight, 2 = six
+ *   other sets of operators, FP64:     0 = three,     1 = six,   2 = four
+ *   other sets of operators, mixed:    0 = four,      1 = six,   2 = five
+ * A new plan takes 1 when more than two thirds of its work units are of
+ * classes with min(la, lb) <= 1 (few accumulators: more warps hide their
+ * latency) and 0 otherwise.  The variants run the same operations in the same
+ * order, so the results are bitwise equal.  SHG_EINVAL for a value outside
+ * 0..2.
  */
 int shg_plan_2c_set_variant(shg_plan_t *plan, int variant);
 

@@ -2,6 +2,7 @@
 // normalisation, device tables, planning and kernel dispatch.
 #include "../../include/shg.h"
 #include "shg_internal.h"
+#include "shg_xf.cuh"
 
 #include <algorithm>
 #include <string>
@@ -180,6 +181,76 @@ void make_boys_table(int per_unit, int ngrid, int nterms, double *tab, double *e
             }
         }
         etab[i] = (double)e;
+    }
+}
+
+// Extended floats from host values: FP64 (also denormal) and double-double, > 0
+static xfp::xf xf_of(dd v)
+{
+    int x;
+    const double f = std::frexp(v.hi, &x);                       // [1/2, 1)
+    int64_t m = (int64_t)std::ldexp(f, 63) + (int64_t)std::llrint(std::ldexp(v.lo, 63 - x));
+    if (m < 0) m = INT64_MAX;                                    // hi rounded up to a power of two
+    int e = x - 63;
+    if (m < (1ll << 62)) {                                       // hi a power of two, lo < 0
+        m *= 2;
+        --e;
+    }
+    return xfp::xf{(uint64_t)m, e};
+}
+
+static XOmega x_omega(double w)
+{
+    if (!(w > 0)) return XOmega{1ull << 62, 1ull << 62, -62, -62};
+    const xfp::xf a = xf_of(dd{w, 0.0}), b = xfp::mul(a, a);
+    return XOmega{a.m, b.m, a.e, b.e};
+}
+
+// Table of BoysEnt (layout there): at the coarse points T_i = i/32 the power series of F_48 and the downward recursion
+// in long double; at the 16 nodes k/512 around each, F_20 by its Taylor series (|d| <= 1/64, ten terms) and downward.
+static void make_boys_cells(std::vector<BoysEnt> &tab)
+{
+    const int ntop = 48, nf = 20;
+    tab.assign((size_t)kBoysCells * kBoysOrders, BoysEnt{});
+#pragma omp parallel for schedule(dynamic, 16)
+    for (int i = 0; i <= kBoysCells / 16; ++i) {
+        const long double T = (long double)i / 32;
+        const long double e = std::exp(-T);
+        long double term = 1.0L / (2 * ntop + 1), sum = term;
+        for (int k = 1; k < 20000; ++k) {
+            term *= 2 * T / (long double)(2 * ntop + 2 * k + 1);
+            sum += term;
+            if (term < sum * 1e-24L) break;
+        }
+        long double F[ntop + 1];
+        F[ntop] = e * sum;
+        for (int n = ntop; n > 0; --n) F[n - 1] = (2 * T * F[n] + e) / (long double)(2 * n - 1);
+        for (int k = 16 * i - 8; k < 16 * i + 8; ++k) {
+            if (k < 1 || k > kBoysCells) continue;
+            const long double d = T - (long double)k / 512, Tk = (long double)k / 512;
+            long double G[nf + 1], pw = 1;
+            G[nf] = 0;
+            for (int t = 0; t <= 10; ++t) {
+                G[nf] += F[nf + t] * pw;
+                pw *= d / (t + 1);
+            }
+            const long double ek = std::exp(-Tk);
+            for (int n = nf; n > 0; --n) G[n - 1] = (2 * Tk * G[n] + ek) / (long double)(2 * n - 1);
+            for (int n = 0; n < kBoysOrders; ++n) {
+                int x;
+                const long double f = std::frexp(G[n], &x);
+                const int s = f < 1 - 1.0L / 256 ? 63 - x : 62 - x;
+                auto fix = [&](int t, long double fac, int unit) {
+                    return (uint64_t)std::rint(std::ldexp(G[n + t] / fac, s - unit));
+                };
+                BoysEnt &b = tab[(size_t)n * kBoysCells + (k - 1)];
+                b.c0 = fix(0, 1, 0);
+                b.c1 = fix(1, 1, 0);
+                b.c2 = ((fix(2, 2, 0) + 128) & ~255ull) | (uint64_t)(s - 62);
+                b.c3 = (uint32_t)fix(3, 6, 30);
+                b.c45 = (uint32_t)fix(4, 24, 35) | (uint32_t)(fix(5, 120, 49) << 24);
+            }
+        }
     }
 }
 
@@ -433,6 +504,8 @@ static double class_cost3(int la, int lt, int lb, int kk)
     return kk * rad + ang + (2.0 * la + 1) * (2 * lt + 1) * (2 * lb + 1) * nL * 2;
 }
 
+static uint8_t g_chunk_class[2][kNClass];   // class of every chunk of a schedule's rank order (the same on all devices)
+
 static std::mutex g_mu;
 static DevState g_dev[64];
 
@@ -543,6 +616,7 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
         for (int s = 0; s < 2 && ok; ++s) {
             std::vector<int> rank, inv;
             make_ranks(s, rank, inv);
+            for (int c = 0; c < kNClass; ++c) g_chunk_class[s][c] = (uint8_t)(inv[(size_t)c * kKbins2c] / kKbins2c);
             rank.insert(rank.end(), inv.begin(), inv.end());
             ok = cudaMemcpy(d_r[s], rank.data(), rank.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
         }
@@ -584,24 +658,42 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
                  cudaMemcpy(d_ge, ge.data(), ge.size() * sizeof(GauntEnt), cudaMemcpyHostToDevice) == cudaSuccess;
         }
         double *d_cg = nullptr, *d_fc = nullptr;
+        float2 *d_cgm = nullptr;
         int *d_cgb = nullptr;
         if (ok) {
             std::vector<double> cg, fc;
             std::vector<int> cgb;
             make_cg(cg, cgb, fc);
+            std::vector<float2> cgm(cg.size());
+            for (size_t i = 0; i < cg.size(); ++i) cgm[i] = split2d(cg[i]);
             ok = cudaMalloc(&d_cg, cg.size() * sizeof(double)) == cudaSuccess &&
                  cudaMalloc(&d_fc, fc.size() * sizeof(double)) == cudaSuccess &&
+                 cudaMalloc(&d_cgm, cgm.size() * sizeof(float2)) == cudaSuccess &&
+                 cudaMemcpy(d_cgm, cgm.data(), cgm.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
                  cudaMalloc(&d_cgb, cgb.size() * sizeof(int)) == cudaSuccess &&
                  cudaMemcpy(d_cg, cg.data(), cg.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
                  cudaMemcpy(d_fc, fc.data(), fc.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
                  cudaMemcpy(d_cgb, cgb.data(), cgb.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
+        }
+        BoysEnt *d_bc = nullptr;
+        uint64_t *d_ex = nullptr;
+        if (ok) {
+            std::vector<BoysEnt> bc;
+            make_boys_cells(bc);
+            uint64_t ex[kExpTab];
+            for (int j = 0; j < kExpTab; ++j) ex[j] = (uint64_t)std::rint(std::ldexp(std::exp((long double)j / 512), 62));
+            ok = cudaMalloc(&d_bc, bc.size() * sizeof(BoysEnt)) == cudaSuccess &&
+                 cudaMalloc(&d_ex, sizeof ex) == cudaSuccess &&
+                 cudaMemcpy(d_bc, bc.data(), bc.size() * sizeof(BoysEnt), cudaMemcpyHostToDevice) == cudaSuccess &&
+                 cudaMemcpy(d_ex, ex, sizeof ex, cudaMemcpyHostToDevice) == cudaSuccess;
         }
         if (!ok) {
             fail(SHG_ECUDA, "device tables: upload failed");
             return nullptr;
         }
         st.bin_rank3 = d_r3;
-        st.t.cg = CGTab{d_cg, d_cgb, d_fc};
+        st.t.cg = CGTab{d_cg, d_cgb, d_fc, d_cgm};
+        st.t.x = XTab{d_bc, d_ex};
         st.t.gaunt_base = d_gb;
         st.t.gaunt_row = d_gr;
         st.t.gaunt = d_ge;
@@ -659,6 +751,13 @@ const Consts &consts()
     static std::once_flag once;
     std::call_once(once, [] { fill_consts(k); });
     return k;
+}
+
+static void fill_kappa_mix(KappaMix &k)
+{
+    for (int l = 0; l < 16; ++l)
+        for (int m = 0; m < 16; ++m)
+            k.v[l][m] = l && m <= l ? split2((long double)(l * l - m * m) / (4 * l * l - 1)) : make_float2(0, 0);
 }
 
 static bool is_finite_d(double x) { return std::isfinite(x); }
@@ -728,6 +827,7 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
     std::vector<ShellRec> sh(n_shells);
     std::vector<PrimRec> pr(n_prims);
     std::vector<CoulPrim> cpr(n_prims);
+    std::vector<XPrim> xpr(n_prims);
     std::vector<int64_t> first(n_shells + 1, 0);
     for (int s = 0; s < n_shells; ++s) first[s + 1] = first[s] + nprim[s];
     // per-l constants: sqrt(pi) (2l+2)! / (2^{2l+3} (l+1)!) and K_l = sqrt((2l+1)/(4 pi))
@@ -781,7 +881,15 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
             const dd cw = dd_mul(w2c, ia);
             // sqrt(2 pi^{5/2}) folded into cw: pre = cw_a cw_b / sqrt(c)
             const dd s2p52 = dd_sqrt(dd_from(2.0L * 17.493418327624862846262821679871554L));   // 2 pi^{5/2}
-            cpr[off + i] = CoulPrim{dd_mul(cw, s2p52).hi, dd_mul(cw, dd_sqrt(ia)).hi};
+            const dd cws = dd_mul(cw, s2p52);
+            cpr[off + i] = CoulPrim{cws.hi, dd_mul(cw, dd_sqrt(ia)).hi};
+            const xfp::xf xa = xf_of(dd{a, 0.0});
+            // a zero weight: a value so small that every term it enters is flushed to 0 (and one that overflowed FP64
+            // gives infinities)
+            const xfp::xf xw = cws.hi == 0 || !std::isfinite(cws.hi)
+                                       ? xfp::xf{1ull << 62, cws.hi == 0 ? -1000000 : 1000000}
+                                       : xf_of(cws.hi < 0 ? dd{-cws.hi, -cws.lo} : cws);
+            xpr[off + i] = XPrim{xa.m, xw.m | (cws.hi < 0 ? 1ull << 63 : 0), xa.e, xw.e, cpr[off + i].fw};
         }
         sh[s] = ShellRec{L, K, (int)off, center_of_shell[s]};
     }
@@ -856,6 +964,7 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
         cudaMalloc(&d.centers, sizeof(Vec4) * n_centers) != cudaSuccess ||
         cudaMalloc(&d.mprims, sizeof(MixPrim) * n_prims) != cudaSuccess ||
         cudaMalloc(&d.cprims, sizeof(CoulPrim) * n_prims) != cudaSuccess ||
+        cudaMalloc(&d.xprims, sizeof(XPrim) * n_prims) != cudaSuccess ||
         cudaMalloc(&d.screen, sizeof(ScreenRec) * n_shells) != cudaSuccess ||
         cudaMalloc(&d.mcenters, sizeof(MixCenter) * n_centers) != cudaSuccess) {
         shg_basis_destroy(b);
@@ -866,6 +975,7 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
         cudaMemcpy(d.centers, ctr.data(), sizeof(Vec4) * n_centers, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.mprims, mpr.data(), sizeof(MixPrim) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.cprims, cpr.data(), sizeof(CoulPrim) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(d.xprims, xpr.data(), sizeof(XPrim) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.screen, scr.data(), sizeof(ScreenRec) * n_shells, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.mcenters, mctr.data(), sizeof(MixCenter) * n_centers, cudaMemcpyHostToDevice) != cudaSuccess) {
         shg_basis_destroy(b);
@@ -926,6 +1036,7 @@ void shg_basis_destroy(shg_basis_t *b)
     cudaFree(b->d.centers);
     cudaFree(b->d.mprims);
     cudaFree(b->d.cprims);
+    cudaFree(b->d.xprims);
     cudaFree(b->d.mcenters);
     cudaFree(b->d.screen);
     cudaFree(b->d.stage_raw);
@@ -974,6 +1085,41 @@ int64_t shg_triple_offsets(const shg_basis_t *orb, const shg_basis_t *aux, int64
     return tot;
 }
 
+} // extern "C"
+int shg::plan_read(PlanDev &d, const int *summary, int schedule)
+{
+    if (summary[kNClass + 1])
+        return fail(SHG_EINVAL, "pair list holds a shell index outside 0..%d", d.basis->n_shells - 1);
+    d.n_tiles = summary[kNClass];
+    for (int c = 0; c <= kNClass; ++c) d.class_tile_begin[c] = summary[c];
+    const int *first = summary + kNClass + 2;
+    TileMap &m = d.map;
+    m.tile[0] = 0;
+    for (int c = 0; c < kNClass; ++c) {
+        m.pair[c] = first[c];
+        m.pair[c + 1] = c + 1 < kNClass ? first[c + 1] : (int)d.n_pairs;
+        m.tile[c + 1] = m.tile[c] + (m.pair[c + 1] - m.pair[c] + kTile - 1) / kTile;
+        m.cls[c] = g_chunk_class[schedule][c];
+    }
+    // register cap: with more registers per thread the accumulators of high J stay in registers, with fewer more warps
+    // hide the latency of the low-J classes (J <= 2), which need few
+    int low = 0;
+    for (int c = 0; c < kNClass; ++c)
+        if (std::min(m.cls[c] / 7, m.cls[c] % 7) <= 1) low += summary[c + 1] - summary[c];
+    d.variant = 3 * (int64_t)low > 2 * (int64_t)d.n_tiles ? 1 : 0;
+    d.mixed_fp64_tiles = d.mixed_fp64_tiles32 = 0;
+    if (schedule == SHG_SCHED_PERSISTENT) {
+        // the persistent rank order is J-major (J descending), so the classes with
+        // both l >= kMixedFp64MinL are its first chunks
+        int n_hi = 0;
+        for (int cls = 0; cls < kNClass; ++cls) n_hi += mixed_runs_fp64(cls);
+        d.mixed_fp64_tiles = summary[n_hi];
+        d.mixed_fp64_tiles32 = m.tile[n_hi];
+    }
+    return SHG_OK;
+}
+extern "C" {
+
 int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, const int32_t *pb, int schedule,
                        void *stream, shg_plan_t **out)
 {
@@ -992,7 +1138,7 @@ int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, c
     if (!device_tables_impl(ranks)) return SHG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
-    const int64_t max_tiles = n / kTile + std::min<int64_t>(n, kNBins) + 1;
+    const int64_t max_tiles = plan_max_tiles(n, kNClass, true);
     const size_t bytes_perm = sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1);
     const size_t bytes_tiles = sizeof(Tile) * (size_t)max_tiles;
     const size_t bytes_ws = sizeof(int) * plan_ws_ints(n, kNBins, kNClass);
@@ -1026,23 +1172,12 @@ int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, c
     };
     cudaError_t e = launch_plan_build(d, ws, kNBins, ranks[schedule], s);
     if (e != cudaSuccess) return cleanup(fail(SHG_ECUDA, "plan build: %s", cudaGetErrorString(e)));
-    // first tile of every class chunk, the tile count and the error flag, in one read-back
-    int chunk_tile[kNClass + 2];
-    if (cudaMemcpyAsync(chunk_tile, plan_summary(ws, kNBins), sizeof(chunk_tile), cudaMemcpyDeviceToHost, s) !=
-            cudaSuccess ||
+    // first tile and first pair of every class chunk, the tile count and the error flag, in one read-back
+    int summary[2 * kNClass + 2];
+    if (cudaMemcpyAsync(summary, plan_summary(ws, kNBins), sizeof(summary), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return cleanup(fail(SHG_ECUDA, "plan build: %s", cudaGetErrorString(cudaGetLastError())));
-    if (chunk_tile[kNClass + 1])
-        return cleanup(fail(SHG_EINVAL, "pair list holds a shell index outside 0..%d", basis->d.n_shells - 1));
-    d.n_tiles = chunk_tile[kNClass];
-    for (int cls = 0; cls <= kNClass; ++cls) d.class_tile_begin[cls] = chunk_tile[cls];
-    if (schedule == SHG_SCHED_PERSISTENT) {
-        // the persistent rank order is J-major (J descending), so the classes with
-        // both l >= kMixedFp64MinL are its first chunks
-        int n_hi = 0;
-        for (int cls = 0; cls < kNClass; ++cls) n_hi += mixed_runs_fp64(cls);
-        d.mixed_fp64_tiles = chunk_tile[n_hi];
-    }
+    if ((r = plan_read(d, summary, schedule)) != SHG_OK) return cleanup(r);
     if (schedule == SHG_SCHED_PERSISTENT) {
         p->launches = d.n_tiles > 0 ? 1 : 0;
     } else {
@@ -1227,9 +1362,9 @@ static int join_sides(shg_plan_t *p, cudaStream_t s)
 // mixed-precision passes run in FP64
 enum { kAllClasses = 0, kMixedFp64Classes = 1 };
 static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const int64_t *off, double *out,
-                     const double *o_pre, cudaStream_t s, int sel = kAllClasses);
-static int exec_fp64_static_range(shg_plan_t *p, int op, double omega, double screen, const int64_t *off,
-                                  double *out, int tile_begin, int tile_end, cudaStream_t s);
+                     const double *o_pre, cudaStream_t s);
+static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, int sel, int variant, cudaStream_t s);
+static int exec_mixed(shg_plan_t *p, const ArgsFused &f, cudaStream_t s);
 
 int shg_plan_2c_exec(shg_plan_t *p, int op, double omega, double screen, int precision, const int64_t *off,
                      double *out, void *stream)
@@ -1248,70 +1383,72 @@ int shg_plan_2c_exec(shg_plan_t *p, int op, double omega, double screen, int pre
     if (!t) return SHG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
     if (precision == SHG_PREC_MIXED) {
-        ArgsMix m;
-        m.shells = p->d.basis->shells;
-        m.prims = p->d.basis->mprims;
-        m.centers = p->d.basis->mcenters;
-        m.pair_a = p->d.pair_a;
-        m.pair_b = p->d.pair_b;
-        m.perm = p->d.perm;
-        m.tiles = p->d.tiles;
-        m.out_off = reinterpret_cast<const long long *>(off);
-        m.out = out;
-        m.omega = split2(omega);
-        m.omega2 = split2((long double)omega * omega);
-        m.omega_d = omega;
-        m.screen_thresh = screen;
-        m.screen = p->d.basis->screen;
-        m.boys = t->boys_mix;
-        m.boys_e = t->boys_e_mix;
-        m.km = consts_mix();
-        // classes with both l >= kMixedFp64MinL in FP64: beside the double-float
-        // launch on the side streams (persistent plans holding both kinds), else first
-        const bool fork = p->d.schedule == SHG_SCHED_PERSISTENT && p->d.mixed_fp64_tiles > 0 &&
-                          p->d.n_tiles > p->d.mixed_fp64_tiles;
-        if (fork) {
-            r = fork_sides(p, s);
-            if (r) return r;
-            r = exec_fp64_static_range(p, op, omega, screen, off, out, 0, p->d.mixed_fp64_tiles, p->d.side);
-            if (r) return r;
-        } else {
-            r = exec_fp64(p, op, omega, screen, off, out, nullptr, s, kMixedFp64Classes);
-            if (r) return r;
-        }
-        if (p->d.schedule == SHG_SCHED_PERSISTENT) {
-            m.tile_begin = p->d.mixed_fp64_tiles;
-            m.tile_end = p->d.n_tiles;
-            if (m.tile_end <= m.tile_begin) return SHG_OK;
-            const cudaStream_t sm = fork ? p->d.side2 : s;
-            SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), sm));
-            m.counter = p->d.counter;
-            SHG_CUDA(launch_2c_mixed(m, op, persistent_grid_2c_mixed(op, p->d.threads, p->d.ctas_per_sm), true, sm,
-                                     p->d.threads));
-            if (fork) return join_sides(p, s);
-        } else {
-            m.counter = nullptr;
-            for (int cls = 0; cls < kNClass; ++cls) {
-                if (mixed_runs_fp64(cls)) continue;
-                m.tile_begin = p->d.class_tile_begin[cls];
-                m.tile_end = p->d.class_tile_begin[cls + 1];
-                if (m.tile_end <= m.tile_begin) continue;
-                SHG_CUDA(launch_2c_mixed(m, op, 0, false, s, p->d.threads));
-            }
-        }
-        return SHG_OK;
+        ArgsFused f;
+        fused_ops(f, 1, &op, &omega, &out);
+        fused_plan(f, *p->d.basis, p->d, *t, off);
+        f.screen_thresh = op == SHG_OP_OVERLAP || op == SHG_OP_GAUSS ? screen : 0.0;
+        return exec_mixed(p, f, s);
     }
     return exec_fp64(p, op, omega, screen, off, out, nullptr, s);
 }
 
+} // extern "C"
+namespace shg {
+void fused_ops(ArgsFused &a, int n_ops, const int *ops, const double *omegas, double *const *outs)
+{
+    double w_erf = 0, w_erfc = 0, w_gauss = 0;
+    for (int i = 0; i < 6; ++i) a.out[i] = nullptr;
+    for (int i = 0; i < n_ops; ++i) {
+        a.out[ops[i]] = outs[i];
+        if (ops[i] == SHG_OP_ERF) w_erf = omegas[i];
+        if (ops[i] == SHG_OP_ERFC) w_erfc = omegas[i];
+        if (ops[i] == SHG_OP_GAUSS || ops[i] == SHG_OP_GAUSS_COULOMB) w_gauss = omegas[i];
+    }
+    a.r.erf = x_omega(w_erf);
+    a.r.erfc = x_omega(w_erfc);
+    a.r.gauss = x_omega(w_gauss);
+    const bool ov = a.out[SHG_OP_OVERLAP], co = a.out[SHG_OP_COULOMB], ec = a.out[SHG_OP_ERFC],
+               er = a.out[SHG_OP_ERF], ga = a.out[SHG_OP_GAUSS];
+    a.r.want = (ov ? kSumOv : 0) | (co || ec ? kSumCo : 0) | (er ? kSumEr : 0) |
+               (ec && !(er && w_erf == w_erfc) ? kSumX : 0) | (ga ? kSumGa : 0) |
+               (a.out[SHG_OP_GAUSS_COULOMB] ? kSumGc : 0);
+    a.screen_thresh = 0.0;
+    a.screen_omega = w_gauss;
+}
+
+void fused_plan(ArgsFused &a, const BasisDev &b, const PlanDev &d, const DeviceTables &t, const int64_t *off)
+{
+    a.shells = b.shells;
+    a.centers = b.centers;
+    a.pair_a = d.pair_a;
+    a.pair_b = d.pair_b;
+    a.perm = d.perm;
+    a.tiles = d.tiles;
+    a.out_off = reinterpret_cast<const long long *>(off);
+    a.r.prims = b.xprims;
+    a.r.t = t.x;
+    a.cg = t.cg;
+    a.screen = b.screen;
+    a.k = consts();
+}
+}  // namespace shg
+extern "C" {
+
 // FP64 execution of a plan; o_pre != null runs the angular part on
 // precomputed contracted radial terms (op = OP_PRE, family path).
 static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const int64_t *off, double *out,
-                     const double *o_pre, cudaStream_t s, int sel)
+                     const double *o_pre, cudaStream_t s)
 {
     const DeviceTables *t = device_tables();
     if (!t) return SHG_ECUDA;
     const int precision = SHG_PREC_FP64;
+    if (op <= SHG_OP_GAUSS_COULOMB) {
+        ArgsFused f;
+        fused_ops(f, 1, &op, &omega, &out);
+        fused_plan(f, *p->d.basis, p->d, *t, off);
+        f.screen_thresh = op == SHG_OP_OVERLAP || op == SHG_OP_GAUSS ? screen : 0.0;
+        return exec_fused_fp64(p, f, kAllClasses, p->d.variant, s);
+    }
     Args2c a;
     a.shells = p->d.basis->shells;
     a.prims = p->d.basis->prims;
@@ -1319,12 +1456,10 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     a.pair_a = p->d.pair_a;
     a.pair_b = p->d.pair_b;
     a.perm = p->d.perm;
-    a.tiles = p->d.tiles;
+    a.map = p->d.map;
     a.out_off = reinterpret_cast<const long long *>(off);
     a.out = out;
     a.omega = omega;
-    a.screen_thresh = screen;
-    a.screen = p->d.basis->screen;
     a.boys = t->boys;
     a.boys_e = t->boys_e;
     a.o_pre = o_pre;
@@ -1332,18 +1467,16 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     a.k = consts();
     if (p->d.schedule == SHG_SCHED_PERSISTENT) {
         a.tile_begin = 0;
-        a.tile_end = sel == kAllClasses ? p->d.n_tiles : p->d.mixed_fp64_tiles;
-        if (a.tile_end <= 0) return SHG_OK;
+        a.tile_end = p->d.map.tile[kNClass];
         SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), s));
         a.counter = p->d.counter;
         SHG_CUDA(launch_2c(a, op, precision, persistent_grid_2c(op, precision, p->d.threads, p->d.ctas_per_sm), true, s,
                            p->d.threads));
     } else {
         a.counter = nullptr;
-        for (int cls = 0; cls < kNClass; ++cls) {
-            if (sel == kMixedFp64Classes && !mixed_runs_fp64(cls)) continue;
-            a.tile_begin = p->d.class_tile_begin[cls];
-            a.tile_end = p->d.class_tile_begin[cls + 1];
+        for (int c = 0; c < kNClass; ++c) {
+            a.tile_begin = p->d.map.tile[c];
+            a.tile_end = p->d.map.tile[c + 1];
             if (a.tile_end <= a.tile_begin) continue;
             SHG_CUDA(launch_2c(a, op, precision, 0, false, s, p->d.threads));
         }
@@ -1351,65 +1484,91 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     return SHG_OK;
 }
 
-// FP64 single-operator pass over the tiles [tile_begin, tile_end) of a plan,
-// one warp per tile (no work counter: it may run beside a persistent launch
-// of the same plan)
-static int exec_fp64_static_range(shg_plan_t *p, int op, double omega, double screen, const int64_t *off,
-                                  double *out, int tile_begin, int tile_end, cudaStream_t s)
+// FP64 pass over the tiles of a plan (all of them, or those that the mixed-precision passes run in FP64)
+static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, int sel, int variant, cudaStream_t s)
 {
-    const DeviceTables *t = device_tables();
-    if (!t) return SHG_ECUDA;
-    Args2c a;
-    a.shells = p->d.basis->shells;
-    a.prims = p->d.basis->prims;
-    a.centers = p->d.basis->centers;
-    a.pair_a = p->d.pair_a;
-    a.pair_b = p->d.pair_b;
-    a.perm = p->d.perm;
-    a.tiles = p->d.tiles;
-    a.out_off = reinterpret_cast<const long long *>(off);
-    a.out = out;
-    a.omega = omega;
-    a.screen_thresh = screen;
-    a.screen = p->d.basis->screen;
-    a.boys = t->boys;
-    a.boys_e = t->boys_e;
-    a.o_pre = nullptr;
-    a.cg = t->cg;
-    a.k = consts();
-    a.tile_begin = tile_begin;
-    a.tile_end = tile_end;
+    if (p->d.schedule == SHG_SCHED_PERSISTENT) {
+        a.tile_begin = 0;
+        a.tile_end = sel == kAllClasses ? p->d.n_tiles : p->d.mixed_fp64_tiles;
+        if (a.tile_end <= 0) return SHG_OK;
+        SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), s));
+        a.counter = p->d.counter;
+        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, p->d.ctas_per_sm, variant));
+        return SHG_OK;
+    }
     a.counter = nullptr;
-    SHG_CUDA(launch_2c(a, op, SHG_PREC_FP64, 0, false, s, 32));
+    for (int cls = 0; cls < kNClass; ++cls) {
+        if (sel == kMixedFp64Classes && !mixed_runs_fp64(cls)) continue;
+        a.tile_begin = p->d.class_tile_begin[cls];
+        a.tile_end = p->d.class_tile_begin[cls + 1];
+        if (a.tile_end <= a.tile_begin) continue;
+        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, 0, variant));
+    }
     return SHG_OK;
 }
 
-// Arguments of a fused pass: the operators are checked (each of overlap,
-// 1/r, erfc, erf and the Gaussian at most once, in the given precision),
-// outputs placed by operator id.
-static int fused_args(shg_plan_t *p, int n_ops, const int *ops, const double *omegas, int precision,
-                      const int64_t *off, double *const *outs, ArgsFused &a)
+// Mixed-precision pass: the classes with both l >= kMixedFp64MinL in FP64 (one warp per tile on a side stream, beside
+// the double-float launch, when a persistent plan holds both kinds), the others with the double-float angular part
+static int exec_mixed(shg_plan_t *p, const ArgsFused &f, cudaStream_t s)
+{
+    const bool persistent = p->d.schedule == SHG_SCHED_PERSISTENT;
+    const bool fork = persistent && p->d.mixed_fp64_tiles > 0 && p->d.n_tiles > p->d.mixed_fp64_tiles;
+    ArgsMixFused m;
+    m.f = f;
+    fill_kappa_mix(m.kappa);
+    int r;
+    if (fork) {
+        r = fork_sides(p, s);
+        if (r) return r;
+        ArgsFused a = f;
+        a.tile_begin = 0;
+        a.tile_end = p->d.mixed_fp64_tiles;
+        a.counter = nullptr;
+        SHG_CUDA(launch_2c_fused(a, p->d.side, 32, 0, 1));
+    } else {
+        r = exec_fused_fp64(p, m.f, kMixedFp64Classes, p->d.variant, s);
+        if (r) return r;
+    }
+    if (persistent) {
+        m.f.tile_begin = p->d.mixed_fp64_tiles;
+        m.f.tile_end = p->d.n_tiles;
+        if (m.f.tile_end <= m.f.tile_begin) return SHG_OK;
+        const cudaStream_t sm = fork ? p->d.side2 : s;
+        SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), sm));
+        m.f.counter = p->d.counter;
+        SHG_CUDA(launch_2c_mixed(m, sm, p->d.threads, p->d.ctas_per_sm, p->d.variant));
+        return fork ? join_sides(p, s) : SHG_OK;
+    }
+    m.f.counter = nullptr;
+    for (int cls = 0; cls < kNClass; ++cls) {
+        if (mixed_runs_fp64(cls)) continue;
+        m.f.tile_begin = p->d.class_tile_begin[cls];
+        m.f.tile_end = p->d.class_tile_begin[cls + 1];
+        if (m.f.tile_end <= m.f.tile_begin) continue;
+        SHG_CUDA(launch_2c_mixed(m, s, p->d.threads, 0, p->d.variant));
+    }
+    return SHG_OK;
+}
+
+// Checks of a fused pass: each of overlap, 1/r, erfc, erf and the Gaussian at most once, in the given precision
+static int check_fused(shg_plan_t *p, int n_ops, const int *ops, const double *omegas, int precision,
+                       const int64_t *off, double *const *outs)
 {
     if (!p) return fail(SHG_EINVAL, "plan is NULL");
     if (n_ops < 1 || n_ops > 5) return fail(SHG_EINVAL, "n_ops must be 1..5 (got %d)", n_ops);
     if (!ops || !omegas || !outs) return fail(SHG_EINVAL, "NULL operator, omega or output array");
-    for (int i = 0; i < 5; ++i) a.out[i] = nullptr;
-    a.w_erf = a.w_erfc = a.w_gauss = 0.0;
+    unsigned seen = 0;
     for (int i = 0; i < n_ops; ++i) {
         const int op = ops[i];
         if (op < SHG_OP_OVERLAP || op > SHG_OP_GAUSS)
             return fail(SHG_EINVAL, "the fused pass takes overlap, 1/r, erfc, erf and the Gaussian only (got %d)", op);
         int r = check_op(op, omegas[i], precision);
         if (r) return r;
-        if (a.out[op]) return fail(SHG_EINVAL, "operator %d listed twice", op);
+        if (seen >> op & 1) return fail(SHG_EINVAL, "operator %d listed twice", op);
         if (!outs[i]) return fail(SHG_EINVAL, "NULL output for operator %d", op);
-        a.out[op] = outs[i];
-        if (op == SHG_OP_ERF) a.w_erf = omegas[i];
-        if (op == SHG_OP_ERFC) a.w_erfc = omegas[i];
-        if (op == SHG_OP_GAUSS) a.w_gauss = omegas[i];
+        seen |= 1u << op;
     }
     if (!off) return fail(SHG_EINVAL, "NULL output offsets");
-    a.share_att = (a.out[SHG_OP_ERF] && a.out[SHG_OP_ERFC] && a.w_erf == a.w_erfc) ? 1 : 0;
     return SHG_OK;
 }
 
@@ -1418,8 +1577,7 @@ int shg_plan_2c_exec_fused(shg_plan_t *p, int n_ops, const int *ops, const doubl
 {
     Phase phase_("shg:plan_2c_exec_fused");
     g_err.clear();
-    ArgsFused a;
-    int r = fused_args(p, n_ops, ops, omegas, precision, off, outs, a);
+    int r = check_fused(p, n_ops, ops, omegas, precision, off, outs);
     if (r) return r;
     if (p->d.n_pairs == 0 || p->d.n_tiles == 0) return SHG_OK;
     r = current_device_matches(p->d.basis->device);
@@ -1427,96 +1585,11 @@ int shg_plan_2c_exec_fused(shg_plan_t *p, int n_ops, const int *ops, const doubl
     const DeviceTables *t = device_tables();
     if (!t) return SHG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    a.shells = p->d.basis->shells;
-    a.prims = p->d.basis->prims;
-    a.centers = p->d.basis->centers;
-    a.pair_a = p->d.pair_a;
-    a.pair_b = p->d.pair_b;
-    a.perm = p->d.perm;
-    a.tiles = p->d.tiles;
-    a.out_off = reinterpret_cast<const long long *>(off);
-    a.boys = t->boys;
-    a.boys_e = t->boys_e;
-    a.cprims = p->d.basis->cprims;
-    a.cg = t->cg;
-    a.k = consts();
-    const bool mixed = precision == SHG_PREC_MIXED;
-    const bool persistent = p->d.schedule == SHG_SCHED_PERSISTENT;
-    // mixed precision on a persistent plan with both kinds of classes: the FP64
-    // tiles (one warp each) and the double-float launch side by side on the plan's
-    // side streams
-    const bool fork = mixed && persistent && p->d.mixed_fp64_tiles > 0 && p->d.n_tiles > p->d.mixed_fp64_tiles;
-    if (fork) {
-        r = fork_sides(p, s);
-        if (r) return r;
-        a.tile_begin = 0;
-        a.tile_end = p->d.mixed_fp64_tiles;
-        a.counter = nullptr;
-        SHG_CUDA(launch_2c_fused(a, 0, false, p->d.side, 32));
-    } else if (persistent) {
-        // FP64 pass: every tile, or under mixed precision the classes with both
-        // l >= kMixedFp64MinL (a prefix of the persistent tile order)
-        a.tile_begin = 0;
-        a.tile_end = mixed ? p->d.mixed_fp64_tiles : p->d.n_tiles;
-        if (a.tile_end > 0) {
-            SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), s));
-            a.counter = p->d.counter;
-            // the variant applies to the FP64 pass of FP64 executions only
-            const int v = mixed ? 0 : p->d.variant;
-            SHG_CUDA(launch_2c_fused(a, persistent_grid_2c_fused(p->d.threads, p->d.ctas_per_sm, v), true, s,
-                                     p->d.threads, v));
-        }
-    } else {
-        a.counter = nullptr;
-        for (int cls = 0; cls < kNClass; ++cls) {
-            if (mixed && !mixed_runs_fp64(cls)) continue;
-            a.tile_begin = p->d.class_tile_begin[cls];
-            a.tile_end = p->d.class_tile_begin[cls + 1];
-            if (a.tile_end <= a.tile_begin) continue;
-            SHG_CUDA(launch_2c_fused(a, 0, false, s, p->d.threads));
-        }
-    }
-    if (!mixed) return SHG_OK;
-    ArgsMixFused m;
-    m.shells = p->d.basis->shells;
-    m.prims = p->d.basis->mprims;
-    m.centers = p->d.basis->mcenters;
-    m.pair_a = p->d.pair_a;
-    m.pair_b = p->d.pair_b;
-    m.perm = p->d.perm;
-    m.tiles = p->d.tiles;
-    m.out_off = reinterpret_cast<const long long *>(off);
-    for (int i = 0; i < 5; ++i) m.out[i] = a.out[i];
-    m.w_erf = split2(a.w_erf);
-    m.w_erf2 = split2((long double)a.w_erf * a.w_erf);
-    m.w_erfc = split2(a.w_erfc);
-    m.w_erfc2 = split2((long double)a.w_erfc * a.w_erfc);
-    m.w_gauss = split2(a.w_gauss);
-    m.share_att = a.share_att;
-    m.boys = t->boys_mix;
-    m.boys_e = t->boys_e_mix;
-    m.km = consts_mix();
-    if (persistent) {
-        m.tile_begin = p->d.mixed_fp64_tiles;
-        m.tile_end = p->d.n_tiles;
-        if (m.tile_end <= m.tile_begin) return SHG_OK;
-        const cudaStream_t sm = fork ? p->d.side2 : s;
-        SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), sm));
-        m.counter = p->d.counter;
-        SHG_CUDA(launch_2c_mixed_fused(m, persistent_grid_2c_mixed_fused(p->d.threads, p->d.ctas_per_sm, p->d.variant),
-                                       true, sm, p->d.threads, p->d.variant));
-        if (fork) return join_sides(p, s);
-    } else {
-        m.counter = nullptr;
-        for (int cls = 0; cls < kNClass; ++cls) {
-            if (mixed_runs_fp64(cls)) continue;
-            m.tile_begin = p->d.class_tile_begin[cls];
-            m.tile_end = p->d.class_tile_begin[cls + 1];
-            if (m.tile_end <= m.tile_begin) continue;
-            SHG_CUDA(launch_2c_mixed_fused(m, 0, false, s, p->d.threads, p->d.variant));
-        }
-    }
-    return SHG_OK;
+    ArgsFused a;
+    fused_ops(a, n_ops, ops, omegas, outs);
+    fused_plan(a, *p->d.basis, p->d, *t, off);
+    if (precision == SHG_PREC_MIXED) return exec_mixed(p, a, s);
+    return exec_fused_fp64(p, a, kAllClasses, p->d.variant, s);
 }
 
 int shg_graph_2c_create_fused(shg_plan_t *p, int n_ops, const int *ops, const double *omegas, int precision,
@@ -1525,8 +1598,7 @@ int shg_graph_2c_create_fused(shg_plan_t *p, int n_ops, const int *ops, const do
     g_err.clear();
     if (!out) return fail(SHG_EINVAL, "out is NULL");
     *out = nullptr;
-    ArgsFused chk;
-    int r = fused_args(p, n_ops, ops, omegas, precision, off, outs, chk);
+    int r = check_fused(p, n_ops, ops, omegas, precision, off, outs);
     if (r) return r;
     return capture_graph(
         [&](cudaStream_t s) { return shg_plan_2c_exec_fused(p, n_ops, ops, omegas, precision, off, outs, s); }, out);
@@ -1567,7 +1639,7 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     if (!t) return SHG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
-    const int64_t max_tiles = n / kTile + std::min<int64_t>(n, kNBins3) + 1;
+    const int64_t max_tiles = plan_max_tiles(n, kNClass3, false);
     const size_t bytes_perm = sizeof(int32_t) * (size_t)n;
     const size_t bytes_tiles = sizeof(Tile) * (size_t)max_tiles;
     const size_t bytes_ws = sizeof(int) * plan_ws_ints(n, kNBins3, kNClass3);
@@ -1673,9 +1745,8 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     a.pair_a = pa;
     a.pair_b = pb;
     a.perm = p->d.perm;
-    a.tiles = p->d.tiles;
+    a.map = p->d.map;
     a.tile_begin = 0;
-    a.tile_end = p->d.n_tiles;
     a.counter = p->d.counter;
     a.omega = omega;
     a.boys = t->boys;
@@ -1691,8 +1762,9 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     // two launches run side by side on the plan's side streams (as in
     // shg_plan_2c_exec_fused): the FP64 tiles one warp each, statically.
     const bool mixed = precision == SHG_PREC_MIXED;
-    const bool fork = mixed && p->d.mixed_fp64_tiles > 0 && p->d.n_tiles > p->d.mixed_fp64_tiles;
-    a.tile_end = mixed ? p->d.mixed_fp64_tiles : p->d.n_tiles;
+    const int hi_tiles = p->d.mixed_fp64_tiles32, all_tiles = p->d.map.tile[kNClass];
+    const bool fork = mixed && hi_tiles > 0 && all_tiles > hi_tiles;
+    a.tile_end = mixed ? hi_tiles : all_tiles;
     cudaError_t e = cudaSuccess;
     if (fork) {
         r = fork_sides(p, s);
@@ -1706,7 +1778,7 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
         e = cudaMemsetAsync(p->d.counter, 0, sizeof(int), s);
         if (e == cudaSuccess) e = launch_2c_grad(a, op, SHG_PREC_FP64, persistent_grid_2c_grad(op, SHG_PREC_FP64), s);
     }
-    if (e == cudaSuccess && mixed && p->d.n_tiles > p->d.mixed_fp64_tiles) {
+    if (e == cudaSuccess && mixed && all_tiles > hi_tiles) {
         ArgsGradMix gm;
         gm.g = a;
         ArgsMix &m = gm.m;
@@ -1716,9 +1788,8 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
         m.pair_a = pa;
         m.pair_b = pb;
         m.perm = p->d.perm;
-        m.tiles = p->d.tiles;
-        m.tile_begin = p->d.mixed_fp64_tiles;
-        m.tile_end = p->d.n_tiles;
+        gm.g.tile_begin = hi_tiles;
+        gm.g.tile_end = all_tiles;
         m.counter = p->d.counter;
         m.out_off = nullptr;
         m.out = nullptr;

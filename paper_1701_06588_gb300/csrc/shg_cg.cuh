@@ -67,52 +67,57 @@ __device__ __forceinline__ void laplace_orders(const double *__restrict__ fc, do
     }
 }
 
-// the block of one operator; PF[M * J + p] = p_{L,M} F_p, g: coefficients of the class
-__device__ __forceinline__ void store_block(const double *__restrict__ g, int la, int lb, int J, const double *PF,
-                                            const double *C, const double *S, double *__restrict__ out)
+// the elements (+-a, +-b) of the block of one operator; PF[M * J + p] = p_{L,M} F_p, g: coefficients of (a, b), o: the
+// block's element (0, 0)
+__device__ __forceinline__ void element(const double *__restrict__ g, int a, int b, int kmax, int J, int nb,
+                                        const double *PF, const double *C, const double *S, double *__restrict__ o)
 {
-    const int nb = 2 * lb + 1, kmax = la + lb;
-    for (int a = 0; a <= la; ++a)
-        for (int b = 0; b <= lb; ++b, g += 2 * J) {
-            const int m1 = a > b ? a - b : b - a, m2 = a + b;
-            // L >= M: p <= (kmax - M) / 2
-            const int n1 = min(J, (kmax - m1) / 2 + 1);
-            double X1 = __ldg(g) * PF[m1 * J];
-            for (int p = 1; p < n1; ++p) X1 = fma(__ldg(g + p), PF[m1 * J + p], X1);
-            double *o = out + la * nb + lb;
-            if (a && b) {
-                const int n2 = min(J, (kmax - m2) / 2 + 1);
-                double X2 = __ldg(g + J) * PF[m2 * J];
-                for (int p = 1; p < n2; ++p) X2 = fma(__ldg(g + J + p), PF[m2 * J + p], X2);
-                const double c1 = C[m1] * X1, s2 = S[m2] * X2;
-                const double s1 = a > b ? S[m1] : -S[m1];
-                o[a * nb + b] = fma(C[m2], X2, c1);
-                o[-a * nb - b] = fma(-C[m2], X2, c1);
-                o[-a * nb + b] = fma(s1, X1, s2);
-                o[a * nb - b] = fma(-s1, X1, s2);
-            } else {
-                o[a * nb + b] = C[m1] * X1;
-                if (a) o[-a * nb] = S[m1] * X1;
-                if (b) o[-b] = S[m1] * X1;
-            }
-        }
+    const int m1 = a > b ? a - b : b - a, m2 = a + b;
+    // L >= M: p <= (kmax - M) / 2
+    const int n1 = min(J, (kmax - m1) / 2 + 1);
+    double X1 = __ldg(g) * PF[m1 * J];
+    for (int p = 1; p < n1; ++p) X1 = fma(__ldg(g + p), PF[m1 * J + p], X1);
+    if (a && b) {
+        const int n2 = min(J, (kmax - m2) / 2 + 1);
+        double X2 = __ldg(g + J) * PF[m2 * J];
+        for (int p = 1; p < n2; ++p) X2 = fma(__ldg(g + J + p), PF[m2 * J + p], X2);
+        const double c1 = C[m1] * X1, s2 = S[m2] * X2;
+        const double s1 = a > b ? S[m1] : -S[m1];
+        o[a * nb + b] = fma(C[m2], X2, c1);
+        o[-a * nb - b] = fma(-C[m2], X2, c1);
+        o[-a * nb + b] = fma(s1, X1, s2);
+        o[a * nb - b] = fma(-s1, X1, s2);
+    } else {
+        o[a * nb + b] = C[m1] * X1;
+        if (a) o[-a * nb] = S[m1] * X1;
+        if (b) o[-b] = S[m1] * X1;
+    }
 }
 
-// Block of one operator from its radial orders, one thread per pair.
+// Block of one operator from its radial orders: lane gl of the `group` lanes of the pair stores every group-th set of
+// elements.  top: a contribution to the order la + lb that
+// belongs to a harmonic part of G (its F_p, p >= 1, vanish).
 template <int J>
 __device__ __forceinline__ void block_from_orders(const CGTab &t, int la, int lb, double r2, const double (&O)[J],
-                                                  const double *P, const double *C, const double *S, double *PF,
-                                                  double *__restrict__ out)
+                                                  double top, const double *P, const double *C, const double *S,
+                                                  double *PF, int gl, int group, double *__restrict__ out)
 {
     double F[J];
-    laplace_orders<J>(t.fc + 28 * (la * (kLmax2c + 1) + lb), r2, O, F);
+    const double *fc = t.fc + 28 * (la * (kLmax2c + 1) + lb);
+    laplace_orders<J>(fc, r2, O, F);
+    F[0] = fma(__ldg(fc), top, F[0]);
     const int kmax = la + lb;
     for (int M = 0; M <= kmax; ++M) {
 #pragma unroll
         for (int p = 0; p < J; ++p)
             if (M + 2 * p <= kmax) PF[M * J + p] = P[M * J + p] * F[p];
     }
-    store_block(t.g + __ldg(t.gbase + la * (kLmax2c + 1) + lb), la, lb, J, PF, C, S, out);
+    const double *g = t.g + __ldg(t.gbase + la * (kLmax2c + 1) + lb);
+    const int nb = 2 * lb + 1;
+    for (int i = gl; i < (la + 1) * (lb + 1); i += group) {
+        const int a = i / (lb + 1), b = i - a * (lb + 1);
+        element(g + i * 2 * J, a, b, kmax, J, nb, PF, C, S, out + la * nb + lb);
+    }
 }
 
 }  // namespace cg

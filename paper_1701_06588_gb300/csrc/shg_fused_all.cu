@@ -1,0 +1,15 @@
+// FP64 two-center passes of any set of operators.
+#include "shg_pair2c.cuh"
+
+namespace shg {
+
+cudaError_t launch_2c_all(const ArgsFused &a, cudaStream_t s, int threads, int ctas_per_sm, int variant)
+{
+    switch (variant) {
+    case 0: return launch_pass<kSumAll, 3>(a, s, threads, ctas_per_sm);
+    case 1: return launch_pass<kSumAll, 6>(a, s, threads, ctas_per_sm);
+    default: return launch_pass<kSumAll, 4>(a, s, threads, ctas_per_sm);
+    }
+}
+
+}  // namespace shg

@@ -17,6 +17,7 @@
 // The radial terms are recomputed here up to order la+lb+1; nothing is kept
 // from a forward evaluation.
 #include "shg_device.cuh"
+#include "shg_tilemap.cuh"
 #include "shg_grad_angular.cuh"
 
 namespace shg {
@@ -98,10 +99,11 @@ __global__ void __launch_bounds__(128) k_2c_grad_fp64_persistent(const Args2c g)
             t = g.tile_begin + blockIdx.x * nw + (threadIdx.x >> 5);
         }
         if (t >= g.tile_end) break;
-        const Tile tl = g.tiles[t];
-        if (lane < tl.count) {
-            const int la = tl.cls / (kLmax2c + 1), lb = tl.cls % (kLmax2c + 1);
-            grad_dispatch<OP>(g, g.perm[tl.start + lane], (la < lb ? la : lb) + 1);
+        int cls;
+        const int q = map_pair(g.map, t, lane, cls);
+        if (q >= 0) {
+            const int la = cls / (kLmax2c + 1), lb = cls % (kLmax2c + 1);
+            grad_dispatch<OP>(g, g.perm[q], (la < lb ? la : lb) + 1);
         }
         __syncwarp();
     }

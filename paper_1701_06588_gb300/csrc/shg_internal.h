@@ -37,6 +37,47 @@ constexpr int kBoysStride = 6;
 constexpr double kBoysTmax = 120.0;
 constexpr int kBoysN = 16;          // orders n = 0..15 from the tables
 
+// Boys function for the extended-float radial sums: from T = kFarT on the asymptotic form (relative error below 5e-18
+// for n <= 13: T^{n-1/2} e^{-T} / Gamma(n+1/2)); below, per order n = 0..kBoysOrders-1 and cell [i, i+1) / 512 of T, the Taylor coefficients c_t = F_{n+t}(T_{i+1}) / t! about the upper end of the cell, scaled by
+// 2^s so that c0 < 2^63 (1 - 2^-8): c0, c1 in units 2^-s, c2 likewise with s - 62 in its low 8 bits, c3 in units
+// 2^{30-s}, c4 (24 bits) in units 2^{35-s}, c5 (8 bits) in units 2^{49-s}.  y = T_{i+1} - T <= 2^-9, so the dropped
+// y^6/720 is below 2^-63.  One 32-byte load per evaluation; 16.5 MB, resident in L2.
+constexpr int kFarT = 72;
+constexpr int kBoysCells = kFarT * 512;
+constexpr int kBoysOrders = 14;
+struct alignas(32) BoysEnt {
+    uint64_t c0, c1, c2;
+    uint32_t c3, c45;
+};
+constexpr int kExpTab = 356;            // exp(j/512) 2^62, j/512 < 0.6954
+struct XTab {
+    const BoysEnt *boys;
+    const uint64_t *exp;
+};
+struct XOmega {
+    uint64_t w_m, w2_m;                 // omega and omega^2 as extended floats
+    int w_e, w2_e;
+};
+// Sums a radial pass can form (bits of RadialIn::want and of the kernels' masks): overlap, 1/r, the attenuated
+// part of erf, that of erfc (not when erf with the same omega is formed), Gaussian, exp(-wr^2)/r (alone)
+enum { kSumOv = 1, kSumCo = 2, kSumEr = 4, kSumX = 8, kSumGa = 16, kSumAll = 31, kSumGc = 32 };
+
+// Per-primitive record of the extended-float radial sums (32 bytes): alpha and cw (see CoulPrim) as m 2^e, m in
+// [2^62, 2^63), the sign of cw in bit 63 of wm; fw as in CoulPrim.
+struct alignas(32) XPrim {
+    uint64_t am, wm;
+    int ae, we;
+    double fw;
+};
+
+// What a radial pass takes beside the pair (by value in the kernel parameters)
+struct RadialIn {
+    const XPrim *prims;
+    XTab t;
+    XOmega erf, erfc, gauss;      // gauss: also of exp(-wr^2)/r
+    unsigned want;                // sums this launch forms
+};
+
 // Per-shell screening data (host-computed): smallest exponent, sum |N c| over
 // the primitives, and (l / (alpha_min e))^{l/2} (1 for l = 0).
 struct alignas(32) ScreenRec {
@@ -127,6 +168,12 @@ struct CGTab {
     const double *g;
     const int *gbase;
     const double *fc;
+    const float2 *gm;             // g as double-float
+};
+
+// kappa of Consts as double-float (mixed-precision angular part)
+struct KappaMix {
+    float2 v[16][16];
 };
 
 // Device-resident tables owned by the library, one set per device.
@@ -141,6 +188,7 @@ struct DeviceTables {
     const float4 *boys_mix;    // [kBoysGrid][kBoysN][3] (layout above)
     const float2 *boys_e_mix;  // [kBoysGrid] exp(-T_i) as hi/lo
     CGTab cg;
+    XTab x;
 };
 
 // Extra constants of the three-index kernels (by value).
@@ -166,6 +214,13 @@ int fail(int code, const char *fmt, ...);          // sets shg_last_error(), ret
 void clear_error();                                // empties shg_last_error() (start of a call)
 const Consts &consts();                            // constant tables (host copy)
 int check_op(int op, double omega, int precision);  // operator / omega / precision check
+struct ArgsFused;
+struct BasisDev;
+struct PlanDev;
+// operators overlap .. Gaussian of a pass (distinct, checked): sums, omegas and outputs
+void fused_ops(ArgsFused &a, int n_ops, const int *ops, const double *omegas, double *const *outs);
+// basis, plan and table pointers of a pass
+void fused_plan(ArgsFused &a, const BasisDev &b, const PlanDev &d, const DeviceTables &t, const int64_t *off);
 
 // Host generation of the Boys table (long double arithmetic).
 void make_boys_table(int per_unit, int ngrid, int nterms, double *tab, double *etab);
@@ -179,6 +234,7 @@ struct BasisDev {
     Vec4 *centers = nullptr;      // device
     MixPrim *mprims = nullptr;    // device, double-float copies for the mixed path
     CoulPrim *cprims = nullptr;   // device, Coulomb-type weights (fused passes)
+    XPrim *xprims = nullptr;      // device, extended-float primitives (radial sums)
     ScreenRec *screen = nullptr;  // device, per-shell screening data
     MixCenter *mcenters = nullptr;
     // shg_basis_set_centers staging (allocated on its first call): raw
@@ -196,17 +252,34 @@ struct BasisDev {
     int n_fams = 0;
 };
 
-// A warp's unit of work: up to kTile consecutive entries of the sorted list,
-// all of one class.  cls = la*7 + lb (two-center) or (la*7 + la~)*7 + lb.
+// A warp's unit of work: up to kTile / group consecutive entries of the sorted list, all of one class (cls = la*7 + lb, or
+// (la*7 + la~)*7 + lb), `group` lanes per entry, which share its primitive pairs.  Two-center pairs get the group by
+// their number of primitive pairs, so that a lane sums 32 of them at most (50 beyond 256): with one lane per pair the
+// longest tiles (400 one after the other) ran 1.5 ms beyond the end of all others on 200,000 pairs of long contractions
+// (2.0 ms in all, 17% of the SMs' time used).  The group follows from the pair alone, so the bits of a block do not
+// depend on the list it is evaluated in.
 struct Tile {
-    int start, count, cls, pad;
+    int start;
+    uint16_t cls;
+    uint8_t count, group;
 };
+constexpr int kNGroups = 4;
+constexpr int kGroupOf[kNGroups] = {8, 4, 2, 1};
+constexpr int kGroupMinK[kNGroups] = {129, 65, 33, 1};     // fewest primitive pairs of each group
 
 constexpr int kKbins2c = kKmax * kKmax;      // two-center bins per class: Ka*Kb - 1
 constexpr int kNBins2c = kNClass * kKbins2c;
 constexpr int kNClass3 = 7 * 7 * 7;          // (la, la~, lb) classes
 constexpr int kKbins3c = 512;                // three-index bins per class: min(Ka*Ka~*Kb, 512) - 1
 
+
+// Class chunks of a plan in rank order: first pair of each, first 32-pair tile of each and its class.  The kernels without
+// a sum over primitive pairs to share take 32 consecutive pairs of a class per warp whatever the tile list says.
+struct TileMap {
+    int pair[kNClass + 1] = {};
+    int tile[kNClass + 1] = {};
+    uint8_t cls[kNClass] = {};
+};
 
 struct PlanDev {
     const BasisDev *basis = nullptr;
@@ -220,7 +293,9 @@ struct PlanDev {
     Tile *tiles = nullptr;         // device [n_tiles]
     int *counter = nullptr;        // device, persistent work counter
     int n_tiles = 0;
+    TileMap map;
     int class_tile_begin[kNClass + 1] = {};   // host, per-class tile ranges (class-major)
+    int mixed_fp64_tiles32 = 0;    // the same in 32-pair tiles of the map
     int mixed_fp64_tiles = 0;      // persistent order: leading tiles of the classes that the
                                    // mixed-precision passes run in FP64 (both l >= kMixedFp64MinL)
     int threads = 128;             // launch shape (autotuned): threads per CTA (32, 64 or 128)
@@ -243,7 +318,7 @@ struct Args2c {
     const Vec4 *centers;
     const int32_t *pair_a, *pair_b;
     const int32_t *perm;
-    const Tile *tiles;
+    TileMap map;                  // 32-pair tiles: tile_begin and tile_end count these
     int tile_begin, tile_end;
     int *counter;                 // persistent schedule (null: static)
     const long long *out_off;
@@ -264,12 +339,10 @@ struct Args2c {
     Consts k;
 };
 
-// Fused multi-operator FP64 pass (overlap, 1/r, erfc, erf, Gaussian): one
-// output per requested operator (null = not requested), all with the block
-// offsets out_off.
+// Pass over overlap, 1/r, erfc, erf and the Gaussian operator, one or several of them, or exp(-wr^2)/r: one output per
+// requested operator (null = not requested), all with the block offsets out_off.
 struct ArgsFused {
     const ShellRec *shells;
-    const PrimRec *prims;
     const Vec4 *centers;
     const int32_t *pair_a, *pair_b;
     const int32_t *perm;
@@ -277,12 +350,11 @@ struct ArgsFused {
     int tile_begin, tile_end;
     int *counter;                 // persistent schedule (null: static)
     const long long *out_off;
-    double *out[5];               // indexed by OP_OVERLAP .. OP_GAUSS
-    double w_erf, w_erfc, w_gauss;
-    int share_att;                // erf and erfc requested with the same omega
-    const double *boys, *boys_e;
-    const CoulPrim *cprims;       // Coulomb-type weights per primitive
+    double *out[6];               // indexed by OP_OVERLAP .. OP_GCOUL
+    RadialIn r;
     CGTab cg;
+    double screen_thresh, screen_omega;   // > 0 (one operator, overlap or Gaussian): pairs bounded below it write zeros
+    const ScreenRec *screen;
     Consts k;
 };
 
@@ -317,8 +389,6 @@ struct ArgsMix {
     const MixCenter *centers;
     const int32_t *pair_a, *pair_b;
     const int32_t *perm;
-    const Tile *tiles;
-    int tile_begin, tile_end;
     int *counter;
     const long long *out_off;
     double *out;
@@ -334,23 +404,10 @@ struct ArgsMix {
 // vector-Jacobian product (g: centers, constants, upstream weights, outputs).
 struct ArgsGradMix;
 
-// Fused multi-operator pass in double-float (outputs as ArgsFused).
+// Mixed-precision pass: radial sums as the FP64 pass, angular part in double-float.
 struct ArgsMixFused {
-    const ShellRec *shells;
-    const MixPrim *prims;
-    const MixCenter *centers;
-    const int32_t *pair_a, *pair_b;
-    const int32_t *perm;
-    const Tile *tiles;
-    int tile_begin, tile_end;
-    int *counter;
-    const long long *out_off;
-    double *out[5];                     // indexed by OP_OVERLAP .. OP_GAUSS
-    float2 w_erf, w_erf2, w_erfc, w_erfc2, w_gauss;   // omega (and omega^2) as double-float
-    int share_att;
-    const float4 *boys;
-    const float2 *boys_e;
-    ConstsMix km;
+    ArgsFused f;
+    KappaMix kappa;
 };
 
 struct ArgsGradMix {
@@ -386,36 +443,40 @@ struct Args3c {
 
 // Kernel launchers (shg_kernels.cu, shg_3c.cu).
 // Planning workspace (ints): err, ticket, 2 spare, hist, bin_start, cursor
-// (n_bins each), tile_start (n_bins + 1), summary (n_chunks + 2), key (n).
+// (n_bins each), tile_start (n_bins + 1), summary (2 n_chunks + 2), key (n).
 // After the build, summary[c] is the first tile of class chunk c
-// (c = 0..n_chunks-1), summary[n_chunks] the number of tiles and
-// summary[n_chunks + 1] the error flag of the classification.
+// (c = 0..n_chunks-1), summary[n_chunks] the number of tiles,
+// summary[n_chunks + 1] the error flag of the classification and
+// summary[n_chunks + 2 + c] the first pair of chunk c.
 constexpr size_t plan_ws_ints(int64_t n, int n_bins, int n_chunks)
 {
-    return 4 + 4 * (size_t)n_bins + 1 + (size_t)n_chunks + 2 + (size_t)n;
+    return 4 + 4 * (size_t)n_bins + 1 + 2 * (size_t)n_chunks + 2 + (size_t)n;
 }
+// largest number of tiles of n entries: every chunk ends in at most one partial tile per group size
+constexpr int64_t plan_max_tiles(int64_t n, int n_chunks, bool grouped)
+{
+    return n * (grouped ? kGroupOf[0] : 1) / kTile + kNGroups * n_chunks + 1;
+}
+// chunk -> first tile, tile count and error flag (n_chunks + 2 ints of the summary) and the tile map of a two-center plan
+int plan_read(PlanDev &d, const int *summary, int schedule);
 inline int *plan_summary(int *ws, int n_bins) { return ws + 4 + 4 * (size_t)n_bins + 1; }
 cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d_bin_rank, cudaStream_t s);
 cudaError_t launch_3c(const Args3c &args, int precision, int grid, cudaStream_t s);
 // grid is ignored when args.counter is null (static launch, one warp per tile)
 cudaError_t launch_2c_grad(const Args2c &args, int op, int precision, int grid, cudaStream_t s, int threads = 128);
 cudaError_t launch_2c_grad_mixed(const ArgsGradMix &args, int op, cudaStream_t s);
-cudaError_t launch_2c_mixed(const ArgsMix &args, int op, int grid, bool persistent, cudaStream_t s,
-                            int threads = 128);
-int persistent_grid_2c_mixed(int op, int threads = 128, int ctas_per_sm = 0);
-cudaError_t launch_2c_mixed_fused(const ArgsMixFused &args, int grid, bool persistent, cudaStream_t s,
-                                  int threads, int variant = 0);
-int persistent_grid_2c_mixed_fused(int threads = 128, int ctas_per_sm = 0, int variant = 0);
+// mixed-precision pass of the classes with min(la, lb) < kMixedFp64MinL (arguments as launch_2c_fused)
+cudaError_t launch_2c_mixed(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
 int persistent_grid_2c_grad(int op, int precision);
 int persistent_grid_3c(int precision);
 cudaError_t launch_2c(const Args2c &args, int op, int precision, int n_tiles_or_grid, bool persistent,
                       cudaStream_t s, int threads = 128);
 int persistent_grid_2c(int op, int precision, int threads = 128, int ctas_per_sm = 0);
-// variant (persistent launches): 0 = the compiler's register allocation, 1 = at
-// most 170 registers (three 128-thread CTAs per SM), 2 = at most 128 (four)
-cudaError_t launch_2c_fused(const ArgsFused &args, int n_tiles_or_grid, bool persistent, cudaStream_t s,
-                            int threads, int variant = 0);
-int persistent_grid_2c_fused(int threads = 128, int ctas_per_sm = 0, int variant = 0);
+// FP64 pass of the operators in args.r.want; persistent when args.counter is set, else one warp per tile.
+// ctas_per_sm: 0 = as many as fit.  variant: register cap (shg_plan_2c_set_variant)
+cudaError_t launch_2c_fused(const ArgsFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
+cudaError_t launch_2c_all(const ArgsFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
+cudaError_t launch_2c_one(const ArgsFused &args, cudaStream_t s, int threads, int ctas_per_sm);
 cudaError_t launch_pack_centers(const double *raw, int n, Vec4 *ctr, MixCenter *mctr, int *bad, cudaStream_t s);
 cudaError_t launch_family_radial(const ArgsFam &a, int op, cudaStream_t s);
 cudaError_t launch_gather_i64(const int64_t *src, const int32_t *idx, int64_t n, int64_t *dst, cudaStream_t s);

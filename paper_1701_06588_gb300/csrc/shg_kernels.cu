@@ -1,5 +1,5 @@
-// CUDA kernels of the SHG integral library (sm_103a), FP64 two-center path,
-// planning kernels, Boys debug kernel and the ALU throughput probe.
+// CUDA kernels of the SHG integral library (sm_103a): FP64 two-center passes of (a|r_a^{2n}|b) and of
+// precomputed radial terms (the other operators: shg_pair2c.cuh), planning kernels, Boys debug kernel and the ALU throughput probe.
 //
 // Two-center integrals follow Sec. II B of Golze et al. (arXiv:1701.06588):
 //   (a|O|b) = (-1)^lb A_{la,ma} A_{lb,mb} sum_j 2^{la+lb-j} O^{(la+lb-j)}
@@ -15,6 +15,7 @@
 // lanes run the same loop trip counts.
 
 #include "shg_cg.cuh"
+#include "shg_tilemap.cuh"
 
 #include <cstdio>
 
@@ -37,13 +38,6 @@ __device__ void pair_2c_fp64(const Args2c &g, int p)
     const double vx = A.x - B.x, vy = A.y - B.y, vz = A.z - B.z;
     const double R2 = vx * vx + vy * vy + vz * vz;
     const int kmax = la + lb;
-    if ((OP == OP_OVERLAP || OP == OP_GAUSS) && g.screen_thresh > 0.0 &&
-        screen_bound(g.screen[g.pair_a[p]], g.screen[g.pair_b[p]], R2, OP, g.omega) < g.screen_thresh) {
-        double *o = g.out + g.out_off[p];
-        for (int i = 0; i < (2 * la + 1) * (2 * lb + 1); ++i) o[i] = 0.0;
-        return;
-    }
-
     double O[J], E[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) O[j] = E[j] = 0.0;
@@ -64,7 +58,7 @@ __device__ void pair_2c_fp64(const Args2c &g, int p)
 
     double P[cg::kNP2], PF[cg::kNP2], C[2 * kLmax2c + 1], S[2 * kLmax2c + 1];
     cg::harmonics(vx, vy, vz, R2, kmax, J, g.k, P, C, S);
-    cg::block_from_orders<J>(g.cg, la, lb, R2, O, P, C, S, PF, g.out + g.out_off[p]);
+    cg::block_from_orders<J>(g.cg, la, lb, R2, O, 0.0, P, C, S, PF, 0, 1, g.out + g.out_off[p]);
 }
 
 // ------------------------------------------------------------------------- //
@@ -303,19 +297,15 @@ __device__ __forceinline__ void pair_2c_fp64_dispatch(const Args2c &g, int p, in
     }
 }
 
-__device__ __forceinline__ void run_tile_fp64(const Args2c &g, int op, const Tile &t, int lane)
+__device__ __forceinline__ void run_tile_fp64(const Args2c &g, int op, int t, int lane)
 {
-    if (lane >= t.count) return;
-    const int p = g.perm[t.start + lane];
-    const int la = t.cls / (kLmax2c + 1), lb = t.cls % (kLmax2c + 1);
+    int cls;
+    const int q = map_pair(g.map, t, lane, cls);
+    if (q < 0) return;
+    const int p = g.perm[q];
+    const int la = cls / (kLmax2c + 1), lb = cls % (kLmax2c + 1);
     const int J = (la < lb ? la : lb) + 1;
     switch (op) {
-    case OP_OVERLAP: pair_2c_fp64_dispatch<OP_OVERLAP>(g, p, J); break;
-    case OP_COULOMB: pair_2c_fp64_dispatch<OP_COULOMB>(g, p, J); break;
-    case OP_ERFC: pair_2c_fp64_dispatch<OP_ERFC>(g, p, J); break;
-    case OP_ERF: pair_2c_fp64_dispatch<OP_ERF>(g, p, J); break;
-    case OP_GAUSS: pair_2c_fp64_dispatch<OP_GAUSS>(g, p, J); break;
-    case OP_GCOUL: pair_2c_fp64_dispatch<OP_GCOUL>(g, p, J); break;
     case OP_RA2N: pair_2c_fp64_dispatch<OP_RA2N>(g, p, J); break;
     default: pair_2c_fp64_dispatch<OP_PRE>(g, p, J); break;
     }
@@ -328,7 +318,7 @@ __global__ void __launch_bounds__(128) k_2c_fp64_static(const Args2c g)
     const int lane = threadIdx.x & 31;
     const int t = g.tile_begin + warp;
     if (t >= g.tile_end) return;
-    run_tile_fp64(g, OP, g.tiles[t], lane);
+    run_tile_fp64(g, OP, t, lane);
 }
 
 template <int OP>
@@ -340,7 +330,7 @@ __global__ void __launch_bounds__(128) k_2c_fp64_persistent(const Args2c g)
         if (lane == 0) t = atomicAdd(g.counter, 1);
         t = __shfl_sync(0xffffffffu, t, 0) + g.tile_begin;
         if (t >= g.tile_end) break;
-        run_tile_fp64(g, OP, g.tiles[t], lane);
+        run_tile_fp64(g, OP, t, lane);
         __syncwarp();
     }
 }
@@ -400,7 +390,8 @@ __global__ void k_classify_3c(int64_t n, const int32_t *__restrict__ ta, const i
 //   cursor[r]            offset of bin r inside its chunk (the scatter cursor)
 //   bin_start[c*chunk]   first pair of chunk c
 //   tile_start[c*chunk]  first tile of chunk c; tile_start[n_bins] = all tiles
-// Every block scans its own chunk and posts the chunk's count; the last block
+// A chunk falls into ranges of ranks with one group size each (GroupRanges).
+// Every block scans its own chunk and posts the chunk's counts; the last block
 // to finish (an atomic ticket, *ticket zero on entry) scans the counts.  No
 // block waits for another.
 __device__ __forceinline__ int block_incl_scan(int x, int *s_warp)
@@ -428,7 +419,19 @@ __device__ __forceinline__ int block_incl_scan(int x, int *s_warp)
     return r;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_chunks(int n_bins, int chunk, const int *__restrict__ hist,
+// end[i]: first rank of a chunk after the range of group size kGroupOf[i]
+struct GroupRanges {
+    int end[kNGroups];
+};
+
+__device__ __forceinline__ int tiles_of(int n, int i)
+{
+    const int cap = kTile >> (kNGroups - 1 - i);
+    return (n + cap - 1) / cap;
+}
+
+__global__ void __launch_bounds__(1024) k_scan_chunks(int n_bins, int chunk, GroupRanges gr,
+                                                      const int *__restrict__ hist,
                                                       int *__restrict__ bin_start, int *__restrict__ cursor,
                                                       int *__restrict__ tile_start, int *ticket,
                                                       int *__restrict__ summary, const int *err)
@@ -440,9 +443,15 @@ __global__ void __launch_bounds__(1024) k_scan_chunks(int n_bins, int chunk, con
     const int v = hist[r];
     const int incl = block_incl_scan(v, s_warp);
     cursor[r] = incl - v;
-    if (threadIdx.x == blockDim.x - 1) {
-        bin_start[c * chunk] = incl;                  // the chunk's count for now
-        __threadfence();
+    // entries up to the end of each range but the last, and the chunk's count for now
+    for (int i = 0; i + 1 < kNGroups; ++i) {
+        if ((int)threadIdx.x == gr.end[i] - 1) bin_start[c * chunk + 1 + i] = incl;
+        if (gr.end[i] == 0 && threadIdx.x == 0) bin_start[c * chunk + 1 + i] = 0;
+    }
+    if (threadIdx.x == blockDim.x - 1) bin_start[c * chunk] = incl;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
         s_last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
     }
     __syncthreads();
@@ -451,13 +460,19 @@ __global__ void __launch_bounds__(1024) k_scan_chunks(int n_bins, int chunk, con
     // last block: offsets of the chunks (gridDim.x <= blockDim.x chunks, one per thread)
     const int k = threadIdx.x;
     const int cnt = k < (int)gridDim.x ? __ldcg(bin_start + k * chunk) : 0;
-    const int til = (cnt + kTile - 1) / kTile;
+    int til = 0;
+    for (int i = 0, done = 0; i < kNGroups && k < (int)gridDim.x; ++i) {
+        const int upto = i + 1 < kNGroups ? __ldcg(bin_start + k * chunk + 1 + i) : cnt;
+        til += tiles_of(upto - done, i);
+        done = upto;
+    }
     const int ic = block_incl_scan(cnt, s_warp);
     const int it = block_incl_scan(til, s_warp);
     if (k < (int)gridDim.x) {
         bin_start[k * chunk] = ic - cnt;
         tile_start[k * chunk] = it - til;
         summary[k] = it - til;
+        summary[gridDim.x + 2 + k] = ic - cnt;
     }
     if (k == (int)gridDim.x - 1) {
         tile_start[n_bins] = it;
@@ -490,13 +505,20 @@ __global__ void k_make_tiles(int n_chunks, int chunk, int bins_per_class, int n_
             if (tile_start[mid * chunk] <= t) lo = mid;
             else hi = mid;
         }
-        const int first = bin_start[lo * chunk] + (t - tile_start[lo * chunk]) * kTile;
-        const int end = lo + 1 < n_chunks ? bin_start[(lo + 1) * chunk] : n_pairs;
+        const int base = bin_start[lo * chunk];
+        const int cnt = (lo + 1 < n_chunks ? bin_start[(lo + 1) * chunk] : n_pairs) - base;
+        int q = t - tile_start[lo * chunk], i = 0, done = 0, upto = bin_start[lo * chunk + 1];
+        for (int nt; q >= (nt = tiles_of(upto - done, i)); ++i) {
+            q -= nt;
+            done = upto;
+            upto = i + 2 < kNGroups ? bin_start[lo * chunk + 2 + i] : cnt;
+        }
+        const int cap = kTile >> (kNGroups - 1 - i), first = done + q * cap;
         Tile tl;
-        tl.start = first;
-        tl.count = end - first < kTile ? end - first : kTile;
-        tl.cls = rank_to_bin[lo * chunk] / bins_per_class;
-        tl.pad = 0;
+        tl.start = base + first;
+        tl.count = (uint8_t)(upto - first < cap ? upto - first : cap);
+        tl.cls = (uint16_t)(rank_to_bin[lo * chunk] / bins_per_class);
+        tl.group = (uint8_t)(kTile / cap);
         tiles[t] = tl;
     }
 }
@@ -584,7 +606,7 @@ __global__ void __launch_bounds__(256) k_dmma_probe(int iters, double *sink)
 cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d_bin_rank, cudaStream_t s)
 {
     // d_ws layout (plan_ws_ints): err | ticket | 2 spare | hist[n_bins] | bin_start[n_bins] | cursor[n_bins] |
-    // tile_start[n_bins+1] | summary[n_chunks+2] | key[n]; one memset clears err, ticket and hist.
+    // tile_start[n_bins+1] | summary[2 n_chunks+2] | key[n]; one memset clears err, ticket and hist.
     // d_bin_rank: bin_rank[n_bins] followed by rank_to_bin[n_bins]
     const int64_t n = plan.n_pairs;
     int *d_err = d_ws;
@@ -596,7 +618,7 @@ cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d
     const int bpc = plan.kind == 2 ? kKbins2c : kKbins3c;
     const int n_chunks = n_bins / bpc;
     int *summary = tile_start + n_bins + 1;
-    int *key = summary + n_chunks + 2;
+    int *key = summary + 2 * n_chunks + 2;
     cudaError_t e = cudaMemsetAsync(d_ws, 0, sizeof(int) * (4 + (size_t)n_bins), s);
     if (e != cudaSuccess) return e;
     const int threads = 256;
@@ -610,9 +632,12 @@ cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d
                                                  d_bin_rank, key, hist, d_err);
     }
     // both rank orders are class-major (each class a chunk of bins_per_class ranks): one tiling per class
-    k_scan_chunks<<<n_chunks, bpc, 0, s>>>(n_bins, bpc, hist, bin_start, cursor, tile_start, ticket, summary, d_err);
+    // rank r of a two-center chunk holds Ka*Kb = kKbins2c - r; triples have one lane each
+    GroupRanges gr{};
+    for (int i = 0; i < kNGroups; ++i) gr.end[i] = plan.kind == 2 ? bpc - kGroupMinK[i] + 1 : (i + 1 < kNGroups ? 0 : bpc);
+    k_scan_chunks<<<n_chunks, bpc, 0, s>>>(n_bins, bpc, gr, hist, bin_start, cursor, tile_start, ticket, summary, d_err);
     if (n > 0) k_scatter<<<blocks, threads, 0, s>>>(n, bpc, key, bin_start, cursor, plan.perm);
-    const int64_t max_tiles = n / kTile + n_chunks + 1;
+    const int64_t max_tiles = plan_max_tiles(n, n_chunks, plan.kind == 2);
     const int tb = (int)((max_tiles + 255) / 256 < 1024 ? (max_tiles + 255) / 256 : 1024);
     k_make_tiles<<<tb, 256, 0, s>>>(n_chunks, bpc, bpc, (int)n, bin_start, tile_start, d_bin_rank + n_bins,
                                     plan.tiles);
@@ -637,12 +662,6 @@ cudaError_t launch_2c(const Args2c &a, int op, int precision, int n, bool persis
 {
     (void)precision;
     switch (op) {
-    case OP_OVERLAP: return launch_2c_op<OP_OVERLAP>(a, n, threads, persistent, s);
-    case OP_COULOMB: return launch_2c_op<OP_COULOMB>(a, n, threads, persistent, s);
-    case OP_ERFC: return launch_2c_op<OP_ERFC>(a, n, threads, persistent, s);
-    case OP_ERF: return launch_2c_op<OP_ERF>(a, n, threads, persistent, s);
-    case OP_GAUSS: return launch_2c_op<OP_GAUSS>(a, n, threads, persistent, s);
-    case OP_GCOUL: return launch_2c_op<OP_GCOUL>(a, n, threads, persistent, s);
     case OP_RA2N: return launch_2c_op<OP_RA2N>(a, n, threads, persistent, s);
     case OP_PRE: return launch_2c_op<OP_PRE>(a, n, threads, persistent, s);
     default: return cudaErrorInvalidValue;
@@ -657,12 +676,6 @@ int persistent_grid_2c(int op, int precision, int threads, int ctas_per_sm)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaSuccess;
     switch (op) {
-    case OP_OVERLAP: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_OVERLAP>, threads, 0); break;
-    case OP_COULOMB: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_COULOMB>, threads, 0); break;
-    case OP_ERFC: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_ERFC>, threads, 0); break;
-    case OP_ERF: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_ERF>, threads, 0); break;
-    case OP_GAUSS: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_GAUSS>, threads, 0); break;
-    case OP_GCOUL: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_GCOUL>, threads, 0); break;
     case OP_RA2N: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_RA2N>, threads, 0); break;
     default: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_2c_fp64_persistent<OP_PRE>, threads, 0); break;
     }

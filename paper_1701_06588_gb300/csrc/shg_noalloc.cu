@@ -32,7 +32,7 @@ namespace {
 
 constexpr int64_t kNoAllocMaxPairs = int64_t(1) << 20;
 // layout: tiles | perm | counter, err | key | hist | bin_start | cursor | tile_start
-constexpr int64_t kNoAllocMaxTiles = kNoAllocMaxPairs / kTile + kNBins2c + 1;
+constexpr int64_t kNoAllocMaxTiles = plan_max_tiles(kNoAllocMaxPairs, kNClass, true);
 constexpr size_t kTilesBytes = ((size_t)kNoAllocMaxTiles * sizeof(Tile) + 255) / 256 * 256;
 constexpr size_t kPermBytes = ((size_t)kNoAllocMaxPairs * sizeof(int32_t) + 255) / 256 * 256;
 constexpr size_t kFlagsBytes = 256;
@@ -109,16 +109,27 @@ extern "C" int shg_eval_2c_noalloc(const shg_basis_t *basis, int64_t n_pairs, co
     int *ws = (int *)c;
 
     cudaError_t e = launch_plan_build(plan, ws, kNBins2c, ranks[SHG_SCHED_PERSISTENT], s);
-    // the end of the build summary: tile count and error flag
-    int h_sum[2] = {0, 0};
+    int summary[2 * kNClass + 2] = {};
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h_sum, plan_summary(ws, kNBins2c) + kNClass, sizeof(h_sum), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(summary, plan_summary(ws, kNBins2c), sizeof(summary), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(SHG_ECUDA, "shg_eval_2c_noalloc planning: %s", cudaGetErrorString(e));
-    if (h_sum[1]) return fail(SHG_EINVAL, "pair list holds a shell index outside 0..%d", b.n_shells - 1);
-    const int n_tiles = h_sum[0];
+    if ((r = plan_read(plan, summary, SHG_SCHED_PERSISTENT)) != SHG_OK) return r;
+    const int n_tiles = plan.n_tiles;
     if (n_tiles <= 0) return SHG_OK;
 
+    if (op <= SHG_OP_GAUSS_COULOMB) {
+        ArgsFused f;
+        fused_ops(f, 1, &op, &omega, &d_out);
+        fused_plan(f, b, plan, *t, d_out_offsets);
+        f.tile_begin = 0;
+        f.tile_end = n_tiles;
+        f.counter = plan.counter;
+        e = cudaMemsetAsync(plan.counter, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = launch_2c_fused(f, s, plan.threads, plan.ctas_per_sm, plan.variant);
+        if (e != cudaSuccess) return fail(SHG_ECUDA, "shg_eval_2c_noalloc launch: %s", cudaGetErrorString(e));
+        return SHG_OK;
+    }
     Args2c a;
     a.shells = b.shells;
     a.prims = b.prims;
@@ -126,15 +137,13 @@ extern "C" int shg_eval_2c_noalloc(const shg_basis_t *basis, int64_t n_pairs, co
     a.pair_a = d_pair_a;
     a.pair_b = d_pair_b;
     a.perm = plan.perm;
-    a.tiles = plan.tiles;
+    a.map = plan.map;
     a.tile_begin = 0;
-    a.tile_end = n_tiles;
+    a.tile_end = plan.map.tile[kNClass];
     a.counter = plan.counter;
     a.out_off = reinterpret_cast<const long long *>(d_out_offsets);
     a.out = d_out;
     a.omega = omega;
-    a.screen_thresh = 0.0;
-    a.screen = b.screen;
     a.boys = t->boys;
     a.boys_e = t->boys_e;
     a.cg = t->cg;

@@ -70,6 +70,38 @@ SHG_HD xf mul(xf a, xf b)
     return xf{r << s, a.e + b.e + 64 - s};
 }
 
+// raw product of two normalised xf: significand in [2^60, 2^62), for one further product by muln
+SHG_HD xf mulr(xf a, xf b) { return xf{mulhi(a.m, b.m), a.e + b.e + 64}; }
+
+SHG_HD int clz32(uint32_t v)
+{
+#ifdef __CUDA_ARCH__
+    return __clz((int)v);
+#else
+    return __builtin_clz(v);
+#endif
+}
+
+// normalised product where one factor may be raw (significand at least 2^60; error below 2^-57)
+SHG_HD xf muln(xf a, xf b)
+{
+    const uint64_t r = mulhi(a.m, b.m);
+    const int s = clz32(hi32(r)) - 1;
+    return xf{r << s, a.e + b.e + 64 - s};
+}
+
+// v >> s, 0 for s > 63 (s >= 0)
+SHG_HD uint64_t shr(uint64_t v, int s)
+{
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+    return r;
+#else
+    return s > 63 ? 0 : v >> s;
+#endif
+}
+
 // x^n, n >= 1
 SHG_HD xf powi(xf x, int n)
 {
@@ -82,8 +114,7 @@ SHG_HD xf powi(xf x, int n)
 SHG_HD xf add(xf a, xf b)
 {
     const int e = a.e > b.e ? a.e : b.e;
-    const int da = e - a.e, db = e - b.e;
-    uint64_t m = (da < 64 ? a.m >> da : 0) + (db < 64 ? b.m >> db : 0);      // < 2^64
+    const uint64_t m = shr(a.m, e - a.e) + shr(b.m, e - b.e);                // < 2^64
     const int c = (int)(hi32(m) >> 31);
     return xf{m >> c, e + c};
 }
