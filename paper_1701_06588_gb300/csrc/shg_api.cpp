@@ -755,6 +755,7 @@ const Consts &consts()
 
 static void fill_kappa_mix(KappaMix &k)
 {
+    for (int n = 0; n < 32; ++n) k.inv[n] = n ? split2(1.0L / n) : make_float2(0, 0);
     for (int l = 0; l < 16; ++l)
         for (int m = 0; m < 16; ++m)
             k.v[l][m] = l && m <= l ? split2((long double)(l * l - m * m) / (4 * l * l - 1)) : make_float2(0, 0);
@@ -1738,72 +1739,62 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     if (r) return r;
     const DeviceTables *t = device_tables();
     cudaStream_t s = (cudaStream_t)stream;
-    Args2c a{};
-    a.shells = basis->d.shells;
-    a.prims = basis->d.prims;
-    a.centers = basis->d.centers;
-    a.pair_a = pa;
-    a.pair_b = pb;
-    a.perm = p->d.perm;
-    a.map = p->d.map;
-    a.tile_begin = 0;
-    a.counter = p->d.counter;
-    a.omega = omega;
-    a.boys = t->boys;
-    a.boys_e = t->boys_e;
-    a.w_off = reinterpret_cast<const long long *>(w_off);
+    cudaError_t e = cudaMemsetAsync(p->d.counter, 0, sizeof(int), s);
+    if (op == SHG_OP_RA2N) {
+        Args2c a{};
+        a.shells = basis->d.shells;
+        a.prims = basis->d.prims;
+        a.centers = basis->d.centers;
+        a.pair_a = pa;
+        a.pair_b = pb;
+        a.perm = p->d.perm;
+        a.map = p->d.map;
+        a.tile_begin = 0;
+        a.tile_end = p->d.map.tile[kNClass];
+        a.counter = p->d.counter;
+        a.omega = omega;
+        a.w_off = reinterpret_cast<const long long *>(w_off);
+        a.w = w;
+        a.grad_a = grad_a;
+        a.grad_b = grad_b;
+        a.cg = t->cg;
+        a.k = consts();
+        if (e == cudaSuccess) e = launch_2c_grad_ra2n(a, s);
+        shg_plan_destroy(p);
+        return e == cudaSuccess ? SHG_OK : fail(SHG_ECUDA, "gradient launch: %s", cudaGetErrorString(e));
+    }
+    ArgsGrad a;
+    double *none = nullptr;
+    fused_ops(a.f, 1, &op, &omega, &none);
+    // fused_ops reads the wanted sums off the outputs
+    a.f.r.want = op == SHG_OP_OVERLAP ? kSumOv : op == SHG_OP_COULOMB ? kSumCo : op == SHG_OP_ERFC ? kSumCo | kSumX
+                 : op == SHG_OP_ERF ? kSumEr : op == SHG_OP_GAUSS ? kSumGa : kSumGc;
+    fused_plan(a.f, basis->d, p->d, *t, w_off);
+    fill_kappa_mix(a.kappa);
     a.w = w;
     a.grad_a = grad_a;
     a.grad_b = grad_b;
-    a.k = consts();
-    // mixed precision: the classes with both l >= kMixedFp64MinL (the leading
-    // tiles of the persistent order) in FP64, the others with double-float
-    // radial orders and the FP64 angular part.  With both kinds present the
-    // two launches run side by side on the plan's side streams (as in
-    // shg_plan_2c_exec_fused): the FP64 tiles one warp each, statically.
+    // mixed precision: the classes with both l >= kMixedFp64MinL (the leading tiles of the persistent order) in FP64.
+    // With both kinds present the two launches run side by side on the plan's side streams (as the integrals), the
+    // FP64 tiles one warp each, statically.
     const bool mixed = precision == SHG_PREC_MIXED;
-    const int hi_tiles = p->d.mixed_fp64_tiles32, all_tiles = p->d.map.tile[kNClass];
-    const bool fork = mixed && hi_tiles > 0 && all_tiles > hi_tiles;
-    a.tile_end = mixed ? hi_tiles : all_tiles;
-    cudaError_t e = cudaSuccess;
-    if (fork) {
-        r = fork_sides(p, s);
-        if (r) {
-            shg_plan_destroy(p);
-            return r;
-        }
-        a.counter = nullptr;
-        e = launch_2c_grad(a, op, SHG_PREC_FP64, 0, p->d.side, 32);
-    } else if (a.tile_end > 0) {
-        e = cudaMemsetAsync(p->d.counter, 0, sizeof(int), s);
-        if (e == cudaSuccess) e = launch_2c_grad(a, op, SHG_PREC_FP64, persistent_grid_2c_grad(op, SHG_PREC_FP64), s);
+    const int hi = mixed ? p->d.mixed_fp64_tiles : p->d.n_tiles, all = p->d.n_tiles;
+    const bool fork = mixed && hi > 0 && all > hi;
+    if (fork && (r = fork_sides(p, s)) != SHG_OK) {
+        shg_plan_destroy(p);
+        return r;
     }
-    if (e == cudaSuccess && mixed && all_tiles > hi_tiles) {
-        ArgsGradMix gm;
-        gm.g = a;
-        ArgsMix &m = gm.m;
-        m.shells = basis->d.shells;
-        m.prims = basis->d.mprims;
-        m.centers = basis->d.mcenters;
-        m.pair_a = pa;
-        m.pair_b = pb;
-        m.perm = p->d.perm;
-        gm.g.tile_begin = hi_tiles;
-        gm.g.tile_end = all_tiles;
-        m.counter = p->d.counter;
-        m.out_off = nullptr;
-        m.out = nullptr;
-        m.omega = split2(omega);
-        m.omega2 = split2((long double)omega * omega);
-        m.omega_d = omega;
-        m.screen_thresh = 0.0;
-        m.screen = basis->d.screen;
-        m.boys = t->boys_mix;
-        m.boys_e = t->boys_e_mix;
-        m.km = consts_mix();
-        const cudaStream_t sm = fork ? p->d.side2 : s;
-        e = cudaMemsetAsync(p->d.counter, 0, sizeof(int), sm);
-        if (e == cudaSuccess) e = launch_2c_grad_mixed(gm, op, sm);
+    if (e == cudaSuccess && hi > 0) {
+        a.f.tile_begin = 0;
+        a.f.tile_end = hi;
+        a.f.counter = fork ? nullptr : p->d.counter;
+        e = launch_2c_grad(a, fork ? p->d.side : s, fork ? 32 : 128);
+    }
+    if (e == cudaSuccess && all > hi) {
+        a.f.tile_begin = hi;
+        a.f.tile_end = all;
+        a.f.counter = p->d.counter;
+        e = launch_2c_grad_mixed(a, fork ? p->d.side2 : s, 128);
     }
     // the plan's memory is released in the order of s: join first, also after
     // a failed launch (the other side stream may hold a running kernel)

@@ -171,9 +171,10 @@ struct CGTab {
     const float2 *gm;             // g as double-float
 };
 
-// kappa of Consts as double-float (mixed-precision angular part)
+// kappa of Consts and 1/n as double-float (mixed-precision angular part)
 struct KappaMix {
     float2 v[16][16];
+    float2 inv[32];
 };
 
 // Device-resident tables owned by the library, one set per device.
@@ -400,19 +401,19 @@ struct ArgsMix {
     ConstsMix km;
 };
 
-// Mixed-precision gradient: double-float radial orders (m) and the FP64 angular
-// vector-Jacobian product (g: centers, constants, upstream weights, outputs).
-struct ArgsGradMix;
-
 // Mixed-precision pass: radial sums as the FP64 pass, angular part in double-float.
 struct ArgsMixFused {
     ArgsFused f;
     KappaMix kappa;
 };
 
-struct ArgsGradMix {
-    Args2c g;
-    ArgsMix m;
+// Vector-Jacobian product of one operator: the pass's pair, radial and table arguments (out unused), upstream weights
+// (blocks at w + f.out_off[p]) and per-pair results; kappa for the mixed-precision launch.
+struct ArgsGrad {
+    ArgsFused f;
+    KappaMix kappa;
+    const double *w;
+    double *grad_a, *grad_b;      // grad_b may be null
 };
 
 // Arguments of the three-index kernels (by value).
@@ -462,12 +463,13 @@ int plan_read(PlanDev &d, const int *summary, int schedule);
 inline int *plan_summary(int *ws, int n_bins) { return ws + 4 + 4 * (size_t)n_bins + 1; }
 cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d_bin_rank, cudaStream_t s);
 cudaError_t launch_3c(const Args3c &args, int precision, int grid, cudaStream_t s);
-// grid is ignored when args.counter is null (static launch, one warp per tile)
-cudaError_t launch_2c_grad(const Args2c &args, int op, int precision, int grid, cudaStream_t s, int threads = 128);
-cudaError_t launch_2c_grad_mixed(const ArgsGradMix &args, int op, cudaStream_t s);
+// vector-Jacobian products (persistent when the counter is set, else one warp per tile): FP64, mixed precision, and
+// (a|r_a^{2n}|b) (32-pair tiles of the map)
+cudaError_t launch_2c_grad(const ArgsGrad &args, cudaStream_t s, int threads);
+cudaError_t launch_2c_grad_mixed(const ArgsGrad &args, cudaStream_t s, int threads);
+cudaError_t launch_2c_grad_ra2n(const Args2c &args, cudaStream_t s);
 // mixed-precision pass of the classes with min(la, lb) < kMixedFp64MinL (arguments as launch_2c_fused)
 cudaError_t launch_2c_mixed(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
-int persistent_grid_2c_grad(int op, int precision);
 int persistent_grid_3c(int precision);
 cudaError_t launch_2c(const Args2c &args, int op, int precision, int n_tiles_or_grid, bool persistent,
                       cudaStream_t s, int threads = 128);
