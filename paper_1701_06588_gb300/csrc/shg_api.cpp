@@ -303,51 +303,20 @@ void fill_consts3(Consts3 &k)
     std::memset(&k, 0, sizeof k);
     for (int n = 0; n < 18; ++n)
         for (int i = 0; i <= n; ++i) k.binom[n][i] = (double)(lfact(n) / (lfact(i) * lfact(n - i)));
-    // d_{m,j} = 2^j (2m+1)!! binom(m,j) / (2j+1)!!   (Eq. I_jab); dd[m][i][j] = d_{m,j} j!/(j-i)!
-    auto dfact = [](int n) { long double f = 1; for (int i = n; i > 1; i -= 2) f *= i; return f; };
+    // L_m^{(1/2)}(-u) = sum_j binom(m + 1/2, m - j) u^j / j!
     for (int m = 0; m < 6; ++m)
         for (int j = 0; j <= m; ++j) {
-            const long double d = std::ldexp(1.0L, j) * dfact(2 * m + 1) * (lfact(m) / (lfact(j) * lfact(m - j))) /
-                                  dfact(2 * j + 1);
-            for (int i = 0; i <= j; ++i) k.dd[m][i][j] = (double)(d * lfact(j) / lfact(j - i));
+            long double v = 1;
+            for (int i = 0; i < m - j; ++i) v *= (m + 0.5L - i) / (i + 1);
+            k.lag[m][j] = (double)(v / lfact(j));
         }
-    // binom(p, j) (L)_j with the rising factorial (L)_j = L (L+1) ... (L+j-1), (0)_0 = 1, (0)_j = 0
     for (int L = 0; L < 11; ++L)
         for (int p = 0; p < 6; ++p)
-            for (int j = 0; j <= p; ++j) {
+            for (int m = 0; m <= p; ++m) {
                 long double r = 1;
-                for (int i = 0; i < j; ++i) r *= (L + i);
-                k.bj[L][p][j] = (double)((lfact(p) / (lfact(j) * lfact(p - j))) * r);
+                for (int i = 0; i < p - m; ++i) r *= (L + i);
+                k.K[L][p][m] = (double)((lfact(p) / (lfact(m) * lfact(p - m))) * r * lfact(m));
             }
-    for (int n = 0; n < 32; ++n) k.sqrt_int[n] = (double)std::sqrt((long double)n);
-}
-
-// Real orthonormal spherical harmonics Y_{l,m} = A_{l,|m|} R^{c/s}_{l,|m|} / sqrt(4pi/(2l+1))
-// at a unit vector (Sec. II E recursions), l <= lmax, stored at l*l + l + m.
-static void real_ylm(long double x, long double y, long double z, int lmax, long double *Y)
-{
-    long double Rc[16][16] = {}, Rs[16][16] = {};
-    const long double r2 = x * x + y * y + z * z;
-    Rc[0][0] = 1;
-    for (int l = 0; l < lmax; ++l) {
-        Rc[l + 1][l + 1] = -(x * Rc[l][l] - y * Rs[l][l]) / (2 * l + 2);
-        Rs[l + 1][l + 1] = -(y * Rc[l][l] + x * Rs[l][l]) / (2 * l + 2);
-        for (int m = 0; m <= l; ++m) {
-            const long double pc = (l >= 1 && m <= l - 1) ? Rc[l - 1][m] : 0, ps = (l >= 1 && m <= l - 1) ? Rs[l - 1][m] : 0;
-            Rc[l + 1][m] = ((2 * l + 1) * z * Rc[l][m] - r2 * pc) / ((l + m + 1) * (l - m + 1));
-            Rs[l + 1][m] = ((2 * l + 1) * z * Rs[l][m] - r2 * ps) / ((l + m + 1) * (l - m + 1));
-        }
-    }
-    const long double pi = 3.14159265358979323846264338327950288L;
-    for (int l = 0; l <= lmax; ++l) {
-        const long double nrm = std::sqrt((2 * l + 1) / (4 * pi));
-        for (int m = -l; m <= l; ++m) {
-            const int mu = m < 0 ? -m : m;
-            long double A = std::sqrt((long double)(mu == 0 ? 1 : 2) * lfact(l + mu) * lfact(l - mu));
-            if (mu & 1) A = -A;
-            Y[l * l + l + m] = nrm * A * (m >= 0 ? Rc[l][mu] : Rs[l][mu]);
-        }
-    }
 }
 
 // Gauss-Legendre nodes and weights on [-1, 1] (Newton on P_n).
@@ -378,7 +347,7 @@ static void gauss_legendre(int n, std::vector<long double> &x, std::vector<long 
 // Coefficients of the expanded angular part (layout at CGTab).  With S_{l,+-m} = nu_{l,m} p_{l,m}(z, r^2) {C_m, S_m},
 // nu_{l,m} = sqrt((2 - delta_{m0}) (l-m)!/(l+m)!) (2l-1)!!/(l-m)!, the product of the two theta functions is
 // expanded in those of (L, M) by Gauss-Legendre quadrature exact for the degrees (<= 2 (kLmaxAabA + kLmax2c)).
-static void make_cg(std::vector<double> &g, std::vector<int> &gbase, std::vector<double> &fc)
+static void make_cg(std::vector<double> &g, std::vector<double> &h, std::vector<int> &gbase, std::vector<double> &fc)
 {
     const int lmax = kLmaxAabA + kLmax2c, nq = 24;
     std::vector<long double> x, w;
@@ -416,13 +385,15 @@ static void make_cg(std::vector<double> &g, std::vector<int> &gbase, std::vector
                     for (int s = 0; s < 2; ++s)
                         for (int p = 0; p < J; ++p) {
                             const int L = la + lb - 2 * p, M = s ? a + b : std::abs(a - b);
-                            long double v = 0;
+                            long double v = 0, vh = 0;
                             if (M <= L && !(s && (!a || !b))) {
                                 const long double *ta = theta(la, a), *tb = theta(lb, b), *tL = theta(L, M);
                                 for (int q = 0; q < nq; ++q) v += w[q] * ta[q] * tb[q] * tL[q];
-                                v *= (2 * L + 1) / (M ? 4.0L : 2.0L) * nu[L * (lmax + 1) + M] * (a && b ? 0.5L : 1.0L);
+                                vh = v * (2 * L + 1) / (M ? 4.0L : 2.0L) * (a && b ? 0.5L : 1.0L);
+                                v = vh * nu[L * (lmax + 1) + M];
                             }
                             g.push_back((double)v);
+                            if (la <= kLmax2c) h.push_back((double)vh);
                         }
             for (int p = 0; p < J; ++p)
                 for (int j = 0; j <= p; ++j) {
@@ -430,50 +401,6 @@ static void make_cg(std::vector<double> &g, std::vector<int> &gbase, std::vector
                     long double v = lfact(p) / (lfact(i) * lfact(p - i)) * std::ldexp((lb & 1) ? -1.0L : 1.0L, la + lb);
                     for (int q = i; q < p; ++q) v *= L + 1.5L + q;
                     fc[(size_t)c * 28 + p * (p + 1) / 2 + j] = (double)v;
-                }
-        }
-}
-
-// Real Gaunt coefficients G = int Y_{L,M} Y_{l,m} Y_{l~,m~} dOmega for
-// l, l~ <= 6, l + l~ <= kLmaxAabA, L = |l-l~|..l+l~ step 2 (the expansion of
-// Eq. CG_expansion written for real harmonics), by product quadrature that is
-// exact for these degrees: 16-point Gauss-Legendre in cos(theta) (polynomial
-// degree <= 20) times the 32-point trapezoid rule in phi (|frequency| <= 20).
-static void make_gaunt(std::vector<int> &base, std::vector<int> &row, std::vector<GauntEnt> &ent)
-{
-    const int nt = 16, np = 32, LY = 16;
-    const long double pi = 3.14159265358979323846264338327950288L;
-    std::vector<long double> gx, gw;
-    gauss_legendre(nt, gx, gw);
-    std::vector<double> Y((size_t)nt * np * LY * LY), W((size_t)nt * np);
-    long double Yl[LY * LY];
-    for (int i = 0; i < nt; ++i)
-        for (int j = 0; j < np; ++j) {
-            const long double ct = gx[i], st = std::sqrt(1 - ct * ct), ph = 2 * pi * j / np;
-            real_ylm(st * std::cos(ph), st * std::sin(ph), ct, 12, Yl);
-            for (int q = 0; q < LY * LY; ++q) Y[((size_t)i * np + j) * LY * LY + q] = (double)Yl[q];
-            W[(size_t)i * np + j] = (double)(gw[i] * 2 * pi / np);
-        }
-    base.assign(49, -1);
-    row.clear();
-    ent.clear();
-    row.push_back(0);
-    for (int l = 0; l <= 6; ++l)
-        for (int lt = 0; lt <= 6; ++lt) {
-            if (l + lt > kLmaxAabA) continue;
-            base[l * 7 + lt] = (int)row.size() - 1;
-            for (int m = -l; m <= l; ++m)
-                for (int mt = -lt; mt <= lt; ++mt) {
-                    for (int L = std::abs(l - lt); L <= l + lt; L += 2)
-                        for (int M = -L; M <= L; ++M) {
-                            double g = 0;
-                            for (size_t q = 0; q < W.size(); ++q) {
-                                const double *Yq = &Y[q * LY * LY];
-                                g += W[q] * Yq[L * L + L + M] * Yq[l * l + l + m] * Yq[lt * lt + lt + mt];
-                            }
-                            if (std::fabs(g) > 1e-13) ent.push_back(GauntEnt{g, L, M});
-                        }
-                    row.push_back((int)ent.size());
                 }
         }
 }
@@ -504,6 +431,7 @@ static double class_cost3(int la, int lt, int lb, int kk)
     return kk * rad + ang + (2.0 * la + 1) * (2 * lt + 1) * (2 * lb + 1) * nL * 2;
 }
 
+static int g_chunk_class3[kNClass3];        // class of every chunk of the three-index rank order
 static uint8_t g_chunk_class[2][kNClass];   // class of every chunk of a schedule's rank order (the same on all devices)
 
 static std::mutex g_mu;
@@ -636,6 +564,7 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
                 if (cx != cy) return ccost[cx] > ccost[cy] || (ccost[cx] == ccost[cy] && cx < cy);
                 return (x % kKbins3c) > (y % kKbins3c);
             });
+            for (int c = 0; c < kNClass3; ++c) g_chunk_class3[c] = order[(size_t)c * kKbins3c] / kKbins3c;
             for (int r = 0; r < kNBins3; ++r) {
                 rank3[order[r]] = r;
                 rank3[kNBins3 + r] = order[r];
@@ -643,30 +572,18 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
             ok = cudaMalloc(&d_r3, rank3.size() * sizeof(int)) == cudaSuccess &&
                  cudaMemcpy(d_r3, rank3.data(), rank3.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
         }
-        // real Gaunt coefficients
-        int *d_gb = nullptr, *d_gr = nullptr;
-        GauntEnt *d_ge = nullptr;
-        if (ok) {
-            std::vector<int> gb, gr;
-            std::vector<GauntEnt> ge;
-            make_gaunt(gb, gr, ge);
-            ok = cudaMalloc(&d_gb, gb.size() * sizeof(int)) == cudaSuccess &&
-                 cudaMalloc(&d_gr, gr.size() * sizeof(int)) == cudaSuccess &&
-                 cudaMalloc(&d_ge, ge.size() * sizeof(GauntEnt)) == cudaSuccess &&
-                 cudaMemcpy(d_gb, gb.data(), gb.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
-                 cudaMemcpy(d_gr, gr.data(), gr.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
-                 cudaMemcpy(d_ge, ge.data(), ge.size() * sizeof(GauntEnt), cudaMemcpyHostToDevice) == cudaSuccess;
-        }
-        double *d_cg = nullptr, *d_fc = nullptr;
+        double *d_cg = nullptr, *d_fc = nullptr, *d_ch = nullptr;
         float2 *d_cgm = nullptr;
         int *d_cgb = nullptr;
         if (ok) {
-            std::vector<double> cg, fc;
+            std::vector<double> cg, ch, fc;
             std::vector<int> cgb;
-            make_cg(cg, cgb, fc);
+            make_cg(cg, ch, cgb, fc);
+            ok = cudaMalloc(&d_ch, ch.size() * sizeof(double)) == cudaSuccess &&
+                 cudaMemcpy(d_ch, ch.data(), ch.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
             std::vector<float2> cgm(cg.size());
             for (size_t i = 0; i < cg.size(); ++i) cgm[i] = split2d(cg[i]);
-            ok = cudaMalloc(&d_cg, cg.size() * sizeof(double)) == cudaSuccess &&
+            ok = ok && cudaMalloc(&d_cg, cg.size() * sizeof(double)) == cudaSuccess &&
                  cudaMalloc(&d_fc, fc.size() * sizeof(double)) == cudaSuccess &&
                  cudaMalloc(&d_cgm, cgm.size() * sizeof(float2)) == cudaSuccess &&
                  cudaMemcpy(d_cgm, cgm.data(), cgm.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -692,11 +609,8 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
             return nullptr;
         }
         st.bin_rank3 = d_r3;
-        st.t.cg = CGTab{d_cg, d_cgb, d_fc, d_cgm};
+        st.t.cg = CGTab{d_cg, d_cgb, d_fc, d_cgm, d_ch};
         st.t.x = XTab{d_bc, d_ex};
-        st.t.gaunt_base = d_gb;
-        st.t.gaunt_row = d_gr;
-        st.t.gaunt = d_ge;
         st.t.boys_mix = d_mtab;
         st.t.boys_e_mix = d_metab;
         st.t.boys = d_tab;
@@ -1139,7 +1053,7 @@ int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, c
     if (!device_tables_impl(ranks)) return SHG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
-    const int64_t max_tiles = plan_max_tiles(n, kNClass, true);
+    const int64_t max_tiles = plan_max_tiles(n, kNClass);
     const size_t bytes_perm = sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1);
     const size_t bytes_tiles = sizeof(Tile) * (size_t)max_tiles;
     const size_t bytes_ws = sizeof(int) * plan_ws_ints(n, kNBins, kNClass);
@@ -1640,7 +1554,7 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     if (!t) return SHG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
 
-    const int64_t max_tiles = plan_max_tiles(n, kNClass3, false);
+    const int64_t max_tiles = plan_max_tiles(n, kNClass3);
     const size_t bytes_perm = sizeof(int32_t) * (size_t)n;
     const size_t bytes_tiles = sizeof(Tile) * (size_t)max_tiles;
     const size_t bytes_ws = sizeof(int) * plan_ws_ints(n, kNBins3, kNClass3);
@@ -1661,13 +1575,12 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     d.perm = (int32_t *)c;               c += (bytes_perm + 15) / 16 * 16;
     d.counter = (int *)c;                c += 16;
     int *ws = (int *)c;
-    // the end of the build summary: sm[0] = tile count, sm[1] = error flags
-    int sm[2] = {0, 0};
+    // first tile of every class chunk, tile count and error flags
+    int sm[kNClass3 + 2] = {};
     cudaError_t e = launch_plan_build(d, ws, kNBins3, rank3, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(sm, plan_summary(ws, kNBins3) + kNClass3, sizeof(sm), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sm, plan_summary(ws, kNBins3), sizeof(sm), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    const int h[2] = {sm[1], sm[0]};              // error flags, tile count
+    const int h[2] = {sm[kNClass3 + 1], sm[kNClass3]};              // error flags, tile count
     if (e != cudaSuccess) {
         cudaFreeAsync(blk, s);
         return fail(SHG_ECUDA, "(aab) planning: %s", cudaGetErrorString(e));
@@ -1681,8 +1594,8 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     Args3c a;
     a.orb_shells = orb->d.shells;
     a.aux_shells = aux->d.shells;
-    a.orb_prims = orb->d.prims;
-    a.aux_prims = aux->d.prims;
+    a.orb_prims = orb->d.xprims;
+    a.aux_prims = aux->d.xprims;
     a.orb_centers = orb->d.centers;
     a.aux_centers = aux->d.centers;
     a.t_a = ta;
@@ -1690,14 +1603,15 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     a.t_b = tb;
     a.perm = d.perm;
     a.tiles = d.tiles;
-    a.tile_begin = 0;
     a.tile_end = h[1];
+    a.slot_doubles = 0;
+    for (int c = 0; c < kNClass3; ++c)
+        if (sm[c + 1] > sm[c])
+            a.slot_doubles = std::max(a.slot_doubles,
+                                      grad_a ? slot_doubles_3c_grad(g_chunk_class3[c]) : slot_doubles_3c(g_chunk_class3[c]));
     a.counter = d.counter;
     a.out_off = reinterpret_cast<const long long *>(off);
     a.out = out;
-    a.gaunt_base = t->gaunt_base;
-    a.gaunt_row = t->gaunt_row;
-    a.gaunt = t->gaunt;
     a.w_off = grad_a ? reinterpret_cast<const long long *>(off) : nullptr;
     a.w = w;
     a.grad_a = grad_a;
@@ -1705,11 +1619,12 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     a.screen_thresh = grad_a ? 0.0 : screen;
     a.orb_screen = orb->d.screen;
     a.aux_screen = aux->d.screen;
+    a.exptab = t->x.exp;
+    a.cg = t->cg;
     a.k = consts();
     a.k3 = consts3();
-    a.km = consts_mix();
     e = cudaMemsetAsync(d.counter, 0, sizeof(int), s);
-    if (e == cudaSuccess && h[1] > 0) e = launch_3c(a, precision, persistent_grid_3c(precision), s);
+    if (e == cudaSuccess && h[1] > 0) e = grad_a ? launch_3c_grad(a, s) : launch_3c(a, s);
     cudaFreeAsync(blk, s);
     if (e != cudaSuccess) return fail(SHG_ECUDA, "(aab) launch: %s", cudaGetErrorString(e));
     return SHG_OK;

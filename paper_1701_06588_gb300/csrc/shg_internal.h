@@ -101,12 +101,6 @@ struct alignas(32) PrimRec {
     double alpha, inv_alpha, w2c, wN;
 };
 
-// Real Gaunt coefficient entry G = int Y_{L,M} Y_{l,m} Y_{l~,m~} dOmega.
-struct GauntEnt {
-    double g;
-    int L, M;
-};
-
 // Per-primitive weights of the Coulomb-type radial terms (Table S1), 16 bytes:
 //   cw = sqrt(2 pi^{5/2}) w2c / alpha   so that 2 pi^{5/2} w / (alpha beta sqrt(c)) = cw_a cw_b / sqrt(c)
 //   fw = w2c alpha^{-3/2}       the far-field weight: for T >= kBoysTmax every order of
@@ -169,6 +163,7 @@ struct CGTab {
     const int *gbase;
     const double *fc;
     const float2 *gm;             // g as double-float
+    const double *h;              // g without nu_{L,M}: coefficients of S_{L,M} in S_{la,ma} S_{lb,mb} (la, lb <= kLmax2c)
 };
 
 // kappa of Consts and 1/n as double-float (mixed-precision angular part)
@@ -181,23 +176,17 @@ struct KappaMix {
 struct DeviceTables {
     const double *boys;   // [kBoysGrid][kBoysN][kBoysStride] (layout above)
     const double *boys_e; // [kBoysGrid] exp(-T_i), T_i = i/32
-    // real Gaunt coefficients for l, l~ <= 6 with l + l~ <= kLmaxAabA:
-    // rows (l, l~, m, m~) -> entries [gaunt_row[r], gaunt_row[r+1]) of gaunt
-    const int *gaunt_base;     // [7*7] first row of the (l, l~) block
-    const int *gaunt_row;      // row pointers
-    const GauntEnt *gaunt;     // entries
     const float4 *boys_mix;    // [kBoysGrid][kBoysN][3] (layout above)
     const float2 *boys_e_mix;  // [kBoysGrid] exp(-T_i) as hi/lo
     CGTab cg;
     XTab x;
 };
 
-// Extra constants of the three-index kernels (by value).
+// Constants of the three-index kernels (by value).
 struct Consts3 {
     double binom[18][18];       // binom(k, i)
-    double dd[6][6][6];         // d_{m,j} j!/(j-i)!: D_m^{(i)}(x) = sum_j dd[m][i][j] x^{j-i}
-    double bj[11][6][6];        // binom(p, j) (L)_j (rising factorial, (0)_0 = 1)
-    double sqrt_int[32];        // sqrt(n)
+    double lag[6][6];           // coefficient of u^j in the Laguerre polynomial L_m^{(1/2)}(-u)
+    double K[11][6][6];         // [L][p][m]: binom(p, m) (L)_{p-m} m! (rising factorial, (0)_0 = 1)
 };
 
 void fill_consts3(Consts3 &k);
@@ -419,27 +408,27 @@ struct ArgsGrad {
 // Arguments of the three-index kernels (by value).
 struct Args3c {
     const ShellRec *orb_shells, *aux_shells;
-    const PrimRec *orb_prims, *aux_prims;
+    const XPrim *orb_prims, *aux_prims;
     const Vec4 *orb_centers, *aux_centers;
     const int32_t *t_a, *t_t, *t_b;
     const int32_t *perm;
-    const Tile *tiles;
-    int tile_begin, tile_end;
+    const Tile *tiles;            // kGroupOf[0] lanes per triple
+    int tile_end;
+    int slot_doubles;             // shared memory of a triple: the largest of the list's classes
     int *counter;
     const long long *out_off;
     double *out;
-    const int *gaunt_base, *gaunt_row;
-    const GauntEnt *gaunt;
-    // gradient kernels only (grad_a != null selects the VJP kernel)
+    // gradient kernel
     const long long *w_off;
     const double *w;
     double *grad_a, *grad_b;
     // screening: > 0 writes zeros for a triple whose bound on every element is below it
     double screen_thresh;
     const ScreenRec *orb_screen, *aux_screen;
+    const uint64_t *exptab;
+    CGTab cg;
     Consts k;
     Consts3 k3;
-    ConstsMix km;                 // mixed-precision angular part
 };
 
 // Kernel launchers (shg_kernels.cu, shg_3c.cu).
@@ -454,15 +443,19 @@ constexpr size_t plan_ws_ints(int64_t n, int n_bins, int n_chunks)
     return 4 + 4 * (size_t)n_bins + 1 + 2 * (size_t)n_chunks + 2 + (size_t)n;
 }
 // largest number of tiles of n entries: every chunk ends in at most one partial tile per group size
-constexpr int64_t plan_max_tiles(int64_t n, int n_chunks, bool grouped)
+constexpr int64_t plan_max_tiles(int64_t n, int n_chunks)
 {
-    return n * (grouped ? kGroupOf[0] : 1) / kTile + kNGroups * n_chunks + 1;
+    return n * kGroupOf[0] / kTile + kNGroups * n_chunks + 1;
 }
 // chunk -> first tile, tile count and error flag (n_chunks + 2 ints of the summary) and the tile map of a two-center plan
 int plan_read(PlanDev &d, const int *summary, int schedule);
 inline int *plan_summary(int *ws, int n_bins) { return ws + 4 + 4 * (size_t)n_bins + 1; }
 cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d_bin_rank, cudaStream_t s);
-cudaError_t launch_3c(const Args3c &args, int precision, int grid, cudaStream_t s);
+cudaError_t launch_3c(const Args3c &args, cudaStream_t s);
+cudaError_t launch_3c_grad(const Args3c &args, cudaStream_t s);
+// doubles of shared memory that a triple of a class takes
+int slot_doubles_3c(int cls);
+int slot_doubles_3c_grad(int cls);
 // vector-Jacobian products (persistent when the counter is set, else one warp per tile): FP64, mixed precision, and
 // (a|r_a^{2n}|b) (32-pair tiles of the map)
 cudaError_t launch_2c_grad(const ArgsGrad &args, cudaStream_t s, int threads);
@@ -470,7 +463,6 @@ cudaError_t launch_2c_grad_mixed(const ArgsGrad &args, cudaStream_t s, int threa
 cudaError_t launch_2c_grad_ra2n(const Args2c &args, cudaStream_t s);
 // mixed-precision pass of the classes with min(la, lb) < kMixedFp64MinL (arguments as launch_2c_fused)
 cudaError_t launch_2c_mixed(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
-int persistent_grid_3c(int precision);
 cudaError_t launch_2c(const Args2c &args, int op, int precision, int n_tiles_or_grid, bool persistent,
                       cudaStream_t s, int threads = 128);
 int persistent_grid_2c(int op, int precision, int threads = 128, int ctas_per_sm = 0);

@@ -632,12 +632,12 @@ cudaError_t launch_plan_build(PlanDev &plan, int *d_ws, int n_bins, const int *d
                                                  d_bin_rank, key, hist, d_err);
     }
     // both rank orders are class-major (each class a chunk of bins_per_class ranks): one tiling per class
-    // rank r of a two-center chunk holds Ka*Kb = kKbins2c - r; triples have one lane each
+    // rank r of a two-center chunk holds Ka*Kb = kKbins2c - r; triples have eight lanes each
     GroupRanges gr{};
-    for (int i = 0; i < kNGroups; ++i) gr.end[i] = plan.kind == 2 ? bpc - kGroupMinK[i] + 1 : (i + 1 < kNGroups ? 0 : bpc);
+    for (int i = 0; i < kNGroups; ++i) gr.end[i] = plan.kind == 2 ? bpc - kGroupMinK[i] + 1 : bpc;
     k_scan_chunks<<<n_chunks, bpc, 0, s>>>(n_bins, bpc, gr, hist, bin_start, cursor, tile_start, ticket, summary, d_err);
     if (n > 0) k_scatter<<<blocks, threads, 0, s>>>(n, bpc, key, bin_start, cursor, plan.perm);
-    const int64_t max_tiles = plan_max_tiles(n, n_chunks, plan.kind == 2);
+    const int64_t max_tiles = plan_max_tiles(n, n_chunks);
     const int tb = (int)((max_tiles + 255) / 256 < 1024 ? (max_tiles + 255) / 256 : 1024);
     k_make_tiles<<<tb, 256, 0, s>>>(n_chunks, bpc, bpc, (int)n, bin_start, tile_start, d_bin_rank + n_bins,
                                     plan.tiles);

@@ -32,7 +32,7 @@ namespace {
 
 constexpr int64_t kNoAllocMaxPairs = int64_t(1) << 20;
 // layout: tiles | perm | counter, err | key | hist | bin_start | cursor | tile_start
-constexpr int64_t kNoAllocMaxTiles = plan_max_tiles(kNoAllocMaxPairs, kNClass, true);
+constexpr int64_t kNoAllocMaxTiles = plan_max_tiles(kNoAllocMaxPairs, kNClass);
 constexpr size_t kTilesBytes = ((size_t)kNoAllocMaxTiles * sizeof(Tile) + 255) / 256 * 256;
 constexpr size_t kPermBytes = ((size_t)kNoAllocMaxPairs * sizeof(int32_t) + 255) / 256 * 256;
 constexpr size_t kFlagsBytes = 256;
