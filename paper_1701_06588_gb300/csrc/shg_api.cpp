@@ -152,38 +152,6 @@ void fill_consts(Consts &k)
         }
 }
 
-// Boys tables, computed in long double: F_N(T) from its power series
-//   F_N(T) = exp(-T) sum_k (2T)^k / ((2N+1)(2N+3)...(2N+2k+1))
-// at N = 48, then the stable downward recursion
-//   F_{n-1}(T) = (2T F_n(T) + exp(-T)) / (2n-1);
-// at T_i = i / per_unit, i = 0..ngrid-1: tab[(i kBoysN + n) nterms + t] =
-// F_{n+t}(T_i) / t!, etab[i] = exp(-T_i).
-void make_boys_table(int per_unit, int ngrid, int nterms, double *tab, double *etab)
-{
-    const int ntop = 48;
-    for (int i = 0; i < ngrid; ++i) {
-        const long double T = (long double)i / (long double)per_unit;
-        const long double e = std::exp(-T);
-        long double term = 1.0L / (2 * ntop + 1), sum = term;
-        for (int k = 1; k < 20000; ++k) {
-            term *= 2 * T / (long double)(2 * ntop + 2 * k + 1);
-            sum += term;
-            if (term < sum * 1e-24L) break;
-        }
-        long double F[ntop + 1];
-        F[ntop] = e * sum;
-        for (int n = ntop; n > 0; --n) F[n - 1] = (2 * T * F[n] + e) / (long double)(2 * n - 1);
-        for (int n = 0; n < kBoysN; ++n) {
-            long double tf = 1;
-            for (int t = 0; t < nterms; ++t) {
-                if (t > 0) tf *= t;
-                tab[((size_t)i * kBoysN + n) * nterms + t] = (double)(F[n + t] / tf);
-            }
-        }
-        etab[i] = (double)e;
-    }
-}
-
 // Extended floats from host values: FP64 (also denormal) and double-double, > 0
 static xfp::xf xf_of(dd v)
 {
@@ -265,37 +233,6 @@ static inline float2 split2d(double v)
 {
     const float hi = (float)v;
     return make_float2(hi, (float)(v - (double)hi));
-}
-
-void fill_consts_mix(ConstsMix &k)
-{
-    std::memset(&k, 0, sizeof k);
-    for (int l = 0; l <= kLmaxR; ++l)
-        for (int mu = 0; mu <= l; ++mu) {
-            long double v = std::sqrt((long double)(mu == 0 ? 1 : 2) * lfact(l + mu) * lfact(l - mu));
-            k.A[l][mu] = split2((mu & 1) ? -v : v);
-        }
-    for (int j = 0; j < kJmax; ++j) {
-        long double df = 1;
-        for (int i = 2 * j - 1; i > 1; i -= 2) df *= i;
-        for (int kp = 0; kp <= j; ++kp) k.jB[j][kp] = split2(df / ((kp == 0 ? 1 : 2) * lfact(j + kp) * lfact(j - kp)));
-    }
-    for (int i = 1; i < 128; ++i) k.inv_int[i] = split2(1.0L / i);
-    for (int t = 0; t < 14; ++t) {
-        k.inv_fact[t] = split2(1.0L / lfact(t));
-        k.inv_fact_f[t] = (float)(1.0L / lfact(t));
-    }
-    const long double pi = 3.14159265358979323846264338327950288L;
-    k.pi32 = split2(std::pow(pi, 1.5L));
-    k.pi3 = split2(pi * pi * pi);
-    k.two_pi52 = split2(2 * std::pow(pi, 2.5L));
-    k.sqrt_pi_half = split2(std::sqrt(pi) / 2);
-    k.two_pi = split2(2 * pi);
-    long double dfc = 1;
-    for (int n = 0; n < kBoysN; ++n) {
-        k.dfact[n] = split2(dfc);
-        dfc *= (2 * n + 1);
-    }
 }
 
 void fill_consts3(Consts3 &k)
@@ -498,49 +435,9 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
     std::lock_guard<std::mutex> lk(g_mu);
     DevState &st = g_dev[dev];
     if (!st.ready) {
-        // FP64 table (step 1/32): c0..c3 as doubles, c4..c6 as floats
-        std::vector<double> raw((size_t)kBoysGrid * kBoysN * 7), etab(kBoysGrid);
-        make_boys_table(32, kBoysGrid, 7, raw.data(), etab.data());
-        std::vector<double> tab((size_t)kBoysGrid * kBoysN * kBoysStride, 0.0);
-        for (size_t q = 0; q < (size_t)kBoysGrid * kBoysN; ++q) {
-            double *d = &tab[q * kBoysStride];
-            const double *r = &raw[q * 7];
-            for (int t = 0; t < 4; ++t) d[t] = r[t];
-            const float f[4] = {(float)r[4], (float)r[5], (float)r[6], 0.0f};
-            std::memcpy(d + 4, f, sizeof f);
-        }
-        // double-float table (the same grid): c0..c2 as hi/lo float pairs, c3..c6 as floats
-        std::vector<float4> mtab((size_t)kBoysGrid * kBoysN * 3);
-        std::vector<float2> metab(kBoysGrid);
-        for (int i = 0; i < kBoysGrid; ++i) {
-            for (int n = 0; n < kBoysN; ++n) {
-                const double *cf = &raw[((size_t)i * kBoysN + n) * 7];
-                float4 *q = &mtab[((size_t)i * kBoysN + n) * 3];
-                const float2 c0 = split2(cf[0]), c1 = split2(cf[1]), c2 = split2(cf[2]);
-                q[0] = make_float4(c0.x, c0.y, c1.x, c1.y);
-                q[1] = make_float4(c2.x, c2.y, (float)cf[3], (float)cf[4]);
-                q[2] = make_float4((float)cf[5], (float)cf[6], 0.0f, 0.0f);
-            }
-            metab[i] = split2(etab[i]);
-        }
-        double *d_tab = nullptr, *d_e = nullptr;
-        float4 *d_mtab = nullptr;
-        float2 *d_metab = nullptr;
         int *d_r[2] = {nullptr, nullptr};
-        if (cudaMalloc(&d_tab, tab.size() * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&d_e, etab.size() * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&d_r[0], 2 * kNBins * sizeof(int)) != cudaSuccess ||
-            cudaMalloc(&d_r[1], 2 * kNBins * sizeof(int)) != cudaSuccess) {
-            cudaFree(d_tab); cudaFree(d_e); cudaFree(d_r[0]); cudaFree(d_r[1]);
-            fail(SHG_ENOMEM, "device tables: cudaMalloc failed");
-            return nullptr;
-        }
-        bool ok = cudaMemcpy(d_tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
-                  cudaMemcpy(d_e, etab.data(), etab.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
-                  cudaMalloc(&d_mtab, mtab.size() * sizeof(float4)) == cudaSuccess &&
-                  cudaMalloc(&d_metab, metab.size() * sizeof(float2)) == cudaSuccess &&
-                  cudaMemcpy(d_mtab, mtab.data(), mtab.size() * sizeof(float4), cudaMemcpyHostToDevice) == cudaSuccess &&
-                  cudaMemcpy(d_metab, metab.data(), metab.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
+        bool ok = cudaMalloc(&d_r[0], 2 * kNBins * sizeof(int)) == cudaSuccess &&
+                  cudaMalloc(&d_r[1], 2 * kNBins * sizeof(int)) == cudaSuccess;
         for (int s = 0; s < 2 && ok; ++s) {
             std::vector<int> rank, inv;
             make_ranks(s, rank, inv);
@@ -611,10 +508,6 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
         st.bin_rank3 = d_r3;
         st.t.cg = CGTab{d_cg, d_cgb, d_fc, d_cgm, d_ch};
         st.t.x = XTab{d_bc, d_ex};
-        st.t.boys_mix = d_mtab;
-        st.t.boys_e_mix = d_metab;
-        st.t.boys = d_tab;
-        st.t.boys_e = d_e;
         st.bin_rank[0] = d_r[0];
         st.bin_rank[1] = d_r[1];
         st.ready = true;
@@ -641,14 +534,6 @@ const DeviceTables *device_tables_if_ready(const int **ranks)
         ranks[1] = st.bin_rank[1];
     }
     return &st.t;
-}
-
-const ConstsMix &consts_mix()
-{
-    static ConstsMix k;
-    static std::once_flag once;
-    std::call_once(once, [] { fill_consts_mix(k); });
-    return k;
 }
 
 const Consts3 &consts3()
@@ -741,7 +626,6 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
 
     std::vector<ShellRec> sh(n_shells);
     std::vector<PrimRec> pr(n_prims);
-    std::vector<CoulPrim> cpr(n_prims);
     std::vector<XPrim> xpr(n_prims);
     std::vector<int64_t> first(n_shells + 1, 0);
     for (int s = 0; s < n_shells; ++s) first[s + 1] = first[s] + nprim[s];
@@ -752,6 +636,8 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
         pref_l[L] = dd_from(std::sqrt(pi) * lfact(2 * L + 2) / (std::ldexp(1.0L, 2 * L + 3) * lfact(L + 1)));
         K_l[L] = dd_from(std::sqrt((2 * L + 1) / (4 * pi)));
     }
+    // sqrt(2 pi^{5/2}) folded into cw: pre = cw_a cw_b / sqrt(c)
+    const dd s2p52 = dd_sqrt(dd_from(2.0L * 17.493418327624862846262821679871554L));
     int bad_shell = -1;
 #pragma omp parallel for schedule(dynamic, 256)
     for (int s = 0; s < n_shells; ++s) {
@@ -794,17 +680,14 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
             p.wN = c.hi;
             pr[off + i] = p;
             const dd cw = dd_mul(w2c, ia);
-            // sqrt(2 pi^{5/2}) folded into cw: pre = cw_a cw_b / sqrt(c)
-            const dd s2p52 = dd_sqrt(dd_from(2.0L * 17.493418327624862846262821679871554L));   // 2 pi^{5/2}
             const dd cws = dd_mul(cw, s2p52);
-            cpr[off + i] = CoulPrim{cws.hi, dd_mul(cw, dd_sqrt(ia)).hi};
             const xfp::xf xa = xf_of(dd{a, 0.0});
             // a zero weight: a value so small that every term it enters is flushed to 0 (and one that overflowed FP64
             // gives infinities)
             const xfp::xf xw = cws.hi == 0 || !std::isfinite(cws.hi)
                                        ? xfp::xf{1ull << 62, cws.hi == 0 ? -1000000 : 1000000}
                                        : xf_of(cws.hi < 0 ? dd{-cws.hi, -cws.lo} : cws);
-            xpr[off + i] = XPrim{xa.m, xw.m | (cws.hi < 0 ? 1ull << 63 : 0), xa.e, xw.e, cpr[off + i].fw};
+            xpr[off + i] = XPrim{xa.m, xw.m | (cws.hi < 0 ? 1ull << 63 : 0), xa.e, xw.e, dd_mul(cw, dd_sqrt(ia)).hi};
         }
         sh[s] = ShellRec{L, K, (int)off, center_of_shell[s]};
     }
@@ -838,21 +721,7 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
         scr[s] = ScreenRec{amin, sabs, lfac, 0.0};
     }
     std::vector<Vec4> ctr(n_centers);
-    std::vector<MixCenter> mctr(n_centers);
-    for (int c = 0; c < n_centers; ++c) {
-        ctr[c] = Vec4{centers[3 * c], centers[3 * c + 1], centers[3 * c + 2], 0.0};
-        mctr[c] = MixCenter{split2d(centers[3 * c]), split2d(centers[3 * c + 1]), split2d(centers[3 * c + 2]),
-                            make_float2(0, 0)};
-    }
-    std::vector<MixPrim> mpr(n_prims);
-#pragma omp parallel for schedule(static)
-    for (int64_t o = 0; o < n_prims; ++o) {
-        const double a = exps[o];
-        const dd ia = dd_div(dd{1.0, 0.0}, dd{a, 0.0});
-        const float ih = (float)ia.hi;
-        mpr[o] = MixPrim{split2d(a), make_float2(ih, (float)((ia.hi - (double)ih) + ia.lo)), split2d(pr[o].wN),
-                         cpr[o].fw};
-    }
+    for (int c = 0; c < n_centers; ++c) ctr[c] = Vec4{centers[3 * c], centers[3 * c + 1], centers[3 * c + 2], 0.0};
 
     shg_basis_t *b = new (std::nothrow) shg_basis_t;
     if (!b) return fail(SHG_ENOMEM, "host allocation failed");
@@ -877,22 +746,16 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
     if (cudaMalloc(&d.shells, sizeof(ShellRec) * n_shells) != cudaSuccess ||
         cudaMalloc(&d.prims, sizeof(PrimRec) * n_prims) != cudaSuccess ||
         cudaMalloc(&d.centers, sizeof(Vec4) * n_centers) != cudaSuccess ||
-        cudaMalloc(&d.mprims, sizeof(MixPrim) * n_prims) != cudaSuccess ||
-        cudaMalloc(&d.cprims, sizeof(CoulPrim) * n_prims) != cudaSuccess ||
         cudaMalloc(&d.xprims, sizeof(XPrim) * n_prims) != cudaSuccess ||
-        cudaMalloc(&d.screen, sizeof(ScreenRec) * n_shells) != cudaSuccess ||
-        cudaMalloc(&d.mcenters, sizeof(MixCenter) * n_centers) != cudaSuccess) {
+        cudaMalloc(&d.screen, sizeof(ScreenRec) * n_shells) != cudaSuccess) {
         shg_basis_destroy(b);
         return fail(SHG_ENOMEM, "basis: cudaMalloc failed");
     }
     if (cudaMemcpy(d.shells, sh.data(), sizeof(ShellRec) * n_shells, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.prims, pr.data(), sizeof(PrimRec) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.centers, ctr.data(), sizeof(Vec4) * n_centers, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(d.mprims, mpr.data(), sizeof(MixPrim) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(d.cprims, cpr.data(), sizeof(CoulPrim) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d.xprims, xpr.data(), sizeof(XPrim) * n_prims, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(d.screen, scr.data(), sizeof(ScreenRec) * n_shells, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(d.mcenters, mctr.data(), sizeof(MixCenter) * n_centers, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaMemcpy(d.screen, scr.data(), sizeof(ScreenRec) * n_shells, cudaMemcpyHostToDevice) != cudaSuccess) {
         shg_basis_destroy(b);
         return fail(SHG_ECUDA, "basis: upload failed");
     }
@@ -915,15 +778,12 @@ int shg_basis_set_centers(shg_basis_t *b, const double *centers)
     if (!d.stage_raw) {
         if (cudaMalloc(&d.stage_raw, sizeof(double) * 3 * n) != cudaSuccess ||
             cudaMalloc(&d.stage_ctr, sizeof(Vec4) * n) != cudaSuccess ||
-            cudaMalloc(&d.stage_mctr, sizeof(MixCenter) * n) != cudaSuccess ||
             cudaMalloc(&d.stage_bad, sizeof(int)) != cudaSuccess) {
             cudaFree(d.stage_raw);
             cudaFree(d.stage_ctr);
-            cudaFree(d.stage_mctr);
             cudaFree(d.stage_bad);
             d.stage_raw = nullptr;
             d.stage_ctr = nullptr;
-            d.stage_mctr = nullptr;
             d.stage_bad = nullptr;
             return fail(SHG_ENOMEM, "set_centers: cudaMalloc failed");
         }
@@ -932,13 +792,12 @@ int shg_basis_set_centers(shg_basis_t *b, const double *centers)
     const cudaStream_t s = 0;
     SHG_CUDA(cudaMemcpyAsync(d.stage_raw, centers, sizeof(double) * 3 * n, cudaMemcpyHostToDevice, s));
     SHG_CUDA(cudaMemsetAsync(d.stage_bad, 0x7f, sizeof(int), s));
-    SHG_CUDA(launch_pack_centers(d.stage_raw, n, d.stage_ctr, d.stage_mctr, d.stage_bad, s));
+    SHG_CUDA(launch_pack_centers(d.stage_raw, n, d.stage_ctr, d.stage_bad, s));
     int bad = 0;
     SHG_CUDA(cudaMemcpyAsync(&bad, d.stage_bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     SHG_CUDA(cudaStreamSynchronize(s));
     if (bad < n) return fail(SHG_EINVAL, "center %d has a non-finite coordinate", bad);
     SHG_CUDA(cudaMemcpyAsync(d.centers, d.stage_ctr, sizeof(Vec4) * n, cudaMemcpyDeviceToDevice, s));
-    SHG_CUDA(cudaMemcpyAsync(d.mcenters, d.stage_mctr, sizeof(MixCenter) * n, cudaMemcpyDeviceToDevice, s));
     SHG_CUDA(cudaStreamSynchronize(s));
     return SHG_OK;
 }
@@ -949,14 +808,10 @@ void shg_basis_destroy(shg_basis_t *b)
     cudaFree(b->d.shells);
     cudaFree(b->d.prims);
     cudaFree(b->d.centers);
-    cudaFree(b->d.mprims);
-    cudaFree(b->d.cprims);
     cudaFree(b->d.xprims);
-    cudaFree(b->d.mcenters);
     cudaFree(b->d.screen);
     cudaFree(b->d.stage_raw);
     cudaFree(b->d.stage_ctr);
-    cudaFree(b->d.stage_mctr);
     cudaFree(b->d.stage_bad);
     delete[] b->d.h_l;
     delete[] b->d.h_nprim;
@@ -1375,8 +1230,6 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     a.out_off = reinterpret_cast<const long long *>(off);
     a.out = out;
     a.omega = omega;
-    a.boys = t->boys;
-    a.boys_e = t->boys_e;
     a.o_pre = o_pre;
     a.cg = t->cg;
     a.k = consts();
@@ -1884,6 +1737,7 @@ int shg_family_plan_exec(shg_family_plan_t *fp, int op, double omega, const int6
         ArgsFam a;
         a.shells = fp->basis->shells;
         a.prims = fp->basis->prims;
+        a.xprims = fp->basis->xprims;
         a.centers = fp->basis->centers;
         a.pair_a = fp->d_pa_fam;
         a.pair_b = fp->d_pb_fam;
@@ -1891,9 +1745,8 @@ int shg_family_plan_exec(shg_family_plan_t *fp, int op, double omega, const int6
         a.n_groups = fp->n_groups;
         a.counter = fp->d_counter;
         a.o_pre = fp->d_o;
-        a.omega = omega;
-        a.boys = t->boys;
-        a.boys_e = t->boys_e;
+        a.omega = x_omega(omega);
+        a.t = t->x;
         a.k = consts();
         SHG_CUDA(cudaMemsetAsync(fp->d_counter, 0, sizeof(int), s));
         SHG_CUDA(launch_family_radial(a, op, s));
@@ -1950,7 +1803,7 @@ int shg_reduce_centers(const shg_basis_t *b, int64_t n, const int32_t *pa, const
 int shg_debug_boys(int64_t n, const double *T, int nmax, double *F, void *stream)
 {
     g_err.clear();
-    if (n < 0 || nmax < 0 || nmax >= kBoysN) return fail(SHG_EINVAL, "bad n or nmax (nmax <= %d)", kBoysN - 1);
+    if (n < 0 || nmax < 0 || nmax >= kBoysOrders) return fail(SHG_EINVAL, "bad n or nmax (nmax <= %d)", kBoysOrders - 1);
     if (n == 0) return SHG_OK;
     if (!T || !F) return fail(SHG_EINVAL, "NULL pointer");
     const DeviceTables *t = device_tables();

@@ -10,75 +10,90 @@
 // group: G in shared memory, lanes over primitive pairs, then over (shell
 // pair, order) items.  The angular part follows in the class-tiled kernel
 // (OP_PRE).
-#include "shg_device.cuh"
+#include "shg_xradial.cuh"
 
 namespace shg {
 namespace {
 using namespace dev;
+using namespace xfp;
 
 constexpr int kFamWarps = 4;
 
-// Unit-weight radial terms G[k] = (0_a|O|0_b)^{(k)}, k = 0..kmax, of one primitive pair.
-template <int OP>
-__device__ __forceinline__ void radial_all(double alpha, double beta, double inv_a, double inv_b, double R2, int kmax,
-                                           const ArgsFam &g, double *G)
+// X_n = P q^n F_n(T), n = kmin..kmax, into G[n - kmin] (added, with the sign of (-1)^n times `sign`): the top order from the
+// Boys head, the others by X_n = (-2R^2 X_{n+1} + P q^n exp(-T)) / (2n+1) (2T/q = -2R^2)
+__device__ __forceinline__ void boys_orders(const ArgsFam &g, xf pre, xf q, xf T, double R2, int kmin, int kmax,
+                                            uint32_t sign, double *G)
 {
-    const double c = alpha + beta;
-    const double rc = rsqrt(c);
-    const double ic = rc * rc;
-    const double rho = alpha * beta * ic;
-    const double T = rho * R2;
-    if (OP == OP_OVERLAP) {
-        double q = kPi32 * ic * rc * exp(-T);
+    xf F, e;
+    xrad::boys_any(T, kmax, g.t, g.k.dfact[kmax], kmax > kmin, F, e);
+    xf t = pre;
+    if (kmin) t = mul(t, xfp::powi(q, kmin));
+    double E[kFamOrd];
+    for (int n = kmin; n < kmax; ++n) {
+        E[n - kmin] = to_double(mul(t, e), xrad::order_sign(sign, n));
+        t = mul(t, q);
+    }
+    double x = to_double(mul(t, F), xrad::order_sign(sign, kmax));
+    G[kmax - kmin] += x;
+    const double m2R2 = -2.0 * R2;
+    for (int n = kmax - 1; n >= kmin; --n) {
+        x = fma(m2R2, x, E[n - kmin]) * g.k.inv_int[2 * n + 1];
+        G[n - kmin] += x;
+    }
+}
+
+// Unit-weight radial terms G[k - kmin] = (0_a|O|0_b)^{(k)}, k = kmin..kmax, of one primitive pair, in extended floats up
+// to the recursion (as shg_xradial.cuh; the FP64 form took 0.27 of the 0.53 ms of a 300-atom pass)
+template <int OP>
+__device__ __forceinline__ void radial_all(xf a, xf b, double R2, int kmin, int kmax, const ArgsFam &g, double *G)
+{
+    const xf rc = xfp::rsqrt(add(a, b)), ic = mul(rc, rc), ab = mulr(a, b);
+    const xf rho = muln(ab, ic);
+    const xf T = mul(rho, from_double(R2));
+    if (OP == OP_OVERLAP || OP == OP_GAUSS) {
+        xf t = mul(ic, rc), f = rho;
+        double c = kPi32;
+        if (OP == OP_OVERLAP) {
+            t = mul(t, xrad::exp_neg(T, g.t.exp));
+        } else {
+            const xf w = {g.omega.w_m, g.omega.w_e};
+            const xf rd = xfp::rsqrt(add(rho, w)), id = mul(rd, rd), wd = mul(w, id);
+            f = mul(rho, wd);
+            t = mul(mul(t, mul(id, rd)), xrad::exp_neg(mul(T, wd), g.t.exp));
+            c = kPi3;
+        }
+        if (kmin) t = mul(t, xfp::powi(f, kmin));
+        for (int k = kmin; k <= kmax; ++k) {
+            G[k - kmin] = c * to_double(t, xrad::order_sign(0, k));
+            t = mul(t, f);
+        }
+        return;
+    }
+    if (OP == OP_GCOUL) {
+        // (pi/c)^{3/2} (2 pi/d) exp(-w T/d) (-rho)^k sum_i C(k,i) (w/d)^{k-i} (rho/d)^i F_i(T rho/d)
+        const xf w = {g.omega.w_m, g.omega.w_e};
+        const xf rd = xfp::rsqrt(add(rho, w)), id = mul(rd, rd), sw = mul(w, id), sr = mul(rho, id);
+        xf T2 = mul(T, sr), F[kBoysOrders], e;
+        xrad::boys_any(T2, kmax, g.t, g.k.dfact[kmax], true, F[kmax], e);
+        T2.e += 1;
+        for (int n = kmax; n > 0; --n) F[n - 1] = mul(add(mul(T2, F[n]), e), from_double(g.k.inv_int[2 * n - 1]));
+        xf pre = mul(mul(mul(ic, rc), id), xrad::exp_neg(mul(T, sw), g.t.exp));
         for (int k = 0; k <= kmax; ++k) {
-            G[k] = q;
-            q *= -rho;
+            if (k >= kmin) G[k - kmin] = kTwoPi52 * to_double(mul(pre, F[0]), xrad::order_sign(0, k));
+            for (int i = 0; i < kmax - k; ++i) F[i] = add(mul(sw, F[i]), mul(sr, F[i + 1]));
+            pre = mul(pre, rho);
         }
-    } else if (OP == OP_GAUSS) {
-        const double rd = rsqrt(rho + g.omega);
-        const double id = rd * rd;
-        const double f = -g.omega * rho * id;
-        double q = kPi3 * ic * rc * id * rd * exp(-g.omega * T * id);
-        for (int k = 0; k <= kmax; ++k) {
-            G[k] = q;
-            q *= f;
-        }
-    } else if (OP == OP_GCOUL) {
-        const double id = 1.0 / (rho + g.omega);
-        const double p = -g.omega * rho * id, q = -rho * rho * id;
-        const double pre = kPi32 * ic * rc * (2.0 * kPi) * id * exp(-g.omega * T * id);
-        double F[kBoysN];
-        boys_all(T * rho * id, kmax, g.boys, g.boys_e, g.k, F);
-        G[0] = pre * F[0];
-        for (int m = 1; m <= kmax; ++m) {
-            for (int i = 0; i <= kmax - m; ++i) F[i] = fma(p, F[i], q * F[i + 1]);
-            G[m] = pre * F[0];
-        }
-    } else {
-        const double pre = kTwoPi52 * inv_a * inv_b * rc;
-        for (int k = 0; k <= kmax; ++k) G[k] = 0.0;
-        double F[kBoysN];
-        if (OP == OP_COULOMB || OP == OP_ERFC) {
-            boys_all(T, kmax, g.boys, g.boys_e, g.k, F);
-            double q = pre;
-            for (int k = 0; k <= kmax; ++k) {
-                G[k] = q * F[k];
-                q *= -rho;
-            }
-        }
-        if (OP == OP_ERF || OP == OP_ERFC) {
-            const double w2 = g.omega * g.omega;
-            const double rw = rsqrt(w2 + rho);
-            const double s = w2 * rw * rw;
-            const double f = -rho * s;
-            boys_all(s * T, kmax, g.boys, g.boys_e, g.k, F);
-            double q = pre * g.omega * rw;
-            if (OP == OP_ERFC) q = -q;
-            for (int k = 0; k <= kmax; ++k) {
-                G[k] += q * F[k];
-                q *= f;
-            }
-        }
+        return;
+    }
+    // 2 pi^{5/2} / (alpha beta sqrt(c)): 1 / (alpha beta) = 1 / (c rho)
+    const xf rr = xfp::rsqrt(rho);
+    const xf pre = mul(mul(mul(rr, rr), mul(ic, rc)), from_double(kTwoPi52));
+    for (int k = kmin; k <= kmax; ++k) G[k - kmin] = 0.0;
+    if (OP == OP_COULOMB || OP == OP_ERFC) boys_orders(g, pre, rho, T, R2, kmin, kmax, 0, G);
+    if (OP == OP_ERF || OP == OP_ERFC) {
+        const xf w = {g.omega.w_m, g.omega.w_e}, w2 = {g.omega.w2_m, g.omega.w2_e};
+        const xf u = mul(w, xfp::rsqrt(add(rho, w2))), s = mul(u, u);
+        boys_orders(g, mul(pre, u), mul(rho, s), mul(s, T), R2, kmin, kmax, OP == OP_ERFC ? 0x80000000u : 0u, G);
     }
 }
 
@@ -101,10 +116,10 @@ __global__ void __launch_bounds__(32 * kFamWarps) k_family_radial(const ArgsFam 
         const int npp = gr.fa_k * gr.fb_k;
         for (int ij = lane; ij < npp; ij += 32) {
             const int i = ij / gr.fb_k, j = ij - i * gr.fb_k;
-            const PrimRec pa = g.prims[gr.fa_prim + i], pb = g.prims[gr.fb_prim + j];
+            const XPrim pa = g.xprims[gr.fa_prim + i], pb = g.xprims[gr.fb_prim + j];
             double G[kFamOrd];
-            radial_all<OP>(pa.alpha, pb.alpha, pa.inv_alpha, pb.inv_alpha, R2, gr.kmax, g, G);
-            for (int k = gr.kmin; k <= gr.kmax; ++k) gs[(k - gr.kmin) * kFamPP + ij] = G[k];
+            radial_all<OP>(xf{pa.am, pa.ae}, xf{pb.am, pb.ae}, R2, gr.kmin, gr.kmax, g, G);
+            for (int k = gr.kmin; k <= gr.kmax; ++k) gs[(k - gr.kmin) * kFamPP + ij] = G[k - gr.kmin];
         }
         __syncwarp();
         // contraction: lanes over (shell pair, order) items, 32 shell pairs at a

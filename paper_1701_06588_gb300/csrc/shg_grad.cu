@@ -24,13 +24,13 @@ __device__ void pair_grad_ra2n(const Args2c &g, int p)
     const Vec4 B = g.centers[sb.center];
     const double v[3] = {A.x - B.x, A.y - B.y, A.z - B.z};
     const double R2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    double Q[J + 1], E[J + 1];
+    double Q[J + 1];
 #pragma unroll
-    for (int j = 0; j <= J; ++j) Q[j] = E[j] = 0.0;
+    for (int j = 0; j <= J; ++j) Q[j] = 0.0;
     const int Kb = sb.nprim, npp = sa.nprim * Kb;
     for (int q = 0; q < npp; ++q) {
         const int ia = q / Kb, ib = q - ia * Kb;
-        radial_acc_fp64<OP_RA2N, J + 1>(g.prims[sa.prim_off + ia], g.prims[sb.prim_off + ib], R2, la + lb + 1, la, g, Q, E);
+        radial_acc_ra2n<J + 1>(g.prims[sa.prim_off + ia], g.prims[sb.prim_off + ib], R2, la + lb + 1, la, g, Q);
     }
     double G[3];
     vjp_d<J>(g.cg, g.k, la, lb, v, R2, Q, 0.0, 0.0, g.w + g.w_off[p], 0, 1, G);

@@ -17,34 +17,19 @@ constexpr int kRa2nMax = 5;                // largest n of the (a|r_a^{2n}|b) op
 constexpr int kNClass = (kLmax2c + 1) * (kLmax2c + 1);
 constexpr int kTile = 32;         // pairs per warp tile
 // Two-center classes that the mixed-precision passes evaluate in FP64: both
-// la and lb >= kMixedFp64MinL (J = min(la, lb) + 1 >= 5).  There the sum over
-// j of Eq. final_r12int_ab cancels by up to ~1e4 (l = 6, exponents to 5000),
-// beyond what double-float (2^-44 of the largest term) carries to 1e-10.
+// la and lb >= kMixedFp64MinL (J = min(la, lb) + 1 >= 5), where the angular sums
+// cancel most (double-float carries 2^-44 of the largest term).
 constexpr int kMixedFp64MinL = 4;
 inline bool mixed_runs_fp64(int cls) { return cls / 7 >= kMixedFp64MinL && cls % 7 >= kMixedFp64MinL; }
-
-// Boys tables: Taylor coefficients c_t = F_{n+t}(T_i)/t!, t = 0..6, about the
-// grid points T_i = i/32, i = 0..kBoysGrid-1 (|delta| <= 1/64), n < kBoysN;
-// Taylor expansion about the nearest grid point.
-//   FP64 table: per (i, n) kBoysStride doubles: c0..c3 as doubles, c4..c6 as
-//     floats (and one float of padding), 48 bytes.
-//   double-float table: per (i, n) three float4: c0..c2 as hi/lo float pairs,
-//     c3..c6 as floats (and two floats of padding), 48 bytes.
-// Above kBoysTmax, F_n(T) = (2n-1)!! / (2T)^n sqrt(pi/(4T)) to better than
-// 1e-30 relative for n <= 16 (the neglected terms carry exp(-T)).
-constexpr int kBoysGrid = 3841;     // covers T < 120 at step 1/32
-constexpr int kBoysStride = 6;
-constexpr double kBoysTmax = 120.0;
-constexpr int kBoysN = 16;          // orders n = 0..15 from the tables
 
 // Boys function for the extended-float radial sums: from T = kFarT on the asymptotic form (relative error below 5e-18
 // for n <= 13: T^{n-1/2} e^{-T} / Gamma(n+1/2)); below, per order n = 0..kBoysOrders-1 and cell [i, i+1) / 512 of T, the Taylor coefficients c_t = F_{n+t}(T_{i+1}) / t! about the upper end of the cell, scaled by
 // 2^s so that c0 < 2^63 (1 - 2^-8): c0, c1 in units 2^-s, c2 likewise with s - 62 in its low 8 bits, c3 in units
 // 2^{30-s}, c4 (24 bits) in units 2^{35-s}, c5 (8 bits) in units 2^{49-s}.  y = T_{i+1} - T <= 2^-9, so the dropped
-// y^6/720 is below 2^-63.  One 32-byte load per evaluation; 16.5 MB, resident in L2.
+// y^6/720 is below 2^-63.  One 32-byte load per evaluation; 18.9 MB, resident in L2.
 constexpr int kFarT = 72;
 constexpr int kBoysCells = kFarT * 512;
-constexpr int kBoysOrders = 14;
+constexpr int kBoysOrders = 16;
 struct alignas(32) BoysEnt {
     uint64_t c0, c1, c2;
     uint32_t c3, c45;
@@ -62,8 +47,12 @@ struct XOmega {
 // part of erf, that of erfc (not when erf with the same omega is formed), Gaussian, exp(-wr^2)/r (alone)
 enum { kSumOv = 1, kSumCo = 2, kSumEr = 4, kSumX = 8, kSumGa = 16, kSumAll = 31, kSumGc = 32 };
 
-// Per-primitive record of the extended-float radial sums (32 bytes): alpha and cw (see CoulPrim) as m 2^e, m in
-// [2^62, 2^63), the sign of cw in bit 63 of wm; fw as in CoulPrim.
+// Per-primitive record of the extended-float radial sums (32 bytes): alpha and cw as m 2^e, m in [2^62, 2^63), the sign of cw
+// in bit 63 of wm,
+//   cw = sqrt(2 pi^{5/2}) w2c / alpha   so that 2 pi^{5/2} w / (alpha beta sqrt(c)) = cw_a cw_b / sqrt(c)
+//   fw = w2c alpha^{-3/2}       the far-field weight: for T >= kFarT every order of
+//                               w 2 pi^{5/2} / (alpha beta sqrt(c)) (-rho)^n F_n(T) equals
+//                               fw_a fw_b pi^3 (-1)^n (2n-1)!! (2R^2)^{-n} / R
 struct alignas(32) XPrim {
     uint64_t am, wm;
     int ae, we;
@@ -96,28 +85,10 @@ struct alignas(32) Vec4 {
 
 // Per-primitive record on the device (32 bytes).
 //   alpha, 1/alpha, w2c = N_l c / (2 alpha)^l (the two-center weight of
-//   Eq. O_rab2_deriv), wN = N_l c (normalised coefficient, used by (aab)).
+//   Eq. O_rab2_deriv), wN = N_l c (normalised coefficient).  Read by the (a|r_a^{2n}|b) kernels and, w2c, by the
+//   family contraction.
 struct alignas(32) PrimRec {
     double alpha, inv_alpha, w2c, wN;
-};
-
-// Per-primitive weights of the Coulomb-type radial terms (Table S1), 16 bytes:
-//   cw = sqrt(2 pi^{5/2}) w2c / alpha   so that 2 pi^{5/2} w / (alpha beta sqrt(c)) = cw_a cw_b / sqrt(c)
-//   fw = w2c alpha^{-3/2}       the far-field weight: for T >= kBoysTmax every order of
-//                               w 2 pi^{5/2} / (alpha beta sqrt(c)) (-rho)^n F_n(T) equals
-//                               fw_a fw_b pi^3 (-1)^n (2n-1)!! (2R^2)^{-n} / R
-struct alignas(16) CoulPrim {
-    double cw, fw;
-};
-
-// Mixed-precision (double-float) copies: each value v as float2 (hi, lo),
-// hi = fl32(v), lo = fl32(v - hi); fw is the FP64 far-field weight of CoulPrim.
-struct alignas(32) MixPrim {
-    float2 alpha, inv_alpha, wN;
-    double fw;
-};
-struct alignas(32) MixCenter {
-    float2 x, y, z, pad;
 };
 
 // Small constant tables, passed by value in kernel parameters.
@@ -138,19 +109,6 @@ struct Consts {
 };
 
 void fill_consts(Consts &k);
-
-// Double-float constants of the mixed-precision kernels.
-struct ConstsMix {
-    float2 A[kLmaxR + 1][kLmaxR + 1];      // A_{l,mu} (l <= 10: two-center and (aab) L_a)
-    float2 jB[kJmax][kJmax];               // (2j-1)!! B_{j,kappa}
-    float2 inv_int[128];                   // 1/n
-    float2 inv_fact[14];                   // 1/t!
-    float inv_fact_f[14];
-    float2 pi32, pi3, two_pi52, sqrt_pi_half, two_pi;
-    float2 dfact[kBoysN];                  // (2n-1)!!
-};
-
-void fill_consts_mix(ConstsMix &k);
 
 // Coefficients of the expanded angular part (shg_cg.cuh), per class (la, lb) with la <= kLmaxAabA, lb <= kLmax2c, class
 // index c = la (kLmax2c + 1) + lb, J = min(la, lb) + 1:
@@ -174,10 +132,6 @@ struct KappaMix {
 
 // Device-resident tables owned by the library, one set per device.
 struct DeviceTables {
-    const double *boys;   // [kBoysGrid][kBoysN][kBoysStride] (layout above)
-    const double *boys_e; // [kBoysGrid] exp(-T_i), T_i = i/32
-    const float4 *boys_mix;    // [kBoysGrid][kBoysN][3] (layout above)
-    const float2 *boys_e_mix;  // [kBoysGrid] exp(-T_i) as hi/lo
     CGTab cg;
     XTab x;
 };
@@ -212,9 +166,6 @@ void fused_ops(ArgsFused &a, int n_ops, const int *ops, const double *omegas, do
 // basis, plan and table pointers of a pass
 void fused_plan(ArgsFused &a, const BasisDev &b, const PlanDev &d, const DeviceTables &t, const int64_t *off);
 
-// Host generation of the Boys table (long double arithmetic).
-void make_boys_table(int per_unit, int ngrid, int nterms, double *tab, double *etab);
-
 struct BasisDev {
     int n_shells = 0, n_centers = 0;
     int64_t n_prims = 0;
@@ -222,17 +173,13 @@ struct BasisDev {
     ShellRec *shells = nullptr;   // device
     PrimRec *prims = nullptr;     // device
     Vec4 *centers = nullptr;      // device
-    MixPrim *mprims = nullptr;    // device, double-float copies for the mixed path
-    CoulPrim *cprims = nullptr;   // device, Coulomb-type weights (fused passes)
     XPrim *xprims = nullptr;      // device, extended-float primitives (radial sums)
     ScreenRec *screen = nullptr;  // device, per-shell screening data
-    MixCenter *mcenters = nullptr;
     // shg_basis_set_centers staging (allocated on its first call): raw
-    // coordinates, packed copies checked before they replace the live ones,
+    // coordinates, a packed copy checked before it replaces the live one,
     // and the smallest non-finite center index
     double *stage_raw = nullptr;
     Vec4 *stage_ctr = nullptr;
-    MixCenter *stage_mctr = nullptr;
     int *stage_bad = nullptr;
     // host copies used for validation and offsets
     int32_t *h_l = nullptr, *h_nprim = nullptr, *h_center = nullptr;
@@ -316,7 +263,6 @@ struct Args2c {
     double omega;
     double screen_thresh;         // > 0: overlap / Gaussian-operator pairs bounded below it write zeros
     const ScreenRec *screen;
-    const double *boys, *boys_e;
     // gradient kernels only: upstream weights W (blocks at w + w_off[p]) and
     // the per-pair outputs dI/dR_a . W and dI/dR_b . W
     const long long *w_off;
@@ -361,33 +307,16 @@ struct FamGroup {
 struct ArgsFam {
     const ShellRec *shells;
     const PrimRec *prims;
+    const XPrim *xprims;
     const Vec4 *centers;
     const int32_t *pair_a, *pair_b;     // the family subset of the pair list, in group order
     const FamGroup *groups;
     int n_groups;
     int *counter;
     double *o_pre;                      // [n_subset][kJmax]
-    double omega;
-    const double *boys, *boys_e;
+    XOmega omega;
+    XTab t;
     Consts k;
-};
-
-// Arguments of the mixed-precision two-center kernels (by value).
-struct ArgsMix {
-    const ShellRec *shells;
-    const MixPrim *prims;
-    const MixCenter *centers;
-    const int32_t *pair_a, *pair_b;
-    const int32_t *perm;
-    int *counter;
-    const long long *out_off;
-    double *out;
-    float2 omega, omega2;
-    double omega_d, screen_thresh;
-    const ScreenRec *screen;
-    const float4 *boys;
-    const float2 *boys_e;
-    ConstsMix km;
 };
 
 // Mixed-precision pass: radial sums as the FP64 pass, angular part in double-float.
@@ -471,7 +400,7 @@ int persistent_grid_2c(int op, int precision, int threads = 128, int ctas_per_sm
 cudaError_t launch_2c_fused(const ArgsFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
 cudaError_t launch_2c_all(const ArgsFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
 cudaError_t launch_2c_one(const ArgsFused &args, cudaStream_t s, int threads, int ctas_per_sm);
-cudaError_t launch_pack_centers(const double *raw, int n, Vec4 *ctr, MixCenter *mctr, int *bad, cudaStream_t s);
+cudaError_t launch_pack_centers(const double *raw, int n, Vec4 *ctr, int *bad, cudaStream_t s);
 cudaError_t launch_family_radial(const ArgsFam &a, int op, cudaStream_t s);
 cudaError_t launch_gather_i64(const int64_t *src, const int32_t *idx, int64_t n, int64_t *dst, cudaStream_t s);
 cudaError_t launch_scatter_2c(const ShellRec *shells, int64_t n, const int32_t *pa, const int32_t *pb,

@@ -16,6 +16,7 @@
 
 #include "shg_cg.cuh"
 #include "shg_tilemap.cuh"
+#include "shg_xradial.cuh"
 
 #include <cstdio>
 
@@ -25,10 +26,10 @@ namespace {
 using namespace dev;
 
 // ------------------------------------------------------------------------- //
-// One shell pair, FP64.                                                     //
+// One shell pair from its contracted radial orders (family path).           //
 // ------------------------------------------------------------------------- //
-template <int OP, int J>
-__device__ void pair_2c_fp64(const Args2c &g, int p)
+template <int J>
+__device__ void pair_2c_pre(const Args2c &g, int p)
 {
     const ShellRec sa = g.shells[g.pair_a[p]];
     const ShellRec sb = g.shells[g.pair_b[p]];
@@ -38,24 +39,9 @@ __device__ void pair_2c_fp64(const Args2c &g, int p)
     const double vx = A.x - B.x, vy = A.y - B.y, vz = A.z - B.z;
     const double R2 = vx * vx + vy * vy + vz * vz;
     const int kmax = la + lb;
-    double O[J], E[J];
+    double O[J];
 #pragma unroll
-    for (int j = 0; j < J; ++j) O[j] = E[j] = 0.0;
-    if (OP == OP_PRE) {
-#pragma unroll
-        for (int j = 0; j < J; ++j) O[j] = g.o_pre[(int64_t)p * kJmax + j];
-    } else {
-        // one flat loop over the Ka*Kb primitive pairs: a tile holds one class's
-        // pairs in descending Ka*Kb, so the lanes' trip counts differ only where
-        // a tile straddles two Ka*Kb values
-        const int Kb = sb.nprim, npp = sa.nprim * Kb;
-        for (int q = 0; q < npp; ++q) {
-            const int ia = q / Kb, ib = q - ia * Kb;
-            radial_acc_fp64<OP, J>(g.prims[sa.prim_off + ia], g.prims[sb.prim_off + ib], R2, kmax, la, g, O, E);
-        }
-        radial_finish_fp64<OP, J>(R2, kmax, g.k, O, E);
-    }
-
+    for (int j = 0; j < J; ++j) O[j] = g.o_pre[(int64_t)p * kJmax + j];
     double P[cg::kNP2], PF[cg::kNP2], C[2 * kLmax2c + 1], S[2 * kLmax2c + 1];
     cg::harmonics(vx, vy, vz, R2, kmax, J, g.k, P, C, S);
     cg::block_from_orders<J>(g.cg, la, lb, R2, O, 0.0, P, C, S, PF, 0, 1, g.out + g.out_off[p]);
@@ -287,13 +273,13 @@ __device__ __forceinline__ void pair_2c_fp64_dispatch(const Args2c &g, int p, in
         }
     }
     switch (J) {
-    case 1: pair_2c_fp64<OP, 1>(g, p); break;
-    case 2: pair_2c_fp64<OP, 2>(g, p); break;
-    case 3: pair_2c_fp64<OP, 3>(g, p); break;
-    case 4: pair_2c_fp64<OP, 4>(g, p); break;
-    case 5: pair_2c_fp64<OP, 5>(g, p); break;
-    case 6: pair_2c_fp64<OP, 6>(g, p); break;
-    default: pair_2c_fp64<OP, 7>(g, p); break;
+    case 1: pair_2c_pre<1>(g, p); break;
+    case 2: pair_2c_pre<2>(g, p); break;
+    case 3: pair_2c_pre<3>(g, p); break;
+    case 4: pair_2c_pre<4>(g, p); break;
+    case 5: pair_2c_pre<5>(g, p); break;
+    case 6: pair_2c_pre<6>(g, p); break;
+    default: pair_2c_pre<7>(g, p); break;
     }
 }
 
@@ -526,34 +512,26 @@ __global__ void k_make_tiles(int n_chunks, int chunk, int bins_per_class, int n_
 // ------------------------------------------------------------------------- //
 // Debug: Boys values through the device code path.                          //
 // ------------------------------------------------------------------------- //
-__global__ void k_debug_boys(int64_t n, const double *__restrict__ T, int nmax, double *__restrict__ F,
-                             const double *tab, const double *etab, const Consts k)
+__global__ void k_debug_boys(int64_t n, const double *__restrict__ T, int nmax, double *__restrict__ F, XTab tab,
+                             const Consts k)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double f[kBoysN];
-        boys_top<kBoysN>(T[i], kBoysN - 1, tab, etab, k, f);
-        for (int m = 0; m <= nmax; ++m) F[i * (nmax + 1) + m] = f[kBoysN - 1 - m];
-    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        for (int m = 0; m <= nmax; ++m) {
+            xfp::xf f, e;
+            xrad::boys_any(xfp::from_double(T[i]), m, tab, k.dfact[m], false, f, e);
+            F[i * (nmax + 1) + m] = xfp::to_double(f, 0);
+        }
 }
 
 // ------------------------------------------------------------------------- //
-// Center packing for shg_basis_set_centers: FP64 Vec4 and the double-float   //
-// split (hi = nearest float, lo = nearest float of the exact remainder).     //
+// Center packing for shg_basis_set_centers.                                  //
 // ------------------------------------------------------------------------- //
-__device__ __forceinline__ float2 split_df(double v)
-{
-    const float hi = __double2float_rn(v);
-    return make_float2(hi, __double2float_rn(v - (double)hi));
-}
-
-__global__ void k_pack_centers(const double *__restrict__ raw, int n, Vec4 *__restrict__ ctr,
-                               MixCenter *__restrict__ mctr, int *bad)
+__global__ void k_pack_centers(const double *__restrict__ raw, int n, Vec4 *__restrict__ ctr, int *bad)
 {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
         const double x = raw[3 * c], y = raw[3 * c + 1], z = raw[3 * c + 2];
         if (!isfinite(x) || !isfinite(y) || !isfinite(z)) atomicMin(bad, c);
         ctr[c] = Vec4{x, y, z, 0.0};
-        mctr[c] = MixCenter{split_df(x), split_df(y), split_df(z), make_float2(0.f, 0.f)};
     }
 }
 
@@ -685,11 +663,11 @@ int persistent_grid_2c(int op, int precision, int threads, int ctas_per_sm)
     return sms * per;
 }
 
-cudaError_t launch_pack_centers(const double *raw, int n, Vec4 *ctr, MixCenter *mctr, int *bad, cudaStream_t s)
+cudaError_t launch_pack_centers(const double *raw, int n, Vec4 *ctr, int *bad, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int blocks = (n + 255) / 256 < 1216 ? (n + 255) / 256 : 1216;
-    k_pack_centers<<<blocks, 256, 0, s>>>(raw, n, ctr, mctr, bad);
+    k_pack_centers<<<blocks, 256, 0, s>>>(raw, n, ctr, bad);
     return cudaGetLastError();
 }
 
@@ -699,7 +677,7 @@ cudaError_t launch_debug_boys(int64_t n, const double *T, int nmax, double *F, c
     fill_consts(k);
     if (n <= 0) return cudaSuccess;
     const int blocks = (int)((n + 127) / 128 < 4096 ? (n + 127) / 128 : 4096);
-    k_debug_boys<<<blocks, 128, 0, s>>>(n, T, nmax, F, t.boys, t.boys_e, k);
+    k_debug_boys<<<blocks, 128, 0, s>>>(n, T, nmax, F, t.x, k);
     return cudaGetLastError();
 }
 
