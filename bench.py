@@ -221,8 +221,8 @@ def run_reference(args, rank, world):
 # the sources that build the two-center kernels the profiles describe (their
 # device code, tables and launch logic); the (aab), family, gradient and
 # allocation-free translation units are not part of them
-KERNEL_SOURCES = ["shg_api.cpp", "shg_device.cuh", "shg_df.cuh", "shg_fused.cu", "shg_grad_angular.cuh",
-                  "shg_internal.h", "shg_kernels.cu", "shg_mix_angular.cuh", "shg_mixed.cu"]
+KERNEL_SOURCES = sorted(f for f in os.listdir(os.path.join(ROOT, "paper_1701_06588_gb300", "csrc"))
+                        if f.endswith((".cu", ".cuh", ".cpp", ".h")))
 
 
 def kernel_sources_sha():
