@@ -26,15 +26,6 @@ __device__ __forceinline__ bool screened(const Args3c &g, int p, double R2)
     return screen_bound(at, rb, R2, OP_OVERLAP, 0.0) < g.screen_thresh;
 }
 
-template <int NP>
-__device__ __forceinline__ void radial_orders(const Args3c &g, const Shape &sh, const ShellRec &sa, const ShellRec &st,
-                                              const ShellRec &sb, double R2, int first, int gl, double *part, double *sum)
-{
-    double P[NP][kJmax];
-    radial<NP, 0>(g, sa, st, sb, R2, sh.Lmin, sh.lb, first, P);
-    reduce<NP, 0>(sh, gl, P, part, sum);
-}
-
 __device__ __forceinline__ void tile_aab(const Args3c &g, const Tile &t, int lane, double *smem)
 {
     const Shape sh(t.cls);
@@ -53,13 +44,14 @@ __device__ __forceinline__ void tile_aab(const Args3c &g, const Tile &t, int lan
     double *sum = smem + slot * g.slot_doubles, *F = sum + nq, *C = F + nq, *S = C + sh.kmax + 1, *PF = S + sh.kmax + 1;
     double *Bk = PF + np;                                       // [mbase + M + L][cosine, sine column]
     switch (sh.nL) {
-    case 1: radial_orders<1>(g, sh, sa, st, sb, R2, first, gl, PF, sum); break;
-    case 2: radial_orders<2>(g, sh, sa, st, sb, R2, first, gl, PF, sum); break;
-    case 3: radial_orders<3>(g, sh, sa, st, sb, R2, first, gl, PF, sum); break;
-    case 4: radial_orders<4>(g, sh, sa, st, sb, R2, first, gl, PF, sum); break;
-    case 5: radial_orders<5>(g, sh, sa, st, sb, R2, first, gl, PF, sum); break;
-    default: radial_orders<6>(g, sh, sa, st, sb, R2, first, gl, PF, sum); break;
+    case 1: radial<1>(g, sh, 0, sa, st, sb, R2, first, PF + gl); break;
+    case 2: radial<2>(g, sh, 0, sa, st, sb, R2, first, PF + gl); break;
+    case 3: radial<3>(g, sh, 0, sa, st, sb, R2, first, PF + gl); break;
+    case 4: radial<4>(g, sh, 0, sa, st, sb, R2, first, PF + gl); break;
+    case 5: radial<5>(g, sh, 0, sa, st, sb, R2, first, PF + gl); break;
+    default: radial<6>(g, sh, 0, sa, st, sb, R2, first, PF + gl); break;
     }
+    reduce(nq, gl, PF, sum);
 
     // F_q of every (L, q)
     for (int v = gl; v < nq; v += kLanes) {
@@ -96,38 +88,40 @@ __device__ __forceinline__ void tile_aab(const Args3c &g, const Tile &t, int lan
     const int la = sh.la, lt = sh.lt, lb = sh.lb, nt = 2 * lt + 1, nb = 2 * lb + 1;
     double *out = g.out + g.out_off[p];
     const double *h0 = g.cg.h + __ldg(g.cg.gbase + la * (kLmax2c + 1) + lt);
-    const int Jat = sh.nL, nat = (la + 1) * (lt + 1);
+    const int Jat = sh.nL, nat = (la + 1) * (lt + 1), nset = (sh.mbase(sh.nL) + sh.nL) / 2;      // (L, |M|) sets
     for (int b = 0; b <= lb; ++b) {
         // columns +b and -b of every block (L, lb): sets (+-m, +-b)
-        for (int i = 0, pb = 0, mb = 0; i < sh.nL; ++i) {
-            const int L = sh.L(i), J = sh.J(i), km = L + lb;
-            const double *g0 = g.cg.g + __ldg(g.cg.gbase + L * (kLmax2c + 1) + lb) + 2 * J * b;
-            for (int m = gl; m <= L; m += kLanes) {
-                const double *gm = g0 + 2 * J * (lb + 1) * m;
-                const int m1 = m > b ? m - b : b - m, m2 = m + b;
-                const int n1 = min(J, (km - m1) / 2 + 1);
-                const double *f1 = PF + pb + m1 * J;
-                double X1 = __ldg(gm) * f1[0];
-                for (int q = 1; q < n1; ++q) X1 = fma(__ldg(gm + q), f1[q], X1);
-                double *o = Bk + 2 * (mb + L);
-                if (m && b) {
-                    const int n2 = min(J, (km - m2) / 2 + 1);
-                    const double *f2 = PF + pb + m2 * J;
-                    double X2 = __ldg(gm + J) * f2[0];
-                    for (int q = 1; q < n2; ++q) X2 = fma(__ldg(gm + J + q), f2[q], X2);
-                    const double c1 = C[m1] * X1, s2 = S[m2] * X2, s1 = m > b ? S[m1] : -S[m1];
-                    o[2 * m] = fma(C[m2], X2, c1);
-                    o[-2 * m + 1] = fma(-C[m2], X2, c1);
-                    o[-2 * m] = fma(s1, X1, s2);
-                    o[2 * m + 1] = fma(-s1, X1, s2);
-                } else {
-                    o[2 * m] = C[m1] * X1;
-                    if (m) o[-2 * m] = S[m1] * X1;
-                    if (b) o[1] = S[m1] * X1;
-                }
+        for (int v = gl, i = 0, m = gl, pb = 0, mb = 0; v < nset; v += kLanes, m += kLanes) {
+            while (m > sh.L(i)) {
+                const int L = sh.L(i);
+                m -= L + 1;
+                pb += (L + lb + 1) * sh.J(i);
+                mb += 2 * L + 1;
+                ++i;
             }
-            pb += (km + 1) * J;
-            mb += 2 * L + 1;
+            const int L = sh.L(i), J = sh.J(i), km = L + lb;
+            const double *gm = g.cg.g + __ldg(g.cg.gbase + L * (kLmax2c + 1) + lb) + 2 * J * (b + (lb + 1) * m);
+            const int m1 = m > b ? m - b : b - m, m2 = m + b;
+            const int n1 = min(J, (km - m1) / 2 + 1);
+            const double *f1 = PF + pb + m1 * J;
+            double X1 = __ldg(gm) * f1[0];
+            for (int q = 1; q < n1; ++q) X1 = fma(__ldg(gm + q), f1[q], X1);
+            double *o = Bk + 2 * (mb + L);
+            if (m && b) {
+                const int n2 = min(J, (km - m2) / 2 + 1);
+                const double *f2 = PF + pb + m2 * J;
+                double X2 = __ldg(gm + J) * f2[0];
+                for (int q = 1; q < n2; ++q) X2 = fma(__ldg(gm + J + q), f2[q], X2);
+                const double c1 = C[m1] * X1, s2 = S[m2] * X2, s1 = m > b ? S[m1] : -S[m1];
+                o[2 * m] = fma(C[m2], X2, c1);
+                o[-2 * m + 1] = fma(-C[m2], X2, c1);
+                o[-2 * m] = fma(s1, X1, s2);
+                o[2 * m + 1] = fma(-s1, X1, s2);
+            } else {
+                o[2 * m] = C[m1] * X1;
+                if (m) o[-2 * m] = S[m1] * X1;
+                if (b) o[1] = S[m1] * X1;
+            }
         }
         __syncwarp();
         // sums over (L, M) for the sets (+-ma, +-mt)
@@ -171,7 +165,7 @@ __device__ __forceinline__ void tile_aab(const Args3c &g, const Tile &t, int lan
     }
 }
 
-__global__ void __launch_bounds__(32, 12) k_3c_fp64(const Args3c g)
+__global__ void __launch_bounds__(32, 16) k_3c_fp64(const Args3c g)
 {
     extern __shared__ double smem[];
     const int lane = threadIdx.x;

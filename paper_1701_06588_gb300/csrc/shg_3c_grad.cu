@@ -18,15 +18,6 @@ __host__ __device__ inline int slot_doubles(const Shape &s)
     return n1 + 2 * nq + 2 * (s.kmax + 1) + (work > ang ? work : ang);
 }
 
-template <int NP>
-__device__ __forceinline__ void radial_orders(const Args3c &g, const Shape &sh, const ShellRec &sa, const ShellRec &st,
-                                              const ShellRec &sb, double R2, int first, int gl, double *part, double *sum)
-{
-    double P[NP][kJmax + 1];
-    radial<NP, 1>(g, sa, st, sb, R2, sh.Lmin, sh.lb, first, P);
-    reduce<NP, 1>(sh, gl, P, part, sum);
-}
-
 __device__ __forceinline__ void tile_aab_grad(const Args3c &g, const Tile &t, int lane, double *smem)
 {
     const Shape sh(t.cls);
@@ -40,17 +31,21 @@ __device__ __forceinline__ void tile_aab_grad(const Args3c &g, const Tile &t, in
 
     const int la = sh.la, lt = sh.lt, lb = sh.lb, nL = sh.nL, nt = 2 * lt + 1, nb = 2 * lb + 1, kmax = sh.kmax;
     const int nq = sh.qbase(nL), np = sh.pbase(nL), nat = (la + 1) * (lt + 1);
+    // (L, |M|) sets and (L, M') coefficients
+    const int nset = (sh.mbase(nL) + nL) / 2, ncoef = nset + nL * lb;
     double *sum = smem + slot * g.slot_doubles, *F = sum + nq + nL, *D = F + nq, *C = D + nq, *S = C + kmax + 1;
     double *Ac = S + kmax + 1, *As = Ac + np, *Wc = As + np, *Uk = Wc + 8 * nat;
     const int first = own ? gl : kNone;
     switch (nL) {
-    case 1: radial_orders<1>(g, sh, sa, st, sb, R2, first, gl, Ac, sum); break;
-    case 2: radial_orders<2>(g, sh, sa, st, sb, R2, first, gl, Ac, sum); break;
-    case 3: radial_orders<3>(g, sh, sa, st, sb, R2, first, gl, Ac, sum); break;
-    case 4: radial_orders<4>(g, sh, sa, st, sb, R2, first, gl, Ac, sum); break;
-    case 5: radial_orders<5>(g, sh, sa, st, sb, R2, first, gl, Ac, sum); break;
-    default: radial_orders<6>(g, sh, sa, st, sb, R2, first, gl, Ac, sum); break;
+    case 1: radial<1>(g, sh, 1, sa, st, sb, R2, first, Ac + gl); break;
+    case 2: radial<2>(g, sh, 1, sa, st, sb, R2, first, Ac + gl); break;
+    case 3: radial<3>(g, sh, 1, sa, st, sb, R2, first, Ac + gl); break;
+    case 4: radial<4>(g, sh, 1, sa, st, sb, R2, first, Ac + gl); break;
+    case 5: radial<5>(g, sh, 1, sa, st, sb, R2, first, Ac + gl); break;
+    default: radial<6>(g, sh, 1, sa, st, sb, R2, first, Ac + gl); break;
     }
+    reduce(nq + nL, gl, Ac, sum);
+
     // F_q and F_q' of every (L, q); O[j] = P^{(L+lb+1-j)}
     for (int v = gl; v < nq; v += kLanes) {
         int i = 0, q = v;
@@ -96,71 +91,79 @@ __device__ __forceinline__ void tile_aab_grad(const Args3c &g, const Tile &t, in
         }
         __syncwarp();
         // U_{L,+-m} of both columns: the sets with ||ma| - |mt|| = m and |ma| + |mt| = m
-        for (int i = 0, mb = 0; i < nL; ++i) {
-            const int L = sh.L(i), p_ = nL - 1 - i;
-            for (int m = gl; m <= L; m += kLanes) {
-                double uc[2] = {0.0, 0.0}, us[2] = {0.0, 0.0};
-                for (int a = 0; a <= la; ++a) {
-                    for (int k = 0; k < 2; ++k) {
-                        const int c = k ? a + m : a - m;
-                        if (c < 0 || c > lt || (k && !m)) continue;
-                        const double hw = __ldg(h0 + (a * (lt + 1) + c) * 2 * nL + p_);
-                        const double *o = Wc + 8 * (a * (lt + 1) + c);
-                        for (int col = 0; col < ncol; ++col) {
-                            uc[col] = fma(hw, o[4 * col], uc[col]);
-                            if (m) us[col] = fma(hw, o[4 * col + 1], us[col]);
-                        }
-                    }
-                    const int c = m - a;
-                    if (a && c > 0 && c <= lt) {
-                        const double hw = __ldg(h0 + (a * (lt + 1) + c) * 2 * nL + nL + p_);
-                        const double *o = Wc + 8 * (a * (lt + 1) + c);
-                        for (int col = 0; col < ncol; ++col) {
-                            uc[col] = fma(hw, o[4 * col + 2], uc[col]);
-                            us[col] = fma(hw, o[4 * col + 3], us[col]);
-                        }
+        for (int v = gl, i = 0, m = gl, mb = 0; v < nset; v += kLanes, m += kLanes) {
+            while (m > sh.L(i)) {
+                m -= sh.L(i) + 1;
+                mb += 2 * sh.L(i) + 1;
+                ++i;
+            }
+            const double *hp = h0 + nL - 1 - i;
+            double uc[2] = {0.0, 0.0}, us[2] = {0.0, 0.0};
+            for (int a = 0; a <= la; ++a) {
+                for (int k = 0; k < 2; ++k) {
+                    const int c = k ? a + m : a - m;
+                    if (c < 0 || c > lt || (k && !m)) continue;
+                    const double hw = __ldg(hp + (a * (lt + 1) + c) * 2 * nL);
+                    const double *o = Wc + 8 * (a * (lt + 1) + c);
+                    uc[0] = fma(hw, o[0], uc[0]);
+                    if (m) us[0] = fma(hw, o[1], us[0]);
+                    if (b) {
+                        uc[1] = fma(hw, o[4], uc[1]);
+                        if (m) us[1] = fma(hw, o[5], us[1]);
                     }
                 }
-                double *o = Uk + 2 * (mb + L);
-                for (int col = 0; col < ncol; ++col) {
-                    o[2 * m + col] = uc[col];
-                    if (m) o[-2 * m + col] = us[col];
+                const int c = m - a;
+                if (a && c > 0 && c <= lt) {
+                    const double hw = __ldg(hp + (a * (lt + 1) + c) * 2 * nL + nL);
+                    const double *o = Wc + 8 * (a * (lt + 1) + c);
+                    uc[0] = fma(hw, o[2], uc[0]);
+                    us[0] = fma(hw, o[3], us[0]);
+                    if (b) {
+                        uc[1] = fma(hw, o[6], uc[1]);
+                        us[1] = fma(hw, o[7], us[1]);
+                    }
                 }
             }
-            mb += 2 * L + 1;
+            double *o = Uk + 2 * (mb + sh.L(i));
+            for (int col = 0; col < ncol; ++col) {
+                o[2 * m + col] = uc[col];
+                if (m) o[-2 * m + col] = us[col];
+            }
         }
         __syncwarp();
         // A_{L,M'}: the sets (+-m, +-b) with |m - b| = M' and m + b = M'
-        for (int i = 0, pb = 0, mb = 0; i < nL; ++i) {
-            const int L = sh.L(i), J = sh.J(i), km = L + lb;
+        for (int v = gl, i = 0, M = gl, pb = 0, mb = 0; v < ncoef; v += kLanes, M += kLanes) {
+            while (M > sh.L(i) + lb) {
+                const int L = sh.L(i);
+                M -= L + lb + 1;
+                pb += (L + lb + 1) * sh.J(i);
+                mb += 2 * L + 1;
+                ++i;
+            }
+            const int L = sh.L(i), J = sh.J(i), n = min(J, (L + lb - M) / 2 + 1);
             const double *g0 = g.cg.g + __ldg(g.cg.gbase + L * (kLmax2c + 1) + lb) + 2 * J * b;
             const double *U = Uk + 2 * (mb + L);
-            for (int M = gl; M <= km; M += kLanes) {
-                const int n = min(J, (km - M) / 2 + 1);
-                double *ac = Ac + pb + M * J, *as = As + pb + M * J;
-                for (int k = 0; k < 3; ++k) {
-                    // m - b = M, b - m = M, m + b = M
-                    const int m = k == 0 ? M + b : k == 1 ? b - M : M - b;
-                    if (m < 0 || m > L || (k == 1 && !M) || (k == 2 && (!m || !b))) continue;
-                    const double *gm = g0 + 2 * J * (lb + 1) * m + (k == 2 ? J : 0);
-                    double u, v;
-                    if (m && b) {
-                        const double cc = U[2 * m], ss = U[-2 * m + 1], sc = U[-2 * m], cs = U[2 * m + 1];
-                        u = k == 2 ? cc - ss : cc + ss;
-                        v = k == 2 ? sc + cs : k == 0 ? sc - cs : cs - sc;
-                    } else {
-                        u = U[2 * m];
-                        v = m ? U[-2 * m] : b ? U[1] : 0.0;
-                    }
-                    for (int q = 0; q < n; ++q) {
-                        const double c = __ldg(gm + q);
-                        ac[q] = fma(c, u, ac[q]);
-                        if (M) as[q] = fma(c, v, as[q]);
-                    }
+            double *ac = Ac + pb + M * J, *as = As + pb + M * J;
+            for (int k = 0; k < 3; ++k) {
+                // m - b = M, b - m = M, m + b = M
+                const int m = k == 0 ? M + b : k == 1 ? b - M : M - b;
+                if (m < 0 || m > L || (k == 1 && !M) || (k == 2 && (!m || !b))) continue;
+                const double *gm = g0 + 2 * J * (lb + 1) * m + (k == 2 ? J : 0);
+                double u, w_;
+                if (m && b) {
+                    const double cc = U[2 * m], ss = U[-2 * m + 1], sc = U[-2 * m], cs = U[2 * m + 1];
+                    u = k == 2 ? cc - ss : cc + ss;
+                    w_ = k == 2 ? sc + cs : k == 0 ? sc - cs : cs - sc;
+                } else {
+                    u = U[2 * m];
+                    w_ = m ? U[-2 * m] : b ? U[1] : 0.0;
+                }
+                for (int q = 0; q < n; ++q) {
+                    const double c = __ldg(gm + q);
+                    ac[q] = fma(c, u, ac[q]);
+                    if (M) as[q] = fma(c, w_, as[q]);
                 }
             }
-            pb += (km + 1) * J;
-            mb += 2 * L + 1;
         }
         __syncwarp();
     }
@@ -220,7 +223,7 @@ __device__ __forceinline__ void tile_aab_grad(const Args3c &g, const Tile &t, in
     __syncwarp();
 }
 
-__global__ void __launch_bounds__(32, 12) k_3c_grad_fp64(const Args3c g)
+__global__ void __launch_bounds__(32, 16) k_3c_grad_fp64(const Args3c g)
 {
     extern __shared__ double smem[];
     const int lane = threadIdx.x;

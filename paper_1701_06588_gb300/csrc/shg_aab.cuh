@@ -60,22 +60,25 @@ constexpr double kWeight = dev::kPi32 / (dev::kTwoPi52 * 5.914967172795613);
 // First primitive combination of a lane that sums none
 constexpr int kNone = 1 << 30;
 
-// Radial orders of one triple, summed over the primitive combinations gl, gl + 8, ..: P[i][j] = P_L^{(L + lb + X - j)},
-// L = Lmin + 2i, j = 0 .. min(L, lb) + X (X = 1 for gradients), NP = number of L.  Per combination
-//   P_L^{(k)} += W (2 alpha')^{-L} (-rho)^k sum_i binom(k,i) r_i,
-//   r_i = (-tau)^i sum_{m=i}^{p} K_{L,m} alpha'^{m-p} c^{-m} Lag_{m-i}^{(1/2+i)}(-u),    tau = beta/alpha', u = beta^2 R^2/c,
-// K_{L,m} = binom(p,m) (L)_{p-m} m!, since d^i/du^i of the polynomial of (0|r_a^{2m}|0) (Eq. I_jab) is 2^m m! times that
-// Laguerre polynomial; all terms of r_i are positive, and the polynomials of one triple follow from row i = 0 by one
+// Radial orders of one triple, summed over the primitive combinations first, first + 8, ..: P_L^{(L + lb + X - j)} of L(i),
+// j = 0 .. min(L, lb) + X (X = 1 for gradients), at part[v * 8] with v counting (i, j).  Per combination
+//   P_L^{(k)} += W (2 alpha')^{-L} (-rho)^k sum_o binom(k,o) r_o,
+//   r_o = (-tau)^o sum_{m=o}^{p} K_{L,m} alpha'^{m-p} c^{-m} Lag_{m-o}^{(1/2+o)}(-u),    tau = beta/alpha', u = beta^2 R^2/c,
+// K_{L,m} = binom(p,m) (L)_{p-m} m!, since d^o/du^o of the polynomial of (0|r_a^{2m}|0) (Eq. I_jab) is 2^m m! times that
+// Laguerre polynomial; all terms of r_o are positive, and the polynomials of one combination follow from row o = 0 by one
 // addition each.  About half the FP64 operations of summing (0|r_a^{2m}|0)^{(k)} order by order; the prefactors are
-// extended floats on the integer pipes.
-template <int NP, int X>
-__device__ __forceinline__ void radial(const Args3c &g, const ShellRec &sa, const ShellRec &st, const ShellRec &sb,
-                                       double R2, int Lmin, int lb, int first, double (&P)[NP][kJmax + X])
+// extended floats on the integer pipes.  NP = number of L (min(la, la~) + 1): the polynomials stay in registers, the sums
+// over the combinations in shared memory (an FP64 instruction holds its unit for 64 cycles, so the access beside it is
+// free).  900,000 triples: 11.2 ms whole call; sums in registers (168 of them, warps waiting for instructions in 41% of
+// their cycles) 13.4 ms, runtime loops over local arrays 12.3 ms.
+template <int NP>
+__device__ __forceinline__ void radial(const Args3c &g, const Shape &sh, int X, const ShellRec &sa, const ShellRec &st,
+                                       const ShellRec &sb, double R2, int first, double *part)
 {
-#pragma unroll
-    for (int i = 0; i < NP; ++i)
-#pragma unroll
-        for (int j = 0; j < kJmax + X; ++j) P[i][j] = 0.0;
+    constexpr int nL = NP;
+    const int Lmin = sh.Lmin, lb = sh.lb;
+    const int nq = sh.qbase(nL) + X * nL;
+    for (int v = 0; v < nq; ++v) part[v * kLanes] = 0.0;
     const int Kb = sb.nprim, Kt = st.nprim, n = sa.nprim * Kt * Kb;
     const float rKb = 1.0f / (float)Kb, rKt = 1.0f / (float)Kt;
     const xf R2x = from_double(R2);
@@ -90,8 +93,7 @@ __device__ __forceinline__ void radial(const Args3c &g, const ShellRec &sa, cons
         const xf rc = xfp::rsqrt(add(ap, be)), ic = mul(rc, rc);
         const xf bic = mul(be, ic);
         const xf rho = mul(ap, bic);
-        const xf ux = mul(mul(be, bic), R2x);
-        // N c = cw alpha (2 alpha)^l and N c / (2 beta)^lb = cw beta up to the constant of CoulPrim (kWeight)
+        // N c = cw alpha (2 alpha)^l and N c / (2 beta)^lb = cw beta up to the constant of cw (kWeight)
         const uint32_t sw = hi32(A.wm) ^ hi32(T.wm) ^ hi32(B.wm);
         constexpr uint64_t mask = ~(1ull << 63);
         xf w = muln(mulr(xf{A.wm & mask, A.we}, xf{T.wm & mask, T.we}), xf{B.wm & mask, B.we});
@@ -99,81 +101,68 @@ __device__ __forceinline__ void radial(const Args3c &g, const ShellRec &sa, cons
         if (sa.l) w = mul(w, xfp::powi(xf{al.m, al.e + 1}, sa.l));
         if (st.l) w = mul(w, xfp::powi(xf{at_.m, at_.e + 1}, st.l));
         w = mul(mul(w, mul(ic, rc)), xrad::exp_neg(mul(rho, R2x), g.exptab));
-        if (Lmin) {
-            xf h = iap;
-            h.e -= 1;                                           // 1 / (2 alpha')
-            w = mul(w, xfp::powi(h, Lmin));
-        }
+        if (Lmin) w = mul(w, xfp::powi(xf{iap.m, iap.e - 1}, Lmin));
         if (k0) w = mul(w, xfp::powi(rho, k0));
         double e = to_double(w, sw ^ ((uint32_t)k0 << 31));     // W (2 alpha')^{-Lmin} (-rho)^{k0}
         const double mrho = -to_double(rho, 0);
-        double ia1 = 0.0, c1 = 0.0, mtau = 0.0, s2 = 0.0, u = 0.0;
-        if (NP > 1) {
-            ia1 = to_double(iap, 0);
-            c1 = to_double(ic, 0);
-            mtau = -to_double(mul(be, iap), 0);
+        double pa[nL], pc[nL], tp[nL], lam[nL][nL];
+        pa[0] = pc[0] = tp[0] = 1.0;
+        lam[0][0] = 1.0;
+        double s2 = 0.0;
+        if (nL > 1) {
+            const double ia1 = to_double(iap, 0), c1 = to_double(ic, 0), mtau = -to_double(mul(be, iap), 0);
+            const double u = to_double(mul(mul(be, bic), R2x), 0);
             s2 = 0.25 * ia1 * ia1;                              // (2 alpha')^{-2}
-            u = to_double(ux, 0);
-        }
-        // row i = 0 of the Laguerre polynomials, then Lag_n^{(a+1)} = Lag_n^{(a)} + Lag_{n-1}^{(a+1)} in place
-        double lam[NP];
-        lam[0] = 1.0;
+            pa[nL > 1 ? 1 : 0] = ia1;
+            pc[nL > 1 ? 1 : 0] = c1;
+            tp[nL > 1 ? 1 : 0] = mtau;
+            lam[0][nL > 1 ? 1 : 0] = u + 1.5;
+            lam[nL > 1 ? 1 : 0][0] = 1.0;
 #pragma unroll
-        for (int m = 1; m < NP; ++m) {
-            double s = g.k3.lag[m][m];
+            for (int m = 2; m < nL; ++m) {
+                pa[m] = pa[m - 1] * ia1;
+                pc[m] = pc[m - 1] * c1;
+                tp[m] = tp[m - 1] * mtau;
+                double s = g.k3.lag[m][m];
 #pragma unroll
-            for (int j = m - 1; j >= 0; --j) s = fma(s, u, g.k3.lag[m][j]);
-            lam[m] = s;
-        }
-        // B[i][m] = K_{L,m} alpha'^{m-p} c^{-m}, then r[i][o] = (-tau)^o sum_m B[i][m] lam[m-o]
-        double pa[NP], pc[NP], B_[NP][NP], r[NP][NP];
-        pa[0] = pc[0] = 1.0;
+                for (int j = m - 1; j >= 0; --j) s = fma(s, u, g.k3.lag[m][j]);
+                lam[0][m] = s;
+                // Lag_n^{(a+1)} = Lag_n^{(a)} + Lag_{n-1}^{(a+1)}
 #pragma unroll
-        for (int m = 1; m < NP; ++m) {
-            pa[m] = m == 1 ? ia1 : pa[m - 1] * ia1;
-            pc[m] = m == 1 ? c1 : pc[m - 1] * c1;
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i)
-#pragma unroll
-            for (int m = 0; m < NP - i; ++m) {
-                const int p = NP - 1 - i;
-                const double kk = g.k3.K[Lmin + 2 * i][p][m];
-                B_[i][m] = p == 0 ? kk : kk * (m == 0 ? pa[p] : m == p ? pc[p] : pa[p - m] * pc[m]);
-            }
-        double tp = 1.0;
-#pragma unroll
-        for (int o = 0; o < NP; ++o) {
-            if (o) {
-#pragma unroll
-                for (int m = 1; m < NP - o; ++m) lam[m] += lam[m - 1];
-                tp = o == 1 ? mtau : tp * mtau;
-            }
-#pragma unroll
-            for (int i = 0; i < NP - o; ++i) {
-                const int p = NP - 1 - i;
-                double s = B_[i][o];                            // lam[0] = 1
-#pragma unroll
-                for (int m = o + 1; m <= p; ++m) s = fma(B_[i][m], lam[m - o], s);
-                r[i][o] = o ? s * tp : s;
+                for (int o = 1; o < m; ++o) lam[o][m - o] = lam[o - 1][m - o] + lam[o][m - o - 1];
+                lam[m][0] = 1.0;
             }
         }
+        double *acc = part;
 #pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            const int L = Lmin + 2 * i, kl = L > lb ? L : lb, J = (L < lb ? L : lb) + 1 + X;
+        for (int i = 0; i < nL; ++i) {
+            const int L = Lmin + 2 * i, p = nL - 1 - i, kl = L > lb ? L : lb, J = (L < lb ? L : lb) + 1 + X;
+            double bm[nL], r[nL];
+            const double *K = g.k3.K[L][p];
+#pragma unroll
+            for (int m = 0; m <= p; ++m) bm[m] = K[m] * (pa[p - m] * pc[m]);
+            r[0] = bm[0];
+#pragma unroll
+            for (int m = 1; m <= p; ++m) r[0] = fma(bm[m], lam[0][m], r[0]);
+#pragma unroll
+            for (int o = 1; o <= p; ++o) {
+                double s = bm[o];
+#pragma unroll
+                for (int m = o + 1; m <= p; ++m) s = fma(bm[m], lam[o][m - o], s);
+                r[o] = s * tp[o];
+            }
             double f = e;
+#pragma unroll 1
+            for (int j = J - 1; j >= 0; --j) {
+                const double *bn = g.k3.binom[kl + J - 1 - j];
+                double s = r[0];
 #pragma unroll
-            for (int j = kJmax + X - 1; j >= 0; --j) {
-                if (j < J) {
-                    const double *bn = g.k3.binom[kl + J - 1 - j];
-                    double s = r[i][0];
-#pragma unroll
-                    for (int o = 1; o < NP - i; ++o) s = fma(bn[o], r[i][o], s);
-                    P[i][j] = fma(f, s, P[i][j]);
-                    if (j) f *= mrho;
-                }
+                for (int o = 1; o <= p; ++o) s = fma(bn[o], r[o], s);
+                acc[j * kLanes] = fma(f, s, acc[j * kLanes]);
+                if (j) f *= mrho;
             }
-            if (i + 1 < NP) {
+            acc += J * kLanes;
+            if (i + 1 < nL) {
                 // next L: (2 alpha')^{-2} and the step of its lowest order
                 const int d = (L + 2 > lb ? L + 2 : lb) - kl;
                 e *= s2;
@@ -184,19 +173,9 @@ __device__ __forceinline__ void radial(const Args3c &g, const ShellRec &sa, cons
     }
 }
 
-// The lanes' partial sums added up through shared memory: part [8][nq] per slot, sum [nq]
-template <int NP, int X>
-__device__ __forceinline__ void reduce(const Shape &sh, int gl, const double (&P)[NP][kJmax + X], double *part, double *sum)
+// the lanes' sums added up: sum[v] over part[v * 8 ..]
+__device__ __forceinline__ void reduce(int nq, int gl, const double *part, double *sum)
 {
-    int nq = 0;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        const int J = sh.J(i) + X;
-#pragma unroll
-        for (int j = 0; j < kJmax + X; ++j)
-            if (j < J) part[(nq + j) * kLanes + gl] = P[i][j];
-        nq += J;
-    }
     __syncwarp();
     for (int v = gl; v < nq; v += kLanes) {
         double s = 0.0;
