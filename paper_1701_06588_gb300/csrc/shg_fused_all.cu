@@ -1,4 +1,5 @@
 // FP64 two-center passes of any set of operators.
+#define SHG_XF_CALLS
 #include "shg_pair2c.cuh"
 
 namespace shg {

@@ -392,6 +392,7 @@ cudaError_t launch_2c_grad_mixed(const ArgsGrad &args, cudaStream_t s, int threa
 cudaError_t launch_2c_grad_ra2n(const Args2c &args, cudaStream_t s);
 // mixed-precision pass of the classes with min(la, lb) < kMixedFp64MinL (arguments as launch_2c_fused)
 cudaError_t launch_2c_mixed(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
+cudaError_t launch_2c_mixed_all(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
 cudaError_t launch_2c(const Args2c &args, int op, int precision, int n_tiles_or_grid, bool persistent,
                       cudaStream_t s, int threads = 128);
 int persistent_grid_2c(int op, int precision, int threads = 128, int ctas_per_sm = 0);

@@ -14,13 +14,19 @@
 #include "shg_device.cuh"
 #include "shg_xf.cuh"
 
+#ifdef SHG_XF_CALLS
+#define SHG_XF_DEV static __device__ __noinline__
+#else
+#define SHG_XF_DEV __device__ __forceinline__
+#endif
+
 namespace shg {
 namespace xrad {
 using namespace xfp;
 
 // exp(-T) for T < 1024 (2^-1477 and below: a value the conversion to FP64 flushes to 0).  n = ceil(T log2 e) or one more,
 // r = n ln2 - T in [0, 0.6932), exp(r) from a table at r_j = j/512 and the series of the rest.
-__device__ __forceinline__ xf exp_neg(xf T, const uint64_t *__restrict__ tab)
+SHG_XF_DEV xf exp_neg(xf T, const uint64_t *__restrict__ tab)
 {
     if (T.e > -53) return xf{1ull << 62, -100000};
     const int s = -53 - T.e;                                                 // >= 0
@@ -46,7 +52,7 @@ __device__ __forceinline__ bool boys_fixed(xf T, uint64_t &Tf)
 
 // F_n(T) from the table of order n (BoysEnt): Taylor series about the upper end of T's cell of width 1/512, all terms
 // positive
-__device__ __forceinline__ xf boys_series(const BoysEnt *__restrict__ tab, uint64_t Tf)
+SHG_XF_DEV xf boys_series(const BoysEnt *__restrict__ tab, uint64_t Tf)
 {
     const uint32_t i = hi32(Tf) >> 15;
     const uint64_t Y = ~(Tf << 8) & 0x7fffffffffffffull;                     // (T_{i+1} - T) 2^64, less 1
