@@ -353,6 +353,8 @@ struct DevState {
     DeviceTables t{};
     int *bin_rank[2] = {nullptr, nullptr};   // [2 * kNBins]: rank of bin, then bin of rank
     int *bin_rank3 = nullptr;                // [2 * kNBins3], three-index bins by cost
+    cudaMemPool_t pool = nullptr;            // plans (plan_alloc)
+    int bases = 0;                           // live bases of the device
     bool ready = false;
 };
 
@@ -424,6 +426,47 @@ static void make_ranks(int schedule, std::vector<int> &rank, std::vector<int> &i
     }
 }
 
+// Plans come from a pool of the library: the default pool returns its memory to the system at every synchronisation
+// (release threshold 0), and planning synchronises, so a one-shot call on 2,000 pairs spent 200 of its 410 us on mapping its
+// 0.9 MB again.  This pool keeps up to kPoolKeep bytes between calls (the plan of 2M pairs takes 22 MB) and gives them
+// back when the last basis of the device is destroyed.  Stream-ordered like the default pool, shared by all threads.
+constexpr uint64_t kPoolKeep = 256ull << 20;
+
+static cudaError_t make_pool(int dev, cudaMemPool_t *pool)
+{
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = kPoolKeep;
+    cudaError_t e = cudaMemPoolCreate(pool, &props);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    return e;
+}
+
+// device memory of a plan on the current device, in the order of s (cudaFreeAsync frees it)
+static cudaError_t plan_alloc(void **p, size_t bytes, cudaStream_t s)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        pool = g_dev[dev].pool;
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+// a basis of the device was made (+1) or destroyed (-1)
+static void count_basis(int dev, int d)
+{
+    std::lock_guard<std::mutex> lk(g_mu);
+    DevState &st = g_dev[dev];
+    st.bases += d;
+    if (st.bases == 0 && st.pool) cudaMemPoolTrimTo(st.pool, 0);
+}
+
 const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
 {
     int dev = 0;
@@ -436,7 +479,7 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
     DevState &st = g_dev[dev];
     if (!st.ready) {
         int *d_r[2] = {nullptr, nullptr};
-        bool ok = cudaMalloc(&d_r[0], 2 * kNBins * sizeof(int)) == cudaSuccess &&
+        bool ok = make_pool(dev, &st.pool) == cudaSuccess && cudaMalloc(&d_r[0], 2 * kNBins * sizeof(int)) == cudaSuccess &&
                   cudaMalloc(&d_r[1], 2 * kNBins * sizeof(int)) == cudaSuccess;
         for (int s = 0; s < 2 && ok; ++s) {
             std::vector<int> rank, inv;
@@ -763,6 +806,8 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
         shg_basis_destroy(b);
         return SHG_ECUDA;
     }
+    count_basis(d.device, 1);
+    d.counted = true;
     *out = b;
     return SHG_OK;
 }
@@ -805,6 +850,7 @@ int shg_basis_set_centers(shg_basis_t *b, const double *centers)
 void shg_basis_destroy(shg_basis_t *b)
 {
     if (!b) return;
+    if (b->d.counted) count_basis(b->d.device, -1);
     cudaFree(b->d.shells);
     cudaFree(b->d.prims);
     cudaFree(b->d.centers);
@@ -914,7 +960,7 @@ int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, c
     const size_t bytes_ws = sizeof(int) * plan_ws_ints(n, kNBins, kNClass);
     const size_t bytes = bytes_perm + bytes_tiles + bytes_ws + 256;
     void *blk = nullptr;
-    SHG_CUDA(cudaMallocAsync(&blk, bytes, s));
+    SHG_CUDA(plan_alloc(&blk, bytes, s));
 
     shg_plan_t *p = new (std::nothrow) shg_plan_t;
     if (!p) {
@@ -1252,6 +1298,11 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     return SHG_OK;
 }
 
+// Most tiles that a persistent plan runs with one CTA each instead of a work counter: all of them are resident at once (8
+// warps or more per SM), spread over the SMs one by one, without the launch that clears the counter (63 tiles of 2,000
+// pairs, overlap and 1/r: 102 us persistent with four-warp CTAs, 95 us with one-warp CTAs)
+constexpr int kStaticTiles = 1024;
+
 // FP64 pass over the tiles of a plan (all of them, or those that the mixed-precision passes run in FP64)
 static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, int sel, int variant, cudaStream_t s)
 {
@@ -1259,6 +1310,11 @@ static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, int sel, int variant, cu
         a.tile_begin = 0;
         a.tile_end = sel == kAllClasses ? p->d.n_tiles : p->d.mixed_fp64_tiles;
         if (a.tile_end <= 0) return SHG_OK;
+        if (a.tile_end <= kStaticTiles) {
+            a.counter = nullptr;
+            SHG_CUDA(launch_2c_fused(a, s, 32, 0, variant));
+            return SHG_OK;
+        }
         SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), s));
         a.counter = p->d.counter;
         SHG_CUDA(launch_2c_fused(a, s, p->d.threads, p->d.ctas_per_sm, variant));
@@ -1413,7 +1469,7 @@ static int eval_3c_common(const shg_basis_t *orb, const shg_basis_t *aux, int64_
     const size_t bytes_ws = sizeof(int) * plan_ws_ints(n, kNBins3, kNClass3);
     const size_t bytes = bytes_perm + bytes_tiles + bytes_ws + 512;
     void *blk = nullptr;
-    SHG_CUDA(cudaMallocAsync(&blk, bytes, s));
+    SHG_CUDA(plan_alloc(&blk, bytes, s));
     PlanDev d;
     d.basis = &orb->d;
     d.aux = &aux->d;

@@ -187,6 +187,7 @@ struct BasisDev {
     int32_t *h_fam = nullptr;                           // family of each shell
     int32_t *h_fam_prim = nullptr, *h_fam_k = nullptr;  // per family: first primitive record, K
     int n_fams = 0;
+    bool counted = false;         // among the live bases of its device
 };
 
 // A warp's unit of work: up to kTile / group consecutive entries of the sorted list, all of one class (cls = la*7 + lb, or
