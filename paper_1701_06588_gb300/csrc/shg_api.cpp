@@ -923,14 +923,19 @@ int shg::plan_read(PlanDev &d, const int *summary, int schedule)
     for (int c = 0; c < kNClass; ++c)
         if (std::min(m.cls[c] / 7, m.cls[c] % 7) <= 1) low += summary[c + 1] - summary[c];
     d.variant = 3 * (int64_t)low > 2 * (int64_t)d.n_tiles ? 1 : 0;
-    d.mixed_fp64_tiles = d.mixed_fp64_tiles32 = 0;
+    d.df_begin = d.df_end = 0;
     if (schedule == SHG_SCHED_PERSISTENT) {
-        // the persistent rank order is J-major (J descending), so the classes with
-        // both l >= kMixedFp64MinL are its first chunks
-        int n_hi = 0;
-        for (int cls = 0; cls < kNClass; ++cls) n_hi += mixed_runs_fp64(cls);
-        d.mixed_fp64_tiles = summary[n_hi];
-        d.mixed_fp64_tiles32 = m.tile[n_hi];
+        // the persistent rank order is J-major (J descending): the classes with both l >= kMixedFp64MinL are its first
+        // chunks, the double-float classes the next
+        int n_from[3] = {};
+        for (int cls = 0; cls < kNClass; ++cls) {
+            n_from[0] += min_l(cls) >= kMixedFp64MinL;
+            n_from[1] += min_l(cls) >= kMixedDfMinL;
+            n_from[2] += min_l(cls) >= kMixedDfMinLGrad;
+        }
+        d.df_begin = summary[n_from[0]];
+        d.df_end = summary[n_from[1]];
+        d.df_end_grad = summary[n_from[2]];
     }
     return SHG_OK;
 }
@@ -1010,7 +1015,8 @@ int shg_plan_launches_prec(const shg_plan_t *p, int precision)
 {
     if (!p || (precision != SHG_PREC_FP64 && precision != SHG_PREC_MIXED)) return -1;
     if (precision == SHG_PREC_FP64 || p->d.schedule != SHG_SCHED_PERSISTENT) return p->launches;
-    return (p->d.mixed_fp64_tiles > 0) + (p->d.n_tiles > p->d.mixed_fp64_tiles);
+    const int df = p->d.df_end - p->d.df_begin;
+    return (df > 0) + (p->d.n_tiles > df);
 }
 
 int shg_plan_2c_set_variant(shg_plan_t *p, int variant)
@@ -1121,65 +1127,13 @@ void shg_plan_destroy(shg_plan_t *p)
 {
     if (!p) return;
     cudaFreeAsync(p->d.owner_block, p->d.stream);
-    if (p->d.ev_fork) cudaEventDestroy(p->d.ev_fork);
-    if (p->d.ev_join) cudaEventDestroy(p->d.ev_join);
-    if (p->d.ev_join2) cudaEventDestroy(p->d.ev_join2);
-    if (p->d.side) cudaStreamDestroy(p->d.side);
-    if (p->d.side2) cudaStreamDestroy(p->d.side2);
     delete p;
 }
 
 
-// Streams and events of a forked mixed-precision pass, created on the first
-// execution that needs them: the FP64 launch of the classes with both l >=
-// kMixedFp64MinL (a few hundred heavy tiles, one warp each) runs on `side`,
-// the double-float persistent launch on `side2`, so that the FP64 pipes work
-// on those tiles while the FP32 pipes of the rest of the GPU run the others.
-// Neither launch goes to the caller's stream, which only forks and joins (on
-// the legacy default stream a launch beside another stream's does not overlap
-// it).  `side` has the highest stream priority: its CTAs are dispatched first
-// and are resident before the persistent launch fills the SMs.
-static int plan_side_streams(shg_plan_t *p)
-{
-    if (p->d.side) return SHG_OK;
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&p->d.side, cudaStreamNonBlocking, hi) != cudaSuccess ||
-        cudaStreamCreateWithPriority(&p->d.side2, cudaStreamNonBlocking, lo) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->d.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->d.ev_join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->d.ev_join2, cudaEventDisableTiming) != cudaSuccess)
-        return fail(SHG_ECUDA, "side streams: %s", cudaGetErrorString(cudaGetLastError()));
-    return SHG_OK;
-}
-
-// fork: both side streams wait for the work already on s
-static int fork_sides(shg_plan_t *p, cudaStream_t s)
-{
-    int r = plan_side_streams(p);
-    if (r) return r;
-    SHG_CUDA(cudaEventRecord(p->d.ev_fork, s));
-    SHG_CUDA(cudaStreamWaitEvent(p->d.side, p->d.ev_fork, 0));
-    SHG_CUDA(cudaStreamWaitEvent(p->d.side2, p->d.ev_fork, 0));
-    return SHG_OK;
-}
-
-// join: s waits for both side streams
-static int join_sides(shg_plan_t *p, cudaStream_t s)
-{
-    SHG_CUDA(cudaEventRecord(p->d.ev_join, p->d.side));
-    SHG_CUDA(cudaEventRecord(p->d.ev_join2, p->d.side2));
-    SHG_CUDA(cudaStreamWaitEvent(s, p->d.ev_join, 0));
-    SHG_CUDA(cudaStreamWaitEvent(s, p->d.ev_join2, 0));
-    return SHG_OK;
-}
-
-// which classes an FP64 execution covers: all of them, or only those the
-// mixed-precision passes run in FP64
-enum { kAllClasses = 0, kMixedFp64Classes = 1 };
 static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const int64_t *off, double *out,
                      const double *o_pre, cudaStream_t s);
-static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, int sel, int variant, cudaStream_t s);
+static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, cudaStream_t s);
 static int exec_mixed(shg_plan_t *p, const ArgsFused &f, cudaStream_t s);
 
 int shg_plan_2c_exec(shg_plan_t *p, int op, double omega, double screen, int precision, const int64_t *off,
@@ -1263,7 +1217,7 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
         fused_ops(f, 1, &op, &omega, &out);
         fused_plan(f, *p->d.basis, p->d, *t, off);
         f.screen_thresh = op == SHG_OP_OVERLAP || op == SHG_OP_GAUSS ? screen : 0.0;
-        return exec_fused_fp64(p, f, kAllClasses, p->d.variant, s);
+        return exec_fused_fp64(p, f, s);
     }
     Args2c a;
     a.shells = p->d.basis->shells;
@@ -1303,73 +1257,71 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
 // pairs, overlap and 1/r: 102 us persistent with four-warp CTAs, 95 us with one-warp CTAs)
 constexpr int kStaticTiles = 1024;
 
-// FP64 pass over the tiles of a plan (all of them, or those that the mixed-precision passes run in FP64)
-static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, int sel, int variant, cudaStream_t s)
+// FP64 pass over the tiles of a plan
+static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, cudaStream_t s)
 {
     if (p->d.schedule == SHG_SCHED_PERSISTENT) {
         a.tile_begin = 0;
-        a.tile_end = sel == kAllClasses ? p->d.n_tiles : p->d.mixed_fp64_tiles;
-        if (a.tile_end <= 0) return SHG_OK;
+        a.tile_end = p->d.n_tiles;
         if (a.tile_end <= kStaticTiles) {
             a.counter = nullptr;
-            SHG_CUDA(launch_2c_fused(a, s, 32, 0, variant));
+            SHG_CUDA(launch_2c_fused(a, s, 32, 0, p->d.variant));
             return SHG_OK;
         }
         SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), s));
         a.counter = p->d.counter;
-        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, p->d.ctas_per_sm, variant));
+        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, p->d.ctas_per_sm, p->d.variant));
         return SHG_OK;
     }
     a.counter = nullptr;
     for (int cls = 0; cls < kNClass; ++cls) {
-        if (sel == kMixedFp64Classes && !mixed_runs_fp64(cls)) continue;
         a.tile_begin = p->d.class_tile_begin[cls];
         a.tile_end = p->d.class_tile_begin[cls + 1];
         if (a.tile_end <= a.tile_begin) continue;
-        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, 0, variant));
+        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, 0, p->d.variant));
     }
     return SHG_OK;
 }
 
-// Mixed-precision pass: the classes with both l >= kMixedFp64MinL in FP64 (one warp per tile on a side stream, beside
-// the double-float launch, when a persistent plan holds both kinds), the others with the double-float angular part
+// Leaves the double-float classes of a mixed-precision pass out of an FP64 launch over all tiles of a plan; with a launch
+// for them before it, the FP64 one runs beside it
+static void skip_df(ArgsFused &f, const PlanDev &d, int df_end, int *counter)
+{
+    f.tile_begin = 0;
+    f.tile_end = d.n_tiles;
+    f.skip_at = d.df_begin;
+    f.skip_n = df_end - d.df_begin;
+    f.beside = f.skip_n > 0;
+    f.counter = counter;
+}
+
+// Mixed-precision pass: the classes of mixed_runs_fp64 by the FP64 kernel, the others with the double-float angular part.
+// A persistent plan starts the double-float launch first (its tiles are among the longest) and the FP64 one beside it.
 static int exec_mixed(shg_plan_t *p, const ArgsFused &f, cudaStream_t s)
 {
-    const bool persistent = p->d.schedule == SHG_SCHED_PERSISTENT;
-    const bool fork = persistent && p->d.mixed_fp64_tiles > 0 && p->d.n_tiles > p->d.mixed_fp64_tiles;
     ArgsMixFused m;
     m.f = f;
     fill_kappa_mix(m.kappa);
-    int r;
-    if (fork) {
-        r = fork_sides(p, s);
-        if (r) return r;
-        ArgsFused a = f;
-        a.tile_begin = 0;
-        a.tile_end = p->d.mixed_fp64_tiles;
-        a.counter = nullptr;
-        SHG_CUDA(launch_2c_fused(a, p->d.side, 32, 0, 1));
-    } else {
-        r = exec_fused_fp64(p, m.f, kMixedFp64Classes, p->d.variant, s);
-        if (r) return r;
+    ArgsFused a = f;
+    if (p->d.schedule == SHG_SCHED_PERSISTENT) {
+        SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, 2 * sizeof(int), s));
+        m.f.tile_begin = p->d.df_begin;
+        m.f.tile_end = p->d.df_end;
+        m.f.counter = p->d.counter + 1;
+        SHG_CUDA(launch_2c_mixed(m, s, p->d.threads, p->d.ctas_per_sm, p->d.variant));
+        skip_df(a, p->d, p->d.df_end, p->d.counter);
+        SHG_CUDA(launch_2c_fused(a, s, p->d.threads, p->d.ctas_per_sm, p->d.variant));
+        return SHG_OK;
     }
-    if (persistent) {
-        m.f.tile_begin = p->d.mixed_fp64_tiles;
-        m.f.tile_end = p->d.n_tiles;
-        if (m.f.tile_end <= m.f.tile_begin) return SHG_OK;
-        const cudaStream_t sm = fork ? p->d.side2 : s;
-        SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), sm));
-        m.f.counter = p->d.counter;
-        SHG_CUDA(launch_2c_mixed(m, sm, p->d.threads, p->d.ctas_per_sm, p->d.variant));
-        return fork ? join_sides(p, s) : SHG_OK;
-    }
-    m.f.counter = nullptr;
+    a.counter = m.f.counter = nullptr;
     for (int cls = 0; cls < kNClass; ++cls) {
-        if (mixed_runs_fp64(cls)) continue;
-        m.f.tile_begin = p->d.class_tile_begin[cls];
-        m.f.tile_end = p->d.class_tile_begin[cls + 1];
-        if (m.f.tile_end <= m.f.tile_begin) continue;
-        SHG_CUDA(launch_2c_mixed(m, s, p->d.threads, 0, p->d.variant));
+        a.tile_begin = m.f.tile_begin = p->d.class_tile_begin[cls];
+        a.tile_end = m.f.tile_end = p->d.class_tile_begin[cls + 1];
+        if (a.tile_end <= a.tile_begin) continue;
+        if (mixed_runs_fp64(cls))
+            SHG_CUDA(launch_2c_fused(a, s, p->d.threads, 0, p->d.variant));
+        else
+            SHG_CUDA(launch_2c_mixed(m, s, p->d.threads, 0, p->d.variant));
     }
     return SHG_OK;
 }
@@ -1413,7 +1365,7 @@ int shg_plan_2c_exec_fused(shg_plan_t *p, int n_ops, const int *ops, const doubl
     fused_ops(a, n_ops, ops, omegas, outs);
     fused_plan(a, *p->d.basis, p->d, *t, off);
     if (precision == SHG_PREC_MIXED) return exec_mixed(p, a, s);
-    return exec_fused_fp64(p, a, kAllClasses, p->d.variant, s);
+    return exec_fused_fp64(p, a, s);
 }
 
 int shg_graph_2c_create_fused(shg_plan_t *p, int n_ops, const int *ops, const double *omegas, int precision,
@@ -1563,7 +1515,7 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     if (r) return r;
     const DeviceTables *t = device_tables();
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(p->d.counter, 0, sizeof(int), s);
+    cudaError_t e = cudaMemsetAsync(p->d.counter, 0, 2 * sizeof(int), s);
     if (op == SHG_OP_RA2N) {
         Args2c a{};
         a.shells = basis->d.shells;
@@ -1598,33 +1550,20 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     a.w = w;
     a.grad_a = grad_a;
     a.grad_b = grad_b;
-    // mixed precision: the classes with both l >= kMixedFp64MinL (the leading tiles of the persistent order) in FP64.
-    // With both kinds present the two launches run side by side on the plan's side streams (as the integrals), the
-    // FP64 tiles one warp each, statically.
-    const bool mixed = precision == SHG_PREC_MIXED;
-    const int hi = mixed ? p->d.mixed_fp64_tiles : p->d.n_tiles, all = p->d.n_tiles;
-    const bool fork = mixed && hi > 0 && all > hi;
-    if (fork && (r = fork_sides(p, s)) != SHG_OK) {
-        shg_plan_destroy(p);
-        return r;
-    }
-    if (e == cudaSuccess && hi > 0) {
+    // mixed precision: two launches, as exec_mixed
+    if (precision == SHG_PREC_MIXED) {
+        a.f.tile_begin = p->d.df_begin;
+        a.f.tile_end = p->d.df_end_grad;
+        a.f.counter = p->d.counter + 1;
+        if (e == cudaSuccess) e = launch_2c_grad_mixed(a, s, 128);
+        skip_df(a.f, p->d, p->d.df_end_grad, p->d.counter);
+    } else {
         a.f.tile_begin = 0;
-        a.f.tile_end = hi;
-        a.f.counter = fork ? nullptr : p->d.counter;
-        e = launch_2c_grad(a, fork ? p->d.side : s, fork ? 32 : 128);
-    }
-    if (e == cudaSuccess && all > hi) {
-        a.f.tile_begin = hi;
-        a.f.tile_end = all;
+        a.f.tile_end = p->d.n_tiles;
         a.f.counter = p->d.counter;
-        e = launch_2c_grad_mixed(a, fork ? p->d.side2 : s, 128);
     }
-    // the plan's memory is released in the order of s: join first, also after
-    // a failed launch (the other side stream may hold a running kernel)
-    if (fork) r = join_sides(p, s);
+    if (e == cudaSuccess) e = launch_2c_grad(a, s, 128);
     shg_plan_destroy(p);
-    if (r) return r;
     if (e != cudaSuccess) return fail(SHG_ECUDA, "gradient launch: %s", cudaGetErrorString(e));
     return SHG_OK;
 }

@@ -111,15 +111,9 @@ __device__ __forceinline__ void run_tile_grad(const ArgsGrad &a, const Tile &t, 
 {
     const int la = t.cls / (kLmax2c + 1), lb = t.cls % (kLmax2c + 1);
     const int J = (la < lb ? la : lb) + 1;
+    static_assert(kMixedDfMinLGrad == 3 && kMixedFp64MinL == 4, "one class of J in double-float");
     if (MIXED) {
-        // J <= 4: the classes with both l >= kMixedFp64MinL run in FP64
-        switch (J) {
-        case 1: tile_grad<MASK, MIXED, 1>(a, t, lane); break;
-        case 2: tile_grad<MASK, MIXED, 2>(a, t, lane); break;
-        case 3: tile_grad<MASK, MIXED, 3>(a, t, lane); break;
-        case 4: tile_grad<MASK, MIXED, 4>(a, t, lane); break;
-        default: break;
-        }
+        if (J == 4) tile_grad<MASK, MIXED, 4>(a, t, lane);
     } else {
         switch (J) {
         case 1: tile_grad<MASK, false, 1>(a, t, lane); break;
@@ -138,28 +132,28 @@ __global__ void __launch_bounds__(128, 4) k_2c_grad(const ArgsGrad a)
 {
     const int lane = threadIdx.x & 31;
     const ArgsFused &g = a.f;
+    if (MIXED) cudaTriggerProgrammaticLaunchCompletion();
     if (!g.counter) {
-        const int t = g.tile_begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-        if (t < g.tile_end) run_tile_grad<MASK, MIXED>(a, g.tiles[t], lane);
+        const int t = tile_at(g, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
+        if (t >= 0) run_tile_grad<MASK, MIXED>(a, g.tiles[t], lane);
         return;
     }
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(g.counter, 1);
-        t = __shfl_sync(0xffffffffu, t, 0) + g.tile_begin;
-        if (t >= g.tile_end) break;
+        t = tile_at(g, __shfl_sync(0xffffffffu, t, 0));
+        if (t < 0) break;
         run_tile_grad<MASK, MIXED>(a, g.tiles[t], lane);
         __syncwarp();
     }
+    if (!MIXED && g.beside) cudaGridDependencySynchronize();
 }
 
 template <unsigned MASK, bool MIXED>
 cudaError_t launch_grad_mask(const ArgsGrad &a, cudaStream_t s, int threads)
 {
     const int grid = pass_grid(a.f, (const void *)k_2c_grad<MASK, MIXED>, threads, 0);
-    if (grid <= 0) return cudaSuccess;
-    k_2c_grad<MASK, MIXED><<<grid, threads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_on(k_2c_grad<MASK, MIXED>, a, a.f.beside, grid, threads, s);
 }
 
 template <bool MIXED>

@@ -1,5 +1,5 @@
-// Mixed-precision gradients: radial orders as the FP64 form, angular part in double-float on the FP32 pipes (the classes
-// with both l >= kMixedFp64MinL run in FP64).
+// Mixed-precision gradients: radial orders as the FP64 form, angular part in double-float on the FP32 pipes (min(la, lb)
+// = 3; the other classes run in FP64, launch_2c_grad, beside this launch).
 #include "shg_grad2c.cuh"
 
 namespace shg {

@@ -16,11 +16,15 @@ constexpr int kJmax = 7;          // min(la, lb) + 1 <= 7
 constexpr int kRa2nMax = 5;                // largest n of the (a|r_a^{2n}|b) operator
 constexpr int kNClass = (kLmax2c + 1) * (kLmax2c + 1);
 constexpr int kTile = 32;         // pairs per warp tile
-// Two-center classes that the mixed-precision passes evaluate in FP64: both
-// la and lb >= kMixedFp64MinL (J = min(la, lb) + 1 >= 5), where the angular sums
-// cancel most (double-float carries 2^-44 of the largest term).
-constexpr int kMixedFp64MinL = 4;
-inline bool mixed_runs_fp64(int cls) { return cls / 7 >= kMixedFp64MinL && cls % 7 >= kMixedFp64MinL; }
+// Two-center classes whose angular part the mixed-precision passes evaluate in double-float: kMixedDfMinL <= min(la, lb)
+// < kMixedFp64MinL (gradients: from kMixedDfMinLGrad).  Above, the angular sums cancel too much (double-float carries 2^-44
+// of the largest term); below, the FP64 units, which are otherwise a third busy, take the few sums sooner than the FP32
+// pipes take 18 instructions for each: 1M pairs, 1/r and erfc, 2.92 ms with all classes below 4 in double-float, 2.53 ms
+// from 2 or from 3 on; 123,000 pairs, erfc, 596, 439 (from 2) and 466 us (from 3); 250,000 gradients of erfc 1.22, 1.16 and
+// 1.09 ms.
+constexpr int kMixedDfMinL = 2, kMixedDfMinLGrad = 3, kMixedFp64MinL = 4;
+inline int min_l(int cls) { return cls / 7 < cls % 7 ? cls / 7 : cls % 7; }
+inline bool mixed_runs_fp64(int cls) { return min_l(cls) < kMixedDfMinL || min_l(cls) >= kMixedFp64MinL; }
 
 // Boys function for the extended-float radial sums: from T = kFarT on the asymptotic form (relative error below 5e-18
 // for n <= 13: T^{n-1/2} e^{-T} / Gamma(n+1/2)); below, per order n = 0..kBoysOrders-1 and cell [i, i+1) / 512 of T, the Taylor coefficients c_t = F_{n+t}(T_{i+1}) / t! about the upper end of the cell, scaled by
@@ -229,22 +233,16 @@ struct PlanDev {
     const int32_t *trip_t = nullptr;                      // a~ of triples (kind 3)
     int32_t *perm = nullptr;       // device [n_pairs], pairs sorted by bin
     Tile *tiles = nullptr;         // device [n_tiles]
-    int *counter = nullptr;        // device, persistent work counter
+    int *counter = nullptr;        // device, two persistent work counters
     int n_tiles = 0;
     TileMap map;
     int class_tile_begin[kNClass + 1] = {};   // host, per-class tile ranges (class-major)
-    int mixed_fp64_tiles32 = 0;    // the same in 32-pair tiles of the map
-    int mixed_fp64_tiles = 0;      // persistent order: leading tiles of the classes that the
-                                   // mixed-precision passes run in FP64 (both l >= kMixedFp64MinL)
+    int df_begin = 0, df_end = 0, df_end_grad = 0;  // persistent order: tiles of the classes that the mixed-precision
+                                                    // passes and gradients run in double-float
     int threads = 128;             // launch shape (autotuned): threads per CTA (32, 64 or 128)
     int ctas_per_sm = 0;           // persistent CTAs per SM, 0 = occupancy limit
     int variant = 1;               // compiled variant of the fused kernels (shg_plan_2c_set_variant)
                                    // (0: free register count, 1: <= 96 registers, 5 CTAs per SM)
-    // streams of a mixed-precision pass that runs the FP64 high-l tiles beside the
-    // double-float launch (created on first use): side (highest priority) takes the
-    // FP64 launch, side2 the double-float one; the caller's stream forks and joins
-    cudaStream_t side = nullptr, side2 = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     void *owner_block = nullptr;   // device allocation holding all of the above
     cudaStream_t stream = nullptr;
 };
@@ -285,6 +283,8 @@ struct ArgsFused {
     const int32_t *perm;
     const Tile *tiles;
     int tile_begin, tile_end;
+    int skip_at = INT32_MAX, skip_n = 0;  // tiles skip_at .. skip_at + skip_n - 1 are left out (a second launch takes them)
+    bool beside = false;          // runs beside the launch before it on the stream, and ends after it
     int *counter;                 // persistent schedule (null: static)
     const long long *out_off;
     double *out[6];               // indexed by OP_OVERLAP .. OP_GCOUL

@@ -1,7 +1,7 @@
 // Mixed-precision two-center passes: the radial sums of the FP64 pass (their extended-float terms cost less than
 // double-float ones and carry more digits), the angular part in double-float on the FP32 pipes (a double-float
-// multiply-add is 18 FP32 instructions of about one cycle, an FP64 one holds its unit for 64).  The classes with both
-// l >= kMixedFp64MinL run in FP64 (launch_2c_fused); J <= 4 here.
+// multiply-add is 18 FP32 instructions of about one cycle, an FP64 one holds its unit for 64).  Only the classes for which
+// that is sooner done (kMixedDfMinL, kMixedFp64MinL); the others run in FP64 (launch_2c_fused) beside this launch.
 #pragma once
 
 #include "shg_cg_mix.cuh"
@@ -55,9 +55,8 @@ template <unsigned MASK>
 __device__ __forceinline__ void run_tile_mix(const ArgsMixFused &a, const Tile &t, int lane)
 {
     const int la = t.cls / (kLmax2c + 1), lb = t.cls % (kLmax2c + 1);
+    static_assert(kMixedDfMinL == 2 && kMixedFp64MinL == 4, "cases below");
     switch ((la < lb ? la : lb) + 1) {
-    case 1: tile_2c_mix<MASK, 1>(a, t, lane); break;
-    case 2: tile_2c_mix<MASK, 2>(a, t, lane); break;
     case 3: tile_2c_mix<MASK, 3>(a, t, lane); break;
     case 4: tile_2c_mix<MASK, 4>(a, t, lane); break;
     default: break;
@@ -69,6 +68,7 @@ __global__ void __launch_bounds__(128, MinB) k_2c_mixed_fused(const ArgsMixFused
 {
     const int lane = threadIdx.x & 31;
     const ArgsFused &g = a.f;
+    cudaTriggerProgrammaticLaunchCompletion();
     if (!g.counter) {
         const int t = g.tile_begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
         if (t < g.tile_end) run_tile_mix<MASK>(a, g.tiles[t], lane);
@@ -88,9 +88,7 @@ template <unsigned MASK, int MinB>
 cudaError_t launch_mix(const ArgsMixFused &a, cudaStream_t s, int threads, int ctas_per_sm)
 {
     const int grid = pass_grid(a.f, (const void *)k_2c_mixed_fused<MASK, MinB>, threads, ctas_per_sm);
-    if (grid <= 0) return cudaSuccess;
-    k_2c_mixed_fused<MASK, MinB><<<grid, threads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_on(k_2c_mixed_fused<MASK, MinB>, a, false, grid, threads, s);
 }
 
 }  // namespace

@@ -96,6 +96,14 @@ __device__ __forceinline__ void run_tile(const ArgsFused &g, const Tile &t, int 
     }
 }
 
+// i-th tile of a launch, or -1 past the last
+__device__ __forceinline__ int tile_at(const ArgsFused &g, int i)
+{
+    int t = g.tile_begin + i;
+    if (t >= g.skip_at) t += g.skip_n;
+    return t < g.tile_end ? t : -1;
+}
+
 // With a tile counter every warp takes tiles from it until none are left; without one (static launch) warp w of block b
 // takes tile tile_begin + b * warps_per_block + w once.  MinB: CTAs of 128 threads that must fit on an SM (a register
 // cap).
@@ -104,39 +112,60 @@ __global__ void __launch_bounds__(128, MinB) k_2c_fp64_fused(const ArgsFused g)
 {
     const int lane = threadIdx.x & 31;
     if (!g.counter) {
-        const int t = g.tile_begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-        if (t < g.tile_end) run_tile<MASK>(g, g.tiles[t], lane);
+        const int t = tile_at(g, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
+        if (t >= 0) run_tile<MASK>(g, g.tiles[t], lane);
         return;
     }
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(g.counter, 1);
-        t = __shfl_sync(0xffffffffu, t, 0) + g.tile_begin;
-        if (t >= g.tile_end) break;
+        t = tile_at(g, __shfl_sync(0xffffffffu, t, 0));
+        if (t < 0) break;
         run_tile<MASK>(g, g.tiles[t], lane);
         __syncwarp();
     }
+    if (g.beside) cudaGridDependencySynchronize();
 }
 
-// CTAs of a pass: a persistent launch takes as many as fit (or ctas_per_sm), a static one a warp per tile
+// CTAs of a pass: a static launch takes a warp per tile, a persistent one at most that and no more than fit (or
+// ctas_per_sm)
 inline int pass_grid(const ArgsFused &a, const void *kernel, int threads, int ctas_per_sm)
 {
-    if (!a.counter) return (a.tile_end - a.tile_begin + threads / 32 - 1) / (threads / 32);
+    const int all = (a.tile_end - a.tile_begin - a.skip_n + threads / 32 - 1) / (threads / 32);
+    if (!a.counter) return all;
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess || per < 1) per = 1;
     if (ctas_per_sm > 0 && ctas_per_sm < per) per = ctas_per_sm;
-    return (sms > 0 ? sms : 1) * per;
+    per *= sms > 0 ? sms : 1;
+    return per < all ? per : all;
+}
+
+// Launch of a pass.  One that runs beside the launch before it starts when the CTAs of that launch are all resident or
+// done (they announce it at their start) and waits for its end before it ends itself, so that later work of the stream is
+// ordered after both; nothing of the one is read by the other.
+template <typename A>
+cudaError_t launch_on(void (*kernel)(const A), const A &a, bool beside, int grid, int threads, cudaStream_t s)
+{
+    if (grid <= 0) return cudaSuccess;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = beside ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, a);
 }
 
 template <unsigned MASK, int MinB>
 cudaError_t launch_pass(const ArgsFused &a, cudaStream_t s, int threads, int ctas_per_sm)
 {
     const int grid = pass_grid(a, (const void *)k_2c_fp64_fused<MASK, MinB>, threads, ctas_per_sm);
-    if (grid <= 0) return cudaSuccess;
-    k_2c_fp64_fused<MASK, MinB><<<grid, threads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_on(k_2c_fp64_fused<MASK, MinB>, a, a.beside, grid, threads, s);
 }
 
 }  // namespace
