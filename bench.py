@@ -534,9 +534,9 @@ def run_ours(args, rank, world):
                      "algorithmic_flops_per_step": flops_step, "kernel_ms_per_step": kern_ms,
                      "far_field_primitive_pairs": (int(n_far.sum()) if n_far is not None else None),
                      "separate_passes_flops_per_step": flops_separate,
-                     "kernel": ("k_2c_%s_fused_persistent (1/r and erfc in one pass)" %
+                     "kernel": ("k_2c_%s_fused<1/r, erfc> (one pass)" %
                                 ("fp64" if args.precision == "fp64" else "mixed") if fused else
-                                "k_2c_%s_persistent<op> / static (one launch per operator)" %
+                                "k_2c_%s_fused<op> (one launch per operator)" %
                                 ("fp64" if args.precision == "fp64" else "mixed"))},
         "forms": forms,
         "e2e": {"value": job_units / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d,

@@ -68,12 +68,13 @@ enum shg_operator {
 
 enum shg_precision {
     SHG_PREC_FP64 = 0,  /* every step in FP64                                     */
-    SHG_PREC_MIXED = 1  /* FP32-based compensated arithmetic, FP64 where needed:
-                           two-center passes evaluate the classes with both la
-                           and lb >= 4 in FP64 (their sum over j of Eq.
-                           final_r12int_ab cancels beyond double-float reach),
-                           every other class in double-float; the FP64 far
-                           field of 1/r (T >= 120) is summed on the FP64 pipe */
+    SHG_PREC_MIXED = 1  /* FP32-based compensated arithmetic where it is the
+                           faster form: the angular part of the classes with
+                           min(la, lb) = 2 or 3 (gradients: 3) in double-float;
+                           the other classes as in FP64 (with both la and
+                           lb >= 4 the sum over j of Eq. final_r12int_ab
+                           cancels beyond double-float reach), and all radial
+                           sums as in FP64                                     */
 };
 
 enum shg_schedule {
@@ -204,13 +205,15 @@ int shg_plan_2c_exec(shg_plan_t *plan, int op, double omega, double screen_thres
  */
 int shg_plan_2c_set_variant(shg_plan_t *plan, int variant);
 
-/* Number of kernel launches one FP64 shg_plan_2c_exec (or fused pass) issues
- * (for accounting). */
+/* Number of kernel launches one FP64 shg_plan_2c_exec (or fused pass over a
+ * list of more than about 30,000 pairs; a shorter one may issue one per
+ * operator) issues (for accounting). */
 int shg_plan_launches(const shg_plan_t *plan);
 
 /* Number of kernel launches one execution of the plan issues in `precision`
- * (SHG_PREC_MIXED adds the FP64 launch of the classes with both l >= 4 to a
- * persistent plan that holds any); -1 for a NULL plan or bad precision. */
+ * (SHG_PREC_MIXED: the double-float launch of the classes with
+ * min(la, lb) = 2 or 3 and the FP64 launch of the others, where a persistent
+ * plan holds any); -1 for a NULL plan or bad precision. */
 int shg_plan_launches_prec(const shg_plan_t *plan, int precision);
 
 /*
@@ -246,8 +249,9 @@ void shg_graph_destroy(shg_graph_t *graph);
  * is formed as 1/r - erf(wr)/r, and erf and erfc with the same omega share
  * one attenuated sum.  Results agree with shg_plan_2c_exec of each operator
  * up to the order of the floating-point sums.  SHG_PREC_MIXED runs the same
- * scheme in double-float (each block sum of Q_j a compensated dot product);
- * its accuracy bar is that of the mixed single-operator pass.
+ * scheme with the mixed angular part; its accuracy bar is that of the mixed
+ * single-operator pass.  A short list (at most 1,024 tiles over all operators)
+ * runs as one launch per operator, all side by side.
  *   ops[n_ops], omegas[n_ops]  host arrays, 1 <= n_ops <= 5; each of
  *                  SHG_OP_OVERLAP, SHG_OP_COULOMB, SHG_OP_ERFC, SHG_OP_ERF,
  *                  SHG_OP_GAUSS at most once; omega rules of shg_eval_2c
@@ -272,9 +276,7 @@ int shg_graph_2c_create_fused(shg_plan_t *plan, int n_ops, const int *ops, const
  * released in the order of the stream the plan was created on
  * (cudaFreeAsync), without a host synchronisation: executions queued on that
  * stream finish first, and executions on another stream must be ordered
- * before it by the caller (an event that stream waits for).  The side streams
- * and events of mixed-precision executions are destroyed with the plan; the
- * executions have already joined them into the caller's stream.
+ * before it by the caller (an event that stream waits for).
  */
 void shg_plan_destroy(shg_plan_t *plan);
 
@@ -340,13 +342,13 @@ int shg_eval_3c_aab_grad(const shg_basis_t *orb, const shg_basis_t *aux, int64_t
  * memory during the call.  The paper has no counterpart: this is a property
  * of the library, not of the integral scheme.
  *
- * shg_eval_2c allocates its plan (the bucketed pair list and tile list) with
- * cudaMallocAsync.  Some callers cannot allow that at call time: a framework
+ * shg_eval_2c allocates its plan (the bucketed pair list and tile list) from
+ * the library's stream-ordered pool.  Some callers cannot allow that at call time: a framework
  * that hands out device memory only from its own pool, a real-time loop that
  * must not pay allocation latency or its implicit synchronisation, a process
  * that has reserved all device memory up front.  This entry point builds the
  * same plan in a fixed array inside the library (a file-scope __device__
- * array of about 10.5 MB that every GPU loading the library keeps until the
+ * array of about 11.3 MB that every GPU loading the library keeps until the
  * process exits) and calls no cudaMalloc, cudaFree or other allocating
  * routine.  Results equal those of shg_eval_2c with the persistent schedule.
  *   arguments      as shg_eval_2c (no screening threshold); FP64 and the

@@ -3,8 +3,8 @@
 Candidates: schedule (one launch per class, or one persistent launch with
 tiles in decreasing estimated cost), threads per CTA (1, 2 or 4 warps, each
 warp owning a class-pure tile of up to 32 pairs), persistent CTAs per SM and,
-for the double-float fused pass, the compiled kernel variant (register count
-left to the compiler, or capped for one more resident CTA per SM).
+for the fused passes, the compiled kernel variant (register caps, see
+shg_plan_2c_set_variant).
 Each candidate runs the requested operators a few times (CUDA events, after a
 warm-up); the fastest is cached in a JSON file keyed by GPU name, precision,
 operators and a signature of the workload's (la, lb, Ka*Kb) histogram.

@@ -36,7 +36,8 @@ def os_contracted_elements(l_a, l_b, k_a, k_b, gradients=False):
 # --------------------------------------------------------------------------- #
 _BOYS = 2 * 8 + 2 * 8 + 1          # Taylor of F_kmax (8 fma), exp Taylor (8 fma), scale by exp(-T_i)
 _BOYS_F = 2 * 8                     # Taylor of F_kmax alone: J = 1 needs no exp(-T) (no recursion)
-KBOYS_TMAX = 120.0                  # T = rho R^2 at and above which the fused 1/r sum takes the far field
+KBOYS_TMAX = 120.0                  # T = rho R^2 at and above which a primitive pair of the 1/r sum counts as one
+                                    # multiply-add (the far field; the kernels take it from 72 on)
 
 
 def _boys(J):

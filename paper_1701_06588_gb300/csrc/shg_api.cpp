@@ -1252,10 +1252,66 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
     return SHG_OK;
 }
 
-// Most tiles that a persistent plan runs with one CTA each instead of a work counter: all of them are resident at once (8
-// warps or more per SM), spread over the SMs one by one, without the launch that clears the counter (63 tiles of 2,000
-// pairs, overlap and 1/r: 102 us persistent with four-warp CTAs, 95 us with one-warp CTAs)
+// Most tiles that a pass of a persistent plan runs with one CTA each instead of a work counter: all of them are resident at
+// once (8 warps or more per SM), spread over the SMs one by one, without the launch that clears the counter (63 tiles of
+// 2,000 pairs, overlap and 1/r: 102 us persistent with four-warp CTAs, 95 us with one-warp CTAs)
 constexpr int kStaticTiles = 1024;
+
+// Radial sums of one operator
+static unsigned want_of(int op)
+{
+    switch (op) {
+    case SHG_OP_OVERLAP: return kSumOv;
+    case SHG_OP_COULOMB: return kSumCo;
+    case SHG_OP_ERFC: return kSumCo | kSumX;
+    case SHG_OP_ERF: return kSumEr;
+    case SHG_OP_GAUSS: return kSumGa;
+    default: return kSumGc;
+    }
+}
+
+// Pass over a list of at most kStaticTiles tiles.  With few enough they leave most warp slots empty, so each operator gets
+// a launch of its own, all side by side (1/r and erfc, which share their sums, together): 2,000 pairs of short
+// contractions, overlap and 1/r, 101 us in one launch, 74 in two; five operators 170 and 107 us.  Beyond the limit the
+// common work of one launch tells (10,000 pairs, five operators: 174 and 234 us).  The kernels of one operator and of
+// several give the same bits.
+static int exec_short(shg_plan_t *p, const ArgsFused &f, bool mixed, cudaStream_t s)
+{
+    const bool pair = f.out[SHG_OP_COULOMB] && f.out[SHG_OP_ERFC];
+    int n = 0;
+    for (int op = 0; op < 6; ++op) n += f.out[op] && !(pair && op == SHG_OP_ERFC);
+    const bool split = n > 1 && n * p->d.n_tiles <= kStaticTiles;
+    ArgsMixFused m;
+    if (mixed) fill_kappa_mix(m.kappa);
+    bool beside = false;
+    for (int op = 0; op < 6; ++op) {
+        if (!f.out[op] || (pair && op == SHG_OP_ERFC)) continue;
+        ArgsFused a = f;
+        if (split) {
+            for (int i = 0; i < 6; ++i)
+                if (i != op && !(pair && op == SHG_OP_COULOMB && i == SHG_OP_ERFC)) a.out[i] = nullptr;
+            a.r.want = want_of(a.out[SHG_OP_ERFC] ? SHG_OP_ERFC : op);
+        }
+        a.counter = nullptr;
+        a.tile_begin = 0;
+        a.tile_end = p->d.n_tiles;
+        if (mixed && p->d.df_end > p->d.df_begin) {
+            m.f = a;
+            m.f.tile_begin = p->d.df_begin;
+            m.f.tile_end = p->d.df_end;
+            m.f.beside = beside;
+            SHG_CUDA(launch_2c_mixed(m, s, 32, 0, p->d.variant));
+            beside = true;
+            a.skip_at = p->d.df_begin;
+            a.skip_n = p->d.df_end - p->d.df_begin;
+        }
+        a.beside = beside;
+        if (a.tile_end > a.skip_n) SHG_CUDA(launch_2c_fused(a, s, 32, 0, p->d.variant));
+        beside = beside || a.tile_end > a.skip_n;
+        if (!split) break;
+    }
+    return SHG_OK;
+}
 
 // FP64 pass over the tiles of a plan
 static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, cudaStream_t s)
@@ -1263,11 +1319,7 @@ static int exec_fused_fp64(shg_plan_t *p, ArgsFused &a, cudaStream_t s)
     if (p->d.schedule == SHG_SCHED_PERSISTENT) {
         a.tile_begin = 0;
         a.tile_end = p->d.n_tiles;
-        if (a.tile_end <= kStaticTiles) {
-            a.counter = nullptr;
-            SHG_CUDA(launch_2c_fused(a, s, 32, 0, p->d.variant));
-            return SHG_OK;
-        }
+        if (a.tile_end <= kStaticTiles) return exec_short(p, a, false, s);
         SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, sizeof(int), s));
         a.counter = p->d.counter;
         SHG_CUDA(launch_2c_fused(a, s, p->d.threads, p->d.ctas_per_sm, p->d.variant));
@@ -1304,6 +1356,7 @@ static int exec_mixed(shg_plan_t *p, const ArgsFused &f, cudaStream_t s)
     fill_kappa_mix(m.kappa);
     ArgsFused a = f;
     if (p->d.schedule == SHG_SCHED_PERSISTENT) {
+        if (p->d.n_tiles <= kStaticTiles) return exec_short(p, f, true, s);
         SHG_CUDA(cudaMemsetAsync(p->d.counter, 0, 2 * sizeof(int), s));
         m.f.tile_begin = p->d.df_begin;
         m.f.tile_end = p->d.df_end;
@@ -1543,8 +1596,7 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     double *none = nullptr;
     fused_ops(a.f, 1, &op, &omega, &none);
     // fused_ops reads the wanted sums off the outputs
-    a.f.r.want = op == SHG_OP_OVERLAP ? kSumOv : op == SHG_OP_COULOMB ? kSumCo : op == SHG_OP_ERFC ? kSumCo | kSumX
-                 : op == SHG_OP_ERF ? kSumEr : op == SHG_OP_GAUSS ? kSumGa : kSumGc;
+    a.f.r.want = want_of(op);
     fused_plan(a.f, basis->d, p->d, *t, w_off);
     fill_kappa_mix(a.kappa);
     a.w = w;

@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(128, 4) k_2c_grad(const ArgsGrad a)
     if (!g.counter) {
         const int t = tile_at(g, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
         if (t >= 0) run_tile_grad<MASK, MIXED>(a, g.tiles[t], lane);
+        if (!MIXED && g.beside) cudaGridDependencySynchronize();
         return;
     }
     for (;;) {

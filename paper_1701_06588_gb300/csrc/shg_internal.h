@@ -241,8 +241,7 @@ struct PlanDev {
                                                     // passes and gradients run in double-float
     int threads = 128;             // launch shape (autotuned): threads per CTA (32, 64 or 128)
     int ctas_per_sm = 0;           // persistent CTAs per SM, 0 = occupancy limit
-    int variant = 1;               // compiled variant of the fused kernels (shg_plan_2c_set_variant)
-                                   // (0: free register count, 1: <= 96 registers, 5 CTAs per SM)
+    int variant = 1;               // register cap of the kernels (shg_plan_2c_set_variant)
     void *owner_block = nullptr;   // device allocation holding all of the above
     cudaStream_t stream = nullptr;
 };
@@ -391,7 +390,7 @@ int slot_doubles_3c_grad(int cls);
 cudaError_t launch_2c_grad(const ArgsGrad &args, cudaStream_t s, int threads);
 cudaError_t launch_2c_grad_mixed(const ArgsGrad &args, cudaStream_t s, int threads);
 cudaError_t launch_2c_grad_ra2n(const Args2c &args, cudaStream_t s);
-// mixed-precision pass of the classes with min(la, lb) < kMixedFp64MinL (arguments as launch_2c_fused)
+// double-float part of a mixed-precision pass, kMixedDfMinL <= min(la, lb) < kMixedFp64MinL (arguments as launch_2c_fused)
 cudaError_t launch_2c_mixed(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
 cudaError_t launch_2c_mixed_all(const ArgsMixFused &args, cudaStream_t s, int threads, int ctas_per_sm, int variant);
 cudaError_t launch_2c(const Args2c &args, int op, int precision, int n_tiles_or_grid, bool persistent,

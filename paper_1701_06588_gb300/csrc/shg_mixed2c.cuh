@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(128, MinB) k_2c_mixed_fused(const ArgsMixFused
     if (!g.counter) {
         const int t = g.tile_begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
         if (t < g.tile_end) run_tile_mix<MASK>(a, g.tiles[t], lane);
+        if (g.beside) cudaGridDependencySynchronize();
         return;
     }
     for (;;) {
@@ -82,13 +83,14 @@ __global__ void __launch_bounds__(128, MinB) k_2c_mixed_fused(const ArgsMixFused
         run_tile_mix<MASK>(a, g.tiles[t], lane);
         __syncwarp();
     }
+    if (g.beside) cudaGridDependencySynchronize();
 }
 
 template <unsigned MASK, int MinB>
 cudaError_t launch_mix(const ArgsMixFused &a, cudaStream_t s, int threads, int ctas_per_sm)
 {
     const int grid = pass_grid(a.f, (const void *)k_2c_mixed_fused<MASK, MinB>, threads, ctas_per_sm);
-    return launch_on(k_2c_mixed_fused<MASK, MinB>, a, false, grid, threads, s);
+    return launch_on(k_2c_mixed_fused<MASK, MinB>, a, a.f.beside, grid, threads, s);
 }
 
 }  // namespace

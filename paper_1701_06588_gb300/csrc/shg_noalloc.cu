@@ -6,11 +6,11 @@
 // is handed out only by its own pool, a real-time loop that has to avoid the
 // implicit synchronisation and latency of allocation, or a host that has
 // already reserved all device memory.  shg_eval_2c builds its plan in memory
-// from cudaMallocAsync; this variant builds the same plan (pair bucketing and
+// from a stream-ordered pool; this variant builds the same plan (pair bucketing and
 // tile list) in a fixed device array that belongs to the library instead.
 //
 // The array is a file-scope __device__ variable, so every GPU that loads this
-// library keeps it (kNoAllocBytes, about 10.5 MB) until the process exits.
+// library keeps it (kNoAllocBytes, about 11.3 MB) until the process exits.
 // Host code cannot use its name as a device address; the address is taken
 // with cudaGetSymbolAddress once per device, on the first call made on that
 // device (so that first call should not be made while a stream is being

@@ -111,9 +111,11 @@ template <unsigned MASK, int MinB>
 __global__ void __launch_bounds__(128, MinB) k_2c_fp64_fused(const ArgsFused g)
 {
     const int lane = threadIdx.x & 31;
+    cudaTriggerProgrammaticLaunchCompletion();
     if (!g.counter) {
         const int t = tile_at(g, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
         if (t >= 0) run_tile<MASK>(g, g.tiles[t], lane);
+        if (g.beside) cudaGridDependencySynchronize();
         return;
     }
     for (;;) {
