@@ -36,10 +36,10 @@ WORKLOAD = "c3_2m_l6_k20"
 OPS = [("coulomb", 1, 0.0), ("erfc", 2, 0.11)]
 DF_FMA_FP32_INSTR = 18.0       # FP32 instructions of one double-float multiply-add
 FP64_NOMINAL_TFLOPS = 1.25   # 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (nominal, context)
-PROFILES = {"fp64_fused": os.path.join(ROOT, "profiles", "k_2c_fp64_fused_persistent_c3_2m.txt"),
-            "mixed_fused": os.path.join(ROOT, "profiles", "k_2c_mixed_fused_persistent_c3_2m.txt"),
-            "fp64": os.path.join(ROOT, "profiles", "k_2c_fp64_persistent_c3_2m.txt"),
-            "mixed": os.path.join(ROOT, "profiles", "k_2c_mixed_persistent_c3_2m.txt")}
+PROFILES = {"fp64_fused": os.path.join(ROOT, "profiles", "k_2c_fp64_fused_c3_2m.txt"),
+            "mixed_fused": os.path.join(ROOT, "profiles", "k_2c_mixed_fused_c3_2m.txt"),
+            "fp64": os.path.join(ROOT, "profiles", "k_2c_fp64_single_c3_2m.txt"),
+            "mixed": os.path.join(ROOT, "profiles", "k_2c_mixed_single_c3_2m.txt")}
 
 
 def parse():
@@ -711,7 +711,7 @@ def other_configs(args):
         "algorithmic_tflops": f3 / (ms * 1e-3) / 1e12}}
     ms = _events_ms(lambda: L.shg_eval_3c_aab(b.handle, b.handle, len(ta), d_ta, d_tt, d_tb, 1, 0.0, d_off, out, st), 3)
     res["c4_aab_20k"]["mixed"] = {"ms_per_pass": ms, "triples_per_s": len(ta) / (ms * 1e-3),
-                                  "form": "radial sums FP64, angular part and Gaunt sum double-float"}
+                                  "form": "as FP64"}
     w = torch.empty(total, dtype=torch.float64, device="cuda").uniform_(-1, 1)
     ga = torch.empty((len(ta), 3), dtype=torch.float64, device="cuda")
     gb = torch.empty((len(ta), 3), dtype=torch.float64, device="cuda")

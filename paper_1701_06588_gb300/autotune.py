@@ -2,9 +2,8 @@
 
 Candidates: schedule (one launch per class, or one persistent launch with
 tiles in decreasing estimated cost), threads per CTA (1, 2 or 4 warps, each
-warp owning a class-pure tile of up to 32 pairs), persistent CTAs per SM and,
-for the fused passes, the compiled kernel variant (register caps, see
-shg_plan_2c_set_variant).
+warp owning a class-pure tile of up to 32 pairs), persistent CTAs per SM, and
+the compiled kernel variant (register caps, see shg_plan_2c_set_variant).
 Each candidate runs the requested operators a few times (CUDA events, after a
 warm-up); the fastest is cached in a JSON file keyed by GPU name, precision,
 operators and a signature of the workload's (la, lb, Ka*Kb) histogram.
@@ -21,7 +20,7 @@ from . import api
 
 CANDIDATES = ([("per_class", t, 0) for t in (32, 64, 128)] +
               [("persistent", t, c) for t in (32, 64, 128) for c in (0, 1, 2, 4, 8)])
-VARIANTS = {"mixed_fused": (0, 1, 2), "fp64_fused": (0, 1, 2)}
+VARIANTS = dict.fromkeys(("fp64", "mixed", "fp64_fused", "mixed_fused"), (0, 1, 2))
 
 
 def cache_path():
