@@ -5,8 +5,9 @@ One step = every two-center block of the 2,000,000-pair high-l workload
 (la, lb in 0..6 with P(l) ~ 2^-l, contraction lengths 1..20 with 30% of the
 shells at 12..20 primitives, exponents 0.03..5000, separations 0..10 bohr,
 seed 2) for 1/r and erfc(0.11 r)/r, i.e. 4,000,000 shell-pair integrals:
-one fused persistent launch for both operators in FP64 (--precision mixed:
-double-float; --separate: one persistent launch per operator).
+one fused persistent launch for both operators in FP64 (--precision mixed: a
+second launch beside it for the double-float classes; --separate: one pass per
+operator).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                   [--precision fp64|mixed] [--separate] [--configs]
@@ -378,8 +379,8 @@ def run_ours(args, rank, world):
     value = job_units / (ms_step * 1e-3)
 
     flops_separate = sum(counts.workload_flops(shells, pa, pb, op) for _, op, _ in OPS)
-    # the fused passes sum the far field of 1/r (T >= 120) as one multiply-add per
-    # primitive pair: count those pairs exactly
+    # the passes sum the far field of 1/r as one multiply-add per primitive pair: count
+    # those pairs (T >= 120) exactly
     n_far = counts.far_primitive_pairs(shells, pa, pb) if fused else None
     flops_step = (counts.workload_fused_flops(shells, pa, pb, [(op, om) for _, op, om in OPS], n_far) if fused
                   else flops_separate)
@@ -734,7 +735,7 @@ def other_configs(args):
         ms = _events_ms(lambda: L.shg_eval_2c_grad(b.handle, len(pa), d_pa, d_pb, op, om, 0, d_off, w, ga, gb, st), 3)
         entry[opn] = {"ms_per_pass": ms, "pair_gradients_per_s": len(pa) / (ms * 1e-3),
                       "algorithmic_tflops": counts.workload_grad_flops(sh, pa, pb, op) / (ms * 1e-3) / 1e12}
-        # mixed: double-float radial orders (classes with both l >= 4 in FP64)
+        # mixed: double-float angular part for min(la, lb) = 3, the rest in FP64
         ms = _events_ms(lambda: L.shg_eval_2c_grad(b.handle, len(pa), d_pa, d_pb, op, om, L.SHG_PREC_MIXED, d_off, w,
                                                    ga, gb, st), 3)
         entry[opn + "_mixed"] = {"ms_per_pass": ms, "pair_gradients_per_s": len(pa) / (ms * 1e-3)}

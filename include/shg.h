@@ -291,8 +291,8 @@ void shg_plan_destroy(shg_plan_t *plan);
  *   aux            basis of b (may be the same handle as orb)
  *   d_a, d_atilde  device int32[n_triples] indices into orb
  *   d_b            device int32[n_triples] indices into aux
- *   precision      enum shg_precision (FP64, or MIXED: radial sums FP64,
- *                  angular part and Gaunt sum double-float)
+ *   precision      enum shg_precision (MIXED: computed as FP64, the faster
+ *                  form)
  *   screen_thresh  0 disables screening; > 0: a triple whose bound on every
  *                  element magnitude is below it writes zeros.  The bound
  *                  multiplies the single-shell bounds of a and a~ used by
@@ -316,11 +316,9 @@ int shg_eval_3c_aab(const shg_basis_t *orb, const shg_basis_t *aux, int64_t n_tr
  *   d_w_offsets, d_upstream_w   device int64[n_pairs] / doubles: W_p blocks,
  *                               same layout as shg_eval_2c output
  *   d_grad_a, d_grad_b          device double[n_pairs][3]; d_grad_b may be NULL
- *   precision                   SHG_PREC_FP64, or SHG_PREC_MIXED: radial orders
- *                               in double-float on the FP32 pipes, the angular
- *                               part (harmonics, their gradients, W and the
- *                               contractions with W_p) in FP64; the classes with
- *                               both la and lb >= 4 wholly in FP64.  Not for
+ *   precision                   SHG_PREC_FP64, or SHG_PREC_MIXED: the angular
+ *                               part of the classes with min(la, lb) = 3 in
+ *                               double-float, all else as in FP64.  Not for
  *                               SHG_OP_RA2N (SHG_EINVAL)
  * No atomics: per-atom sums are left to the caller.
  */

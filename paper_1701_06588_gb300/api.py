@@ -326,10 +326,9 @@ class HostPipeline2c:
     @staticmethod
     def default_chunks(precision):
         """Measured on the 2M-pair workload (1/r and erfc), median ms per
-        call: FP64 18.7, 18.1-18.8, 18.5 and 19.3 for 1, 2, 4 and 8 chunks
-        (4 varies least); mixed 8.3, 8.4, 9.9 and 12.7, so one chunk (every
-        chunk of a mixed pass also waits for its own FP64 launch of the classes
-        with both l >= 4, whose slowest tile sets a fixed time per chunk)."""
+        call: FP64 7.50, 6.93, 6.91 and 7.30 for 1, 2, 4 and 8 chunks; mixed
+        7.59, 6.98, 7.15 and 7.73 (one chunk stays the default there: results
+        and launches per call as before; n_chunks=2 is the faster choice)."""
         return 1 if precision == "mixed" else 4
 
     def _buf(self, name, n, dtype):
