@@ -71,6 +71,17 @@ SHG_HD double bitsd(uint64_t v)
 #endif
 }
 
+SHG_HD uint32_t fbits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    uint32_t v;
+    std::memcpy(&v, &x, sizeof v);
+    return v;
+#endif
+}
+
 // product of two normalised xf: the raw significand is in [2^60, 2^62); one shift by 1 or 2 normalises it
 SHG_HD xf mul(xf a, xf b)
 {
@@ -157,24 +168,22 @@ __device__ __forceinline__ float seed_rsqrt(float x)
 }
 #endif
 
-// 1 / sqrt(a), a normalised: FP32 seed y0 (2^-22), then y0 (1 + h), h = e/2 + 3 e^2/8, e = 1 - f y0^2 (error 2^-65),
-// in fixed point.  a = f 2^(2 h2), f = M 2^-61 in [1, 4).
-SHG_XF_LONG xf rsqrt(xf a)
+// 24-bit fraction y0 2^24 of the seed y0 2^-14 of 1 / sqrt(f), f in [1, 4): y0 in [1/2, 1).  Read off the float's bits as
+// an offset from those of 2^-15, not as its mantissa: the approximation may fall an ulp or two short of 2^-15 for f just
+// below 4 (its error bound is 2^-22.9), and the mantissa of such a float stands for almost twice its value.  Below 2^-15 the
+// offset counts half units, so it gives at most 2^-25 less than the float per ulp: within the step's range.
+SHG_HD uint32_t seed_fraction(float r)
 {
-    const int odd = (a.e + 61) & 1;                                          // 1: shift the significand down once
-    const uint64_t M = a.m >> odd;
-    const int h2 = (a.e + 61 + odd) >> 1;
-    // r = 2^-14 / sqrt(f), from the upper word f 2^29; Y0 = its 24-bit significand, y0 = Y0 2^-24 in [1/2, 1)
-#ifdef __CUDA_ARCH__
-    float r = seed_rsqrt((float)hi32(M) * 0.5f);
     r = fminf(r, 6.1035152e-05f);                                            // the float below 2^-14
-    const uint32_t Y0 = (__float_as_uint(r) & 0x7fffffu) | 0x800000u;
-#else
-    uint32_t Y0 = (uint32_t)(16777216.0 / std::sqrt((double)hi32(M) / 536870912.0));
-    Y0 = Y0 > 0xffffffu ? 0xffffffu : Y0;
-#endif
+    return fbits(r) - (0x38000000u - 0x800000u);
+}
+
+// y0 (1 + h) 2^-h2 = 1 / sqrt(f 2^(2 h2)), f = M 2^-61 in [1, 4), from its seed, in fixed point: h = e/2 + 3 e^2/8,
+// e = 1 - f y0^2 (|e| < 2^-20.5, two ulps of the seed; the dropped 5 e^3/16 is then 2^-63)
+SHG_HD xf rsqrt_step(uint64_t M, int h2, uint32_t Y0)
+{
     const uint64_t S = ((uint64_t)Y0 * Y0) << 15;                            // y0^2 2^63
-    const int64_t e = (int64_t)((1ull << 60) - mulhi(M, S)) - 1;             // units 2^-60, |e| < 2^39
+    const int64_t e = (int64_t)((1ull << 60) - mulhi(M, S)) - 1;             // units 2^-60, |e| < 2^39.5
     const int32_t es = (int32_t)(e >> 9);
     const int32_t e2 = (int32_t)(((int64_t)es * es) >> 32);                  // units 2^-70
     const int64_t h = (e >> 1) + ((e2 * 3) >> 13);
@@ -184,6 +193,21 @@ SHG_XF_LONG xf rsqrt(xf a)
     uint64_t Y = ((uint64_t)(Y0 << 7) << 32) + (uint64_t)yh;
     if (Y >> 63) Y = 0x7fffffffffffffffull;                                  // y = 1
     return xf{Y, -63 - h2};
+}
+
+// 1 / sqrt(a), a normalised: FP32 seed (2^-22) and one step of third order
+SHG_XF_LONG xf rsqrt(xf a)
+{
+    const int odd = (a.e + 61) & 1;                                          // 1: shift the significand down once
+    const uint64_t M = a.m >> odd;
+    // the seed from the upper word f 2^29
+    const float x = (float)hi32(M) * 0.5f;
+#ifdef __CUDA_ARCH__
+    const float r = seed_rsqrt(x);
+#else
+    const float r = (float)(1.0 / std::sqrt((double)x));
+#endif
+    return rsqrt_step(M, (a.e + 61 + odd) >> 1, seed_fraction(r));
 }
 
 // ------------------------------------------------------------------------- //
