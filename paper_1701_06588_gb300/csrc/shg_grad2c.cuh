@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(128, 4) k_2c_grad(const ArgsGrad a)
     const ArgsFused &g = a.f;
     if (MIXED) cudaTriggerProgrammaticLaunchCompletion();
     if (!g.counter) {
-        const int t = tile_at(g, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
+        const int t = tile_at(g, launch_warp(blockIdx.x, blockDim.x, threadIdx.x));
         if (t >= 0) run_tile_grad<MASK, MIXED>(a, g.tiles[t], lane);
         if (!MIXED && g.beside) cudaGridDependencySynchronize();
         return;

@@ -300,7 +300,7 @@ __device__ __forceinline__ void run_tile_fp64(const Args2c &g, int op, int t, in
 template <int OP>
 __global__ void __launch_bounds__(128) k_2c_fp64_static(const Args2c g)
 {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int warp = launch_warp(blockIdx.x, blockDim.x, threadIdx.x);
     const int lane = threadIdx.x & 31;
     const int t = g.tile_begin + warp;
     if (t >= g.tile_end) return;

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(128, MinB) k_2c_mixed_fused(const ArgsMixFused
     const ArgsFused &g = a.f;
     cudaTriggerProgrammaticLaunchCompletion();
     if (!g.counter) {
-        const int t = g.tile_begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+        const int t = g.tile_begin + launch_warp(blockIdx.x, blockDim.x, threadIdx.x);
         if (t < g.tile_end) run_tile_mix<MASK>(a, g.tiles[t], lane);
         if (g.beside) cudaGridDependencySynchronize();
         return;

@@ -8,6 +8,7 @@
 #pragma once
 
 #include "shg_cg.cuh"
+#include "shg_tilemap.cuh"
 #include "shg_xradial.cuh"
 
 namespace shg {
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(128, MinB) k_2c_fp64_fused(const ArgsFused g)
     const int lane = threadIdx.x & 31;
     cudaTriggerProgrammaticLaunchCompletion();
     if (!g.counter) {
-        const int t = tile_at(g, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
+        const int t = tile_at(g, launch_warp(blockIdx.x, blockDim.x, threadIdx.x));
         if (t >= 0) run_tile<MASK>(g, g.tiles[t], lane);
         if (g.beside) cudaGridDependencySynchronize();
         return;
