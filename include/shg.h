@@ -178,6 +178,14 @@ int shg_eval_2c(const shg_basis_t *basis, int64_t n_pairs, const int32_t *d_pair
  * list and the l and K of the shells, not on centers, exponents or operator.
  * Validates the shell indices on the device and synchronises `stream` once.
  * d_pair_a/b must stay valid and unchanged for the plan's lifetime.
+ *
+ * Plans (also those inside shg_eval_2c, the gradient and the (aab) calls) come
+ * from a stream-ordered memory pool of the library, one per device.  While the
+ * device has a basis or a plan the pool keeps up to 256 MB of freed memory for
+ * the next plan; that memory belongs to no other pool and other allocators
+ * cannot use it.  When the last basis and plan of the device are destroyed it
+ * is given back: what is free at once, what a stream still holds at the first
+ * synchronisation after its release.
  */
 int shg_plan_2c_create(const shg_basis_t *basis, int64_t n_pairs, const int32_t *d_pair_a,
                        const int32_t *d_pair_b, int schedule, void *stream, shg_plan_t **out);
@@ -437,6 +445,14 @@ int shg_reduce_centers(const shg_basis_t *basis, int64_t n_pairs, const int32_t 
  * d_T[n_T] writes F_n for n = 0..nmax (nmax <= 24) to d_F[i*(nmax+1) + n].
  */
 int shg_debug_boys(int64_t n_T, const double *d_T, int nmax, double *d_F, void *stream);
+
+/*
+ * shg_debug_pool - bytes of the current device's plan pool (see
+ * shg_plan_2c_create): reserved from the system, in use by plans, and the
+ * most that was in use since the last call with reset_high != 0 (all 0 before
+ * the first basis).
+ */
+int shg_debug_pool(int reset_high, uint64_t *reserved, uint64_t *used, uint64_t *used_high);
 
 /*
  * shg_measure_alu_peak - ALU throughput probe: a grid of independent FMA

@@ -59,6 +59,7 @@ SIGNATURES = [
     ("shg_gather_2c", _I, [_P, _L, _P, _P, _P, _P, _P, _L, _I, _P, _P]),
     ("shg_reduce_centers", _I, [_P, _L, _P, _P, _P, _P, _P, _P]),
     ("shg_debug_boys", _I, [_L, _P, _I, _P, _P]),
+    ("shg_debug_pool", _I, [_I, _P, _P, _P]),
     ("shg_measure_alu_peak", _I, [_I, _I, ctypes.POINTER(_D), _P]),
     ("shg_last_error", ctypes.c_char_p, []),
     ("shg_version", ctypes.c_char_p, []),
@@ -274,6 +275,13 @@ def shg_reduce_centers(basis, n, d_pa, d_pb, d_grad_a, d_grad_b, d_center_grad, 
 
 def shg_debug_boys(n, d_T, nmax, d_F, stream):
     return check(load().shg_debug_boys(n, _ptr(d_T), nmax, _ptr(d_F), stream))
+
+
+def shg_debug_pool(reset_high=False):
+    """(reserved, in use, most in use) bytes of the current device's plan pool."""
+    v = [ctypes.c_uint64() for _ in range(3)]
+    check(load().shg_debug_pool(int(reset_high), *[ctypes.addressof(x) for x in v]))
+    return tuple(int(x.value) for x in v)
 
 
 def shg_measure_alu_peak(kind, iters, stream):

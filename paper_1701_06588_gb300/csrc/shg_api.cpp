@@ -354,7 +354,7 @@ struct DevState {
     int *bin_rank[2] = {nullptr, nullptr};   // [2 * kNBins]: rank of bin, then bin of rank
     int *bin_rank3 = nullptr;                // [2 * kNBins3], three-index bins by cost
     cudaMemPool_t pool = nullptr;            // plans (plan_alloc)
-    int bases = 0;                           // live bases of the device
+    int users = 0;                           // live bases and plans of the device
     bool ready = false;
 };
 
@@ -428,8 +428,8 @@ static void make_ranks(int schedule, std::vector<int> &rank, std::vector<int> &i
 
 // Plans come from a pool of the library: the default pool returns its memory to the system at every synchronisation
 // (release threshold 0), and planning synchronises, so a one-shot call on 2,000 pairs spent 200 of its 410 us on mapping its
-// 0.9 MB again.  This pool keeps up to kPoolKeep bytes between calls (the plan of 2M pairs takes 22 MB) and gives them
-// back when the last basis of the device is destroyed.  Stream-ordered like the default pool, shared by all threads.
+// 0.9 MB again.  This pool keeps up to kPoolKeep bytes between calls (the plan of 2M pairs takes 22 MB) while the device has
+// a basis or a plan, and nothing after the last of them.  Stream-ordered like the default pool, shared by all threads.
 constexpr uint64_t kPoolKeep = 256ull << 20;
 
 static cudaError_t make_pool(int dev, cudaMemPool_t *pool)
@@ -438,10 +438,13 @@ static cudaError_t make_pool(int dev, cudaMemPool_t *pool)
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
-    uint64_t keep = kPoolKeep;
-    cudaError_t e = cudaMemPoolCreate(pool, &props);
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    return e;
+    return cudaMemPoolCreate(pool, &props);
+}
+
+static cudaMemPool_t pool_of(int dev)
+{
+    std::lock_guard<std::mutex> lk(g_mu);
+    return g_dev[dev].pool;
 }
 
 // device memory of a plan on the current device, in the order of s (cudaFreeAsync frees it)
@@ -450,21 +453,22 @@ static cudaError_t plan_alloc(void **p, size_t bytes, cudaStream_t s)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    cudaMemPool_t pool;
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        pool = g_dev[dev].pool;
-    }
-    return cudaMallocFromPoolAsync(p, bytes, pool, s);
+    return cudaMallocFromPoolAsync(p, bytes, pool_of(dev), s);
 }
 
-// a basis of the device was made (+1) or destroyed (-1)
-static void count_basis(int dev, int d)
+// A basis or plan of the device was made (+1) or destroyed (-1, after its memory was freed).  Plans may outlive their
+// basis, and frees are still queued when the last one goes: from then on the threshold is 0, so the pool returns what the
+// trim finds in use at the first synchronisation after those frees.
+static void count_user(int dev, int d)
 {
     std::lock_guard<std::mutex> lk(g_mu);
     DevState &st = g_dev[dev];
-    st.bases += d;
-    if (st.bases == 0 && st.pool) cudaMemPoolTrimTo(st.pool, 0);
+    const bool was = st.users > 0;
+    st.users += d;
+    if (was == (st.users > 0) || !st.pool) return;
+    uint64_t keep = was ? 0 : kPoolKeep;
+    cudaMemPoolSetAttribute(st.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (was) cudaMemPoolTrimTo(st.pool, 0);
 }
 
 const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
@@ -479,7 +483,7 @@ const DeviceTables *device_tables_impl(int **ranks, int **rank3 = nullptr)
     DevState &st = g_dev[dev];
     if (!st.ready) {
         int *d_r[2] = {nullptr, nullptr};
-        bool ok = make_pool(dev, &st.pool) == cudaSuccess && cudaMalloc(&d_r[0], 2 * kNBins * sizeof(int)) == cudaSuccess &&
+        bool ok = (st.pool || make_pool(dev, &st.pool) == cudaSuccess) && cudaMalloc(&d_r[0], 2 * kNBins * sizeof(int)) == cudaSuccess &&
                   cudaMalloc(&d_r[1], 2 * kNBins * sizeof(int)) == cudaSuccess;
         for (int s = 0; s < 2 && ok; ++s) {
             std::vector<int> rank, inv;
@@ -806,7 +810,7 @@ int shg_basis_create(int n_shells, const int32_t *l, const int32_t *nprim, const
         shg_basis_destroy(b);
         return SHG_ECUDA;
     }
-    count_basis(d.device, 1);
+    count_user(d.device, 1);
     d.counted = true;
     *out = b;
     return SHG_OK;
@@ -850,7 +854,6 @@ int shg_basis_set_centers(shg_basis_t *b, const double *centers)
 void shg_basis_destroy(shg_basis_t *b)
 {
     if (!b) return;
-    if (b->d.counted) count_basis(b->d.device, -1);
     cudaFree(b->d.shells);
     cudaFree(b->d.prims);
     cudaFree(b->d.centers);
@@ -859,6 +862,7 @@ void shg_basis_destroy(shg_basis_t *b)
     cudaFree(b->d.stage_raw);
     cudaFree(b->d.stage_ctr);
     cudaFree(b->d.stage_bad);
+    if (b->d.counted) count_user(b->d.device, -1);
     delete[] b->d.h_l;
     delete[] b->d.h_nprim;
     delete[] b->d.h_center;
@@ -979,6 +983,7 @@ int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, c
     d.pair_a = pa;
     d.pair_b = pb;
     d.owner_block = blk;
+    d.device = basis->d.device;
     d.stream = s;
     char *c = (char *)blk;
     d.tiles = (Tile *)c;                 c += (bytes_tiles + 15) / 16 * 16;
@@ -1005,6 +1010,7 @@ int shg_plan_2c_create(const shg_basis_t *basis, int64_t n, const int32_t *pa, c
         p->launches = 0;
         for (int cls = 0; cls < kNClass; ++cls) p->launches += d.class_tile_begin[cls + 1] > d.class_tile_begin[cls];
     }
+    count_user(d.device, 1);
     *out = p;
     return SHG_OK;
 }
@@ -1127,6 +1133,7 @@ void shg_plan_destroy(shg_plan_t *p)
 {
     if (!p) return;
     cudaFreeAsync(p->d.owner_block, p->d.stream);
+    count_user(p->d.device, -1);
     delete p;
 }
 
@@ -1856,6 +1863,23 @@ int shg_debug_boys(int64_t n, const double *T, int nmax, double *F, void *stream
     const DeviceTables *t = device_tables();
     if (!t) return SHG_ECUDA;
     SHG_CUDA(launch_debug_boys(n, T, nmax, F, *t, (cudaStream_t)stream));
+    return SHG_OK;
+}
+
+int shg_debug_pool(int reset_high, uint64_t *reserved, uint64_t *used, uint64_t *used_high)
+{
+    g_err.clear();
+    if (!reserved || !used || !used_high) return fail(SHG_EINVAL, "NULL pointer");
+    int dev = 0;
+    SHG_CUDA(cudaGetDevice(&dev));
+    *reserved = *used = *used_high = 0;
+    cudaMemPool_t pool = dev < 64 ? pool_of(dev) : nullptr;
+    if (!pool) return SHG_OK;
+    SHG_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, reserved));
+    SHG_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, used));
+    SHG_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, used_high));
+    uint64_t zero = 0;
+    if (reset_high) SHG_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero));
     return SHG_OK;
 }
 

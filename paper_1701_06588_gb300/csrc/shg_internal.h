@@ -191,7 +191,7 @@ struct BasisDev {
     int32_t *h_fam = nullptr;                           // family of each shell
     int32_t *h_fam_prim = nullptr, *h_fam_k = nullptr;  // per family: first primitive record, K
     int n_fams = 0;
-    bool counted = false;         // among the live bases of its device
+    bool counted = false;         // among the users of the plan pool of its device
 };
 
 // A warp's unit of work: up to kTile / group consecutive entries of the sorted list, all of one class (cls = la*7 + lb, or
@@ -242,6 +242,7 @@ struct PlanDev {
     int threads = 128;             // launch shape (autotuned): threads per CTA (32, 64 or 128)
     int ctas_per_sm = 0;           // persistent CTAs per SM, 0 = occupancy limit
     int variant = 1;               // register cap of the kernels (shg_plan_2c_set_variant)
+    int device = 0;
     void *owner_block = nullptr;   // device allocation holding all of the above
     cudaStream_t stream = nullptr;
 };
