@@ -8,11 +8,12 @@ using namespace aab;
 
 // Shared memory of a slot in doubles: orders, F_q, C and S, then the partial sums or (L, M', q) products and two columns
 // of the blocks
-__host__ __device__ inline int slot_doubles(const Shape &s)
+__host__ __device__ constexpr int slot_doubles(const Shape &s)
 {
     const int nq = s.qbase(s.nL), work = kLanes * nq, ang = s.pbase(s.nL) + 2 * s.mbase(s.nL);
     return 2 * nq + 2 * (s.kmax + 1) + (work > ang ? work : ang);
 }
+static_assert(largest_slots([](const Shape &s) constexpr { return slot_doubles(s); }) <= kSharedLimit, "see kSharedLimit");
 
 // Screening of one triple: |phi_a phi_a~| <= 2 sabs_a sabs_a~ lfac_a lfac_a~
 // exp(-(amin_a + amin_a~) r^2 / 2) (the single-shell bound of the two-center
@@ -185,7 +186,7 @@ int slot_doubles_3c(int cls) { return slot_doubles(Shape(cls)); }
 
 cudaError_t launch_3c(const Args3c &a, cudaStream_t s)
 {
-    return launch_slots((const void *)k_3c_fp64, a, s, [&](int grid, size_t bytes) { k_3c_fp64<<<grid, 32, bytes, s>>>(a); });
+    return launch_slots((const void *)k_3c_fp64, a, [&](int grid, size_t bytes) { k_3c_fp64<<<grid, 32, bytes, s>>>(a); });
 }
 
 }  // namespace shg

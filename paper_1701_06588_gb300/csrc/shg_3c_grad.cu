@@ -11,12 +11,13 @@ using namespace aab;
 
 // Orders (one more per L than the integrals), F and F', C and S, the coefficients A (cosine and sine), then the partial
 // sums or the weight combinations of two columns and their projections
-__host__ __device__ inline int slot_doubles(const Shape &s)
+__host__ __device__ constexpr int slot_doubles(const Shape &s)
 {
     const int nq = s.qbase(s.nL), n1 = nq + s.nL, work = kLanes * n1;
     const int ang = 2 * s.pbase(s.nL) + 8 * (s.la + 1) * (s.lt + 1) + 2 * s.mbase(s.nL);
     return n1 + 2 * nq + 2 * (s.kmax + 1) + (work > ang ? work : ang);
 }
+static_assert(largest_slots([](const Shape &s) constexpr { return slot_doubles(s); }) <= kSharedLimit, "see kSharedLimit");
 
 __device__ __forceinline__ void tile_aab_grad(const Args3c &g, const Tile &t, int lane, double *smem)
 {
@@ -243,7 +244,7 @@ int slot_doubles_3c_grad(int cls) { return slot_doubles(Shape(cls)); }
 
 cudaError_t launch_3c_grad(const Args3c &a, cudaStream_t s)
 {
-    return launch_slots((const void *)k_3c_grad_fp64, a, s,
+    return launch_slots((const void *)k_3c_grad_fp64, a,
                         [&](int grid, size_t bytes) { k_3c_grad_fp64<<<grid, 32, bytes, s>>>(a); });
 }
 

@@ -26,27 +26,27 @@ constexpr int kSlots = 32 / kLanes;
 // Sizes of one (la, lt, lb) class
 struct Shape {
     int la, lt, lb, Lmin, Lmax, nL, kmax;          // kmax = Lmax + lb
-    __host__ __device__ Shape(int cls)
+    __host__ __device__ constexpr Shape(int cls)
         : la(cls / 49), lt(cls / 7 % 7), lb(cls % 7), Lmin(la > lt ? la - lt : lt - la), Lmax(la + lt),
           nL((Lmax - Lmin) / 2 + 1), kmax(Lmax + lb)
     {
     }
-    __host__ __device__ int L(int i) const { return Lmin + 2 * i; }
-    __host__ __device__ int J(int i) const { return (L(i) < lb ? L(i) : lb) + 1; }
+    __host__ __device__ constexpr int L(int i) const { return Lmin + 2 * i; }
+    __host__ __device__ constexpr int J(int i) const { return (L(i) < lb ? L(i) : lb) + 1; }
     // first (L, q) entry, first (L, M', q) entry (M' = 0..L+lb) and first (L, M) entry of L(i)
-    __host__ __device__ int qbase(int i) const
+    __host__ __device__ constexpr int qbase(int i) const
     {
         int n = 0;
         for (int j = 0; j < i; ++j) n += J(j);
         return n;
     }
-    __host__ __device__ int pbase(int i) const
+    __host__ __device__ constexpr int pbase(int i) const
     {
         int n = 0;
         for (int j = 0; j < i; ++j) n += (L(j) + lb + 1) * J(j);
         return n;
     }
-    __host__ __device__ int mbase(int i) const
+    __host__ __device__ constexpr int mbase(int i) const
     {
         int n = 0;
         for (int j = 0; j < i; ++j) n += 2 * L(j) + 1;
@@ -200,18 +200,32 @@ __device__ __forceinline__ void circular(double x, double y, int kmax, int gl, d
     }
 }
 
+// Dynamic shared memory that every kernel may take without raising its own limit.  That limit belongs to the function, not
+// to a launch: a call that set it for its own list could lower it between another thread's setting and launch.  The largest
+// class takes 20,160 bytes (integrals) and 43,456 bytes (gradients).
+constexpr size_t kSharedLimit = 48 << 10;
+
+// bytes of a warp's slots, the largest over the valid classes (la + la~ <= kLmaxAabA)
+template <class Doubles>
+constexpr size_t largest_slots(Doubles doubles)
+{
+    int most = 0;
+    for (int cls = 0; cls < kNClass3; ++cls) {
+        const Shape s(cls);
+        if (s.Lmax <= kLmaxAabA && doubles(s) > most) most = doubles(s);
+    }
+    return kSlots * sizeof(double) * (size_t)most;
+}
+
 // Persistent launch of one-warp CTAs with the shared memory of four slots each
 template <class Launch>
-cudaError_t launch_slots(const void *kernel, const Args3c &a, cudaStream_t s, Launch launch)
+cudaError_t launch_slots(const void *kernel, const Args3c &a, Launch launch)
 {
-    (void)s;
     const size_t bytes = (size_t)kSlots * a.slot_doubles * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 32, bytes);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 32, bytes);
     if (e != cudaSuccess) return e;
     launch((sms > 0 ? sms : 1) * (per > 0 ? per : 1), bytes);
     return cudaGetLastError();
