@@ -202,14 +202,16 @@ int shg_plan_2c_exec(shg_plan_t *plan, int op, double omega, double screen_thres
  * shg_plan_2c_set_variant - register cap of the two-center kernels used by
  * later executions of the plan (an autotuner knob), as 128-thread CTAs that
  * must fit on an SM; capped kernels spill some values to local memory.
- *   1/r and erfc, alone or together:   0 = four CTAs, 1 = eight, 2 = six
+ *   erfc, 1/r and erfc (mixed precision: also 1/r, in the double-float
+ *   launch):                           0 = four CTAs, 1 = eight, 2 = six
  *   other sets of operators, FP64:     0 = three,     1 = six,   2 = four
- *   other sets of operators, mixed:    0 = four,      1 = six,   2 = five
- * A new plan takes 1 when more than two thirds of its work units are of
- * classes with min(la, lb) <= 1 (few accumulators: more warps hide their
- * latency) and 0 otherwise.  The variants run the same operations in the same
- * order, so the results are bitwise equal.  SHG_EINVAL for a value outside
- * 0..2.
+ *   other sets, double-float launch:   0 = four,      1 = six,   2 = five
+ * Passes of one operator other than these have one kernel (four CTAs), which
+ * every variant runs.  A new plan takes 1 when more than two thirds of its
+ * tiles are of classes with min(la, lb) <= 1 (few accumulators: more warps
+ * hide their latency) and 0 otherwise.  The variants run the same operations
+ * in the same order, so the results are bitwise equal.  SHG_EINVAL for a value
+ * outside 0..2.
  */
 int shg_plan_2c_set_variant(shg_plan_t *plan, int variant);
 
@@ -228,8 +230,14 @@ int shg_plan_launches_prec(const shg_plan_t *plan, int precision);
  * shg_plan_2c_set_launch - launch shape of later executions of a plan (the
  * autotuner's knobs): threads per CTA (32, 64 or 128; each warp owns one
  * tile of up to 32 pairs) and, for the persistent schedule, CTAs per SM
- * (0 = as many as occupancy allows).  Returns SHG_EINVAL for other values.
+ * (0 = as many as occupancy allows).  A persistent plan of at most
+ * SHG_SHORT_LIST_TILES tiles runs one 32-thread CTA per tile whatever is set
+ * here (SHG_OP_RA2N excepted).  Returns SHG_EINVAL for other values.
+ * shg_plan_tiles - number of tiles (work units of one warp) of a plan; -1 for
+ * a NULL plan.
  */
+#define SHG_SHORT_LIST_TILES 1024
+int64_t shg_plan_tiles(const shg_plan_t *plan);
 int shg_plan_2c_set_launch(shg_plan_t *plan, int threads_per_cta, int ctas_per_sm);
 
 /*

@@ -15,6 +15,7 @@ SHG_OK, SHG_EINVAL, SHG_ENOMEM, SHG_ECUDA, SHG_ETIMEOUT, SHG_ERANGE = 0, -1, -2,
 SHG_OP_OVERLAP, SHG_OP_COULOMB, SHG_OP_ERFC, SHG_OP_ERF, SHG_OP_GAUSS, SHG_OP_GAUSS_COULOMB, SHG_OP_RA2N = range(7)
 SHG_PREC_FP64, SHG_PREC_MIXED = 0, 1
 SHG_SCHED_PER_CLASS, SHG_SCHED_PERSISTENT = 0, 1
+SHG_SHORT_LIST_TILES = 1024
 
 OPERATORS = {"overlap": SHG_OP_OVERLAP, "coulomb": SHG_OP_COULOMB, "erfc": SHG_OP_ERFC, "erf": SHG_OP_ERF,
              "gauss": SHG_OP_GAUSS, "gauss_coulomb": SHG_OP_GAUSS_COULOMB, "ra2n": SHG_OP_RA2N}
@@ -39,6 +40,7 @@ SIGNATURES = [
     ("shg_plan_2c_exec", _I, [_P, _I, _D, _D, _I, _P, _P, _P]),
     ("shg_plan_launches", _I, [_P]),
     ("shg_plan_launches_prec", _I, [_P, _I]),
+    ("shg_plan_tiles", _L, [_P]),
     ("shg_plan_2c_set_variant", _I, [_P, _I]),
     ("shg_plan_destroy", None, [_P]),
     ("shg_family_plan_create", _I, [_P, _L, _P, _P, _P, ctypes.POINTER(_P)]),
@@ -176,6 +178,10 @@ def shg_family_plan_destroy(plan):
 
 def shg_plan_launches(plan):
     return load().shg_plan_launches(plan)
+
+
+def shg_plan_tiles(plan):
+    return load().shg_plan_tiles(plan)
 
 
 def shg_plan_2c_set_variant(plan, variant):

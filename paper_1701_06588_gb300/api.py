@@ -101,6 +101,7 @@ class Plan2c:
         self.handle = L.shg_plan_2c_create(basis.handle, self.n, self.pair_a, self.pair_b, _sched(schedule),
                                            _stream(stream))
         self.launches = L.shg_plan_launches(self.handle)
+        self.tiles = L.shg_plan_tiles(self.handle)
 
     def launches_for(self, precision):
         """Kernel launches one execution of this plan issues in `precision`."""
@@ -375,7 +376,7 @@ class HostPipeline2c:
             plans.append(plan)
             if self.launch:
                 set_launch(plan, self.launch["threads_per_cta"], self.launch["ctas_per_sm"],
-                           self.launch.get("variant", 1))
+                           self.launch.get("variant"))
             planned = torch.cuda.Event()
             planned.record(up)
             cs = self.compute_streams[len(plans) % 2]
@@ -403,12 +404,13 @@ class HostPipeline2c:
         return outs
 
 
-def set_launch(plan, threads_per_cta=128, ctas_per_sm=0, variant=1):
+def set_launch(plan, threads_per_cta=128, ctas_per_sm=0, variant=None):
     """Launch shape of later executions of a plan: threads per CTA, persistent
-    CTAs per SM (0 = occupancy limit) and the compiled variant of the
-    fused kernel (0, 1 or 2, see shg_plan_2c_set_variant)."""
+    CTAs per SM (0 = occupancy limit) and the register cap (0, 1 or 2, see
+    shg_plan_2c_set_variant; None leaves the plan's)."""
     L.shg_plan_2c_set_launch(plan.handle, int(threads_per_cta), int(ctas_per_sm))
-    L.shg_plan_2c_set_variant(plan.handle, int(variant))
+    if variant is not None:
+        L.shg_plan_2c_set_variant(plan.handle, int(variant))
 
 
 def eval_3c_aab_grad(orb, aux, t_a, t_atilde, t_b, upstream, offsets=None, precision="fp64", stream=None):

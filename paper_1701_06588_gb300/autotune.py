@@ -3,7 +3,9 @@
 Candidates: schedule (one launch per class, or one persistent launch with
 tiles in decreasing estimated cost), threads per CTA (1, 2 or 4 warps, each
 warp owning a class-pure tile of up to 32 pairs), persistent CTAs per SM, and
-the compiled kernel variant (register caps, see shg_plan_2c_set_variant).
+the compiled kernel variant (register caps, see shg_plan_2c_set_variant) of the
+passes that have more than one.  Lists that run one CTA per tile whatever the
+launch shape is have one persistent candidate.
 Each candidate runs the requested operators a few times (CUDA events, after a
 warm-up); the fastest is cached in a JSON file keyed by GPU name, precision,
 operators and a signature of the workload's (la, lb, Ka*Kb) histogram.
@@ -16,11 +18,11 @@ import os
 import numpy as np
 import torch
 
+from . import _lib as L
 from . import api
 
 CANDIDATES = ([("per_class", t, 0) for t in (32, 64, 128)] +
               [("persistent", t, c) for t in (32, 64, 128) for c in (0, 1, 2, 4, 8)])
-VARIANTS = dict.fromkeys(("fp64", "mixed", "fp64_fused", "mixed_fused"), (0, 1, 2))
 
 
 def cache_path():
@@ -34,6 +36,20 @@ def workload_signature(basis, pair_a, pair_b):
     key = (l[pair_a] * 7 + l[pair_b]) * 1024 + np.minimum(k[pair_a] * k[pair_b], 1023)
     hist = np.bincount(key, minlength=49 * 1024)
     return hashlib.sha256(hist.astype(np.int64).tobytes()).hexdigest()[:16]
+
+
+def variants(ops, precision):
+    """Register caps to try: (None,), the plan's own, when every pass over `ops` has one kernel."""
+    ids = [api._op(o) for o in ops]
+    passes = [set(ids)] if precision.endswith("_fused") else [{i} for i in ids]
+    capped = {L.SHG_OP_ERFC} | ({L.SHG_OP_COULOMB} if precision.startswith("mixed") else set())
+    return (0, 1, 2) if any(len(p) > 1 or p & capped for p in passes) else (None,)
+
+
+def candidates(tiles, ops):
+    """Launch shapes to try: (schedule, threads per CTA, CTAs per SM); tiles: of a persistent plan."""
+    short = tiles <= L.SHG_SHORT_LIST_TILES and L.SHG_OP_RA2N not in [api._op(o) for o in ops]
+    return [c for c in CANDIDATES if not (short and c[0] == "persistent" and c[1:] != (128, 0))]
 
 
 def _load():
@@ -65,18 +81,16 @@ def tune_2c(basis, pair_a, pair_b, ops, omegas, out_offsets, outs, precision="fp
             for op, om, o in zip(ops, omegas, outs):
                 plan.exec(op, out_offsets, o, omega=om, precision=precision)
 
-    key = "|".join(["v3", torch.cuda.get_device_name(), precision, ",".join(map(str, ops)),
+    key = "|".join(["v4", torch.cuda.get_device_name(), precision, ",".join(map(str, ops)),
                     workload_signature(basis, pair_a, pair_b)])
     db = _load()
     if not force and key in db:
         return db[key]
     results = []
-    plans = {}
-    for sched, threads, ctas in CANDIDATES:
-        if sched not in plans:
-            plans[sched] = api.Plan2c(basis, pair_a, pair_b, schedule=sched)
+    plans = {s: api.Plan2c(basis, pair_a, pair_b, schedule=s) for s in ("per_class", "persistent")}
+    for sched, threads, ctas in candidates(plans["persistent"].tiles, ops):
         plan = plans[sched]
-        for variant in VARIANTS.get(precision, (0,)):
+        for variant in variants(ops, precision):
             api.set_launch(plan, threads, ctas, variant)
             one_pass(plan)
             torch.cuda.synchronize()
@@ -101,5 +115,5 @@ def tune_2c(basis, pair_a, pair_b, ops, omegas, out_offsets, outs, precision="fp
 
 def tuned_plan(basis, pair_a, pair_b, config):
     plan = api.Plan2c(basis, pair_a, pair_b, schedule=config["schedule"])
-    api.set_launch(plan, config["threads_per_cta"], config["ctas_per_sm"], config.get("variant", 1))
+    api.set_launch(plan, config["threads_per_cta"], config["ctas_per_sm"], config.get("variant"))
     return plan

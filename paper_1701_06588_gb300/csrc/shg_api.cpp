@@ -1025,6 +1025,8 @@ int shg_plan_launches_prec(const shg_plan_t *p, int precision)
     return (df > 0) + (p->d.n_tiles > df);
 }
 
+int64_t shg_plan_tiles(const shg_plan_t *p) { return p ? p->d.n_tiles : -1; }
+
 int shg_plan_2c_set_variant(shg_plan_t *p, int variant)
 {
     g_err.clear();
@@ -1262,7 +1264,7 @@ static int exec_fp64(shg_plan_t *p, int op, double omega, double screen, const i
 // Most tiles that a pass of a persistent plan runs with one CTA each instead of a work counter: all of them are resident at
 // once (8 warps or more per SM), spread over the SMs one by one, without the launch that clears the counter (63 tiles of
 // 2,000 pairs, overlap and 1/r: 102 us persistent with four-warp CTAs, 95 us with one-warp CTAs)
-constexpr int kStaticTiles = 1024;
+constexpr int kStaticTiles = SHG_SHORT_LIST_TILES;
 
 // Radial sums of one operator
 static unsigned want_of(int op)
