@@ -553,7 +553,8 @@ def run_ours(args, rank, world):
                          "k's copy on a second stream overlaps operator k+1's kernel)"),
                 "unchunked_ms": 1e3 * e2e_single_s,
                 "unchunked_ms_parts": {k: 1e3 * statistics.mean(v) for k, v in parts.items() if v}},
-        "gpu_launches": args.steps * (1 if fused else len(OPS)) * plan.launches_for(args.precision),
+        "gpu_launches": args.steps * (plan.launches_for(args.precision, names) if fused else
+                                      len(OPS) * plan.launches_for(args.precision)),
         "clocks": clk,
         "measured_peaks_tflops": {"fp64": fp64_peak / 1e12, "fp32": fp32_peak / 1e12,
                                   "fp64_tensor_mma_m8n8k4": dmma_peak / 1e12},

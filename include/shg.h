@@ -215,16 +215,21 @@ int shg_plan_2c_exec(shg_plan_t *plan, int op, double omega, double screen_thres
  */
 int shg_plan_2c_set_variant(shg_plan_t *plan, int variant);
 
-/* Number of kernel launches one FP64 shg_plan_2c_exec (or fused pass over a
- * list of more than about 30,000 pairs; a shorter one may issue one per
- * operator) issues (for accounting). */
+/* Number of kernel launches one FP64 shg_plan_2c_exec issues (for
+ * accounting). */
 int shg_plan_launches(const shg_plan_t *plan);
 
-/* Number of kernel launches one execution of the plan issues in `precision`
+/* Number of kernel launches one shg_plan_2c_exec issues in `precision`
  * (SHG_PREC_MIXED: the double-float launch of the classes with
  * min(la, lb) = 2 or 3 and the FP64 launch of the others, where a persistent
- * plan holds any); -1 for a NULL plan or bad precision. */
+ * plan holds any; not for SHG_OP_RA2N); -1 for a NULL plan or bad precision. */
 int shg_plan_launches_prec(const shg_plan_t *plan, int precision);
+
+/* Number of kernel launches one shg_plan_2c_exec_fused over ops[n_ops] issues
+ * in `precision`: those of shg_plan_launches_prec, once per operator (1/r and
+ * erfc count as one) for a persistent plan whose tiles times these operators
+ * are at most SHG_SHORT_LIST_TILES; -1 as above and for bad operators. */
+int shg_plan_launches_fused(const shg_plan_t *plan, int n_ops, const int *ops, int precision);
 
 /*
  * shg_plan_2c_set_launch - launch shape of later executions of a plan (the
@@ -266,8 +271,8 @@ void shg_graph_destroy(shg_graph_t *graph);
  * one attenuated sum.  Results agree with shg_plan_2c_exec of each operator
  * up to the order of the floating-point sums.  SHG_PREC_MIXED runs the same
  * scheme with the mixed angular part; its accuracy bar is that of the mixed
- * single-operator pass.  A short list (at most 1,024 tiles over all operators)
- * runs as one launch per operator, all side by side.
+ * single-operator pass.  A short list runs as one launch per operator, all
+ * side by side (shg_plan_launches_fused).
  *   ops[n_ops], omegas[n_ops]  host arrays, 1 <= n_ops <= 5; each of
  *                  SHG_OP_OVERLAP, SHG_OP_COULOMB, SHG_OP_ERFC, SHG_OP_ERF,
  *                  SHG_OP_GAUSS at most once; omega rules of shg_eval_2c

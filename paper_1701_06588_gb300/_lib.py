@@ -40,6 +40,7 @@ SIGNATURES = [
     ("shg_plan_2c_exec", _I, [_P, _I, _D, _D, _I, _P, _P, _P]),
     ("shg_plan_launches", _I, [_P]),
     ("shg_plan_launches_prec", _I, [_P, _I]),
+    ("shg_plan_launches_fused", _I, [_P, _I, _P, _I]),
     ("shg_plan_tiles", _L, [_P]),
     ("shg_plan_2c_set_variant", _I, [_P, _I]),
     ("shg_plan_destroy", None, [_P]),
@@ -178,6 +179,11 @@ def shg_family_plan_destroy(plan):
 
 def shg_plan_launches(plan):
     return load().shg_plan_launches(plan)
+
+
+def shg_plan_launches_fused(plan, ops, precision):
+    a = (_I * len(ops))(*ops)
+    return check(load().shg_plan_launches_fused(plan, len(ops), ctypes.cast(a, _P), precision))
 
 
 def shg_plan_tiles(plan):

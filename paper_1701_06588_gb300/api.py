@@ -103,8 +103,11 @@ class Plan2c:
         self.launches = L.shg_plan_launches(self.handle)
         self.tiles = L.shg_plan_tiles(self.handle)
 
-    def launches_for(self, precision):
-        """Kernel launches one execution of this plan issues in `precision`."""
+    def launches_for(self, precision, ops=None):
+        """Kernel launches one exec of this plan issues in `precision`, or one
+        exec_fused over `ops`."""
+        if ops is not None:
+            return L.shg_plan_launches_fused(self.handle, [_op(o) for o in ops], _prec(precision))
         return L.shg_plan_launches_prec(self.handle, _prec(precision))
 
     def exec(self, op, out_offsets, out, omega=0.0, precision="fp64", screen_thresh=0.0, stream=None):

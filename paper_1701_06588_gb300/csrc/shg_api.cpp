@@ -1279,6 +1279,16 @@ static unsigned want_of(int op)
     }
 }
 
+// Parts that a pass of a persistent plan over the operators `ops` (bits) is launched in: one per operator (1/r and erfc
+// count as one) where all of them take at most kStaticTiles warps, else one
+static int pass_parts(const PlanDev &d, unsigned ops)
+{
+    const unsigned pair = 1u << SHG_OP_COULOMB | 1u << SHG_OP_ERFC;
+    int n = (ops & pair) == pair ? -1 : 0;
+    for (int op = 0; op < 6; ++op) n += ops >> op & 1;
+    return n > 1 && (int64_t)n * d.n_tiles <= kStaticTiles ? n : 1;
+}
+
 // Pass over a list of at most kStaticTiles tiles.  With few enough they leave most warp slots empty, so each operator gets
 // a launch of its own, all side by side (1/r and erfc, which share their sums, together): 2,000 pairs of short
 // contractions, overlap and 1/r, 101 us in one launch, 74 in two; five operators 170 and 107 us.  Beyond the limit the
@@ -1287,9 +1297,9 @@ static unsigned want_of(int op)
 static int exec_short(shg_plan_t *p, const ArgsFused &f, bool mixed, cudaStream_t s)
 {
     const bool pair = f.out[SHG_OP_COULOMB] && f.out[SHG_OP_ERFC];
-    int n = 0;
-    for (int op = 0; op < 6; ++op) n += f.out[op] && !(pair && op == SHG_OP_ERFC);
-    const bool split = n > 1 && n * p->d.n_tiles <= kStaticTiles;
+    unsigned ops = 0;
+    for (int op = 0; op < 6; ++op) ops |= f.out[op] ? 1u << op : 0u;
+    const bool split = pass_parts(p->d, ops) > 1;
     ArgsMixFused m;
     if (mixed) fill_kappa_mix(m.kappa);
     bool beside = false;
@@ -1428,6 +1438,18 @@ int shg_plan_2c_exec_fused(shg_plan_t *p, int n_ops, const int *ops, const doubl
     fused_plan(a, *p->d.basis, p->d, *t, off);
     if (precision == SHG_PREC_MIXED) return exec_mixed(p, a, s);
     return exec_fused_fp64(p, a, s);
+}
+
+int shg_plan_launches_fused(const shg_plan_t *p, int n_ops, const int *ops, int precision)
+{
+    const int one = shg_plan_launches_prec(p, precision);
+    if (one < 0 || n_ops < 1 || n_ops > 5 || !ops) return -1;
+    unsigned bits = 0;
+    for (int i = 0; i < n_ops; ++i) {
+        if (ops[i] < SHG_OP_OVERLAP || ops[i] > SHG_OP_GAUSS) return -1;
+        bits |= 1u << ops[i];
+    }
+    return p->d.schedule == SHG_SCHED_PERSISTENT ? one * pass_parts(p->d, bits) : one;
 }
 
 int shg_graph_2c_create_fused(shg_plan_t *p, int n_ops, const int *ops, const double *omegas, int precision,
