@@ -149,13 +149,15 @@ SHG_HD xf from_double(double x)
 }
 
 // FP64 value with the sign of bit 31 of `sign`: round to nearest (ties up) of the 62-bit significand;
-// below the normal range 0, above it infinity.  a.m in [2^62, 2^63)
+// below the normal range 0, above it infinity.  a.m in [2^62, 2^63).  Denormal results would take a shift by a variable
+// count: five operators on 200,000 pairs 749 -> 765 us, 1/r and erfc on 1M pairs 2.489 -> 2.506 ms, 900,000 (a b a~) triples
+// 11.36 -> 11.53 ms; in a branch of their own 790 us and 2.506 ms.
 SHG_HD double to_double(xf a, uint32_t sign)
 {
     const uint64_t r = (a.m + 512u) >> 10;                                   // 2^52 .. 2^53
     const int E = a.e + 1084;                                                // biased exponent less the implicit bit
     uint64_t v = r + ((uint64_t)(uint32_t)E << 52);
-    if ((unsigned)E >= 2045u) v = E < 0 ? 0 : 0x7ff0000000000000ull;
+    if ((unsigned)E >= 2046u) v = E < 0 ? 0 : 0x7ff0000000000000ull;
     return bitsd(v | ((uint64_t)(sign & 0x80000000u) << 32));
 }
 
