@@ -56,7 +56,5 @@ __device__ __forceinline__ df mul_f(df a, float b)
     return fast_two_sum(p, e);
 }
 
-__device__ __forceinline__ double to_double(df a) { return (double)a.hi + (double)a.lo; }
-
 }  // namespace dfm
 }  // namespace shg

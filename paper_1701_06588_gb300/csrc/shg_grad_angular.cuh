@@ -22,14 +22,12 @@ struct NumD {
     using C = double;
     static __device__ __forceinline__ T zero() { return 0.0; }
     static __device__ __forceinline__ T one() { return 1.0; }
-    static __device__ __forceinline__ T con(double v) { return v; }
     static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
     static __device__ __forceinline__ T add(T a, T b) { return a + b; }
     static __device__ __forceinline__ T sub(T a, T b) { return a - b; }
     static __device__ __forceinline__ T fma(T a, T b, T c) { return ::fma(a, b, c); }
     static __device__ __forceinline__ T fnma(T a, T b, T c) { return ::fma(-a, b, c); }
     static __device__ __forceinline__ T smul(float n, T a) { return (double)n * a; }       // exact small n
-    static __device__ __forceinline__ const C *table(const CGTab &t) { return t.g; }
     static __device__ __forceinline__ T ld(const C *p) { return __ldg(p); }
 };
 
@@ -38,14 +36,12 @@ struct NumF {
     using C = float2;
     static __device__ __forceinline__ T zero() { return dfm::df_f(0.0f); }
     static __device__ __forceinline__ T one() { return dfm::df_f(1.0f); }
-    static __device__ __forceinline__ T con(double v) { return cgm::split(v); }
     static __device__ __forceinline__ T mul(T a, T b) { return dfm::mul(a, b); }
     static __device__ __forceinline__ T add(T a, T b) { return dfm::add(a, b); }
     static __device__ __forceinline__ T sub(T a, T b) { return dfm::sub(a, b); }
     static __device__ __forceinline__ T fma(T a, T b, T c) { return dfm::add(dfm::mul(a, b), c); }
     static __device__ __forceinline__ T fnma(T a, T b, T c) { return dfm::sub(c, dfm::mul(a, b)); }
     static __device__ __forceinline__ T smul(float n, T a) { return dfm::mul_f(a, n); }
-    static __device__ __forceinline__ const C *table(const CGTab &t) { return t.gm; }
     static __device__ __forceinline__ T ld(const C *p) { return cgm::ldf(__ldg(p)); }
 };
 
@@ -119,7 +115,7 @@ __device__ __forceinline__ void project(const typename N::C *__restrict__ g, int
     }
 }
 
-// gradient of sum_{L,M} A_{L,M} S_{L,M} F_p: G = (dx, dy, dz).  P, R: work arrays of (kmax + 2) J entries
+// gradient of sum_{L,M} A_{L,M} S_{L,M} F_p: G = (dx, dy, dz).  P, R: work arrays of (kmax + 1) J entries
 template <class N, int J, class Kap>
 __device__ __forceinline__ void contract(typename N::T x, typename N::T y, typename N::T z, typename N::T q, int kmax,
                                          const Kap &kap, const typename N::T (&F)[J], const typename N::T (&D)[J],
