@@ -67,14 +67,17 @@ enum shg_operator {
 };
 
 enum shg_precision {
-    SHG_PREC_FP64 = 0,  /* every step in FP64                                     */
-    SHG_PREC_MIXED = 1  /* FP32-based compensated arithmetic where it is the
-                           faster form: the angular part of the classes with
-                           min(la, lb) = 2 or 3 (gradients: 3) in double-float;
-                           the other classes as in FP64 (with both la and
-                           lb >= 4 the sum over j of Eq. final_r12int_ab
-                           cancels beyond double-float reach), and all radial
-                           sums as in FP64                                     */
+    SHG_PREC_FP64 = 0,  /* FP64, and for the primitive terms of the radial sums
+                           63-bit significands on the integer units (every
+                           term rounded to FP64 once; terms below 2^-1022
+                           count as 0)                                         */
+    SHG_PREC_MIXED = 1  /* FP32-based compensated arithmetic (double-float) in
+                           the angular part of the classes with
+                           min(la, lb) = 2 or 3 (gradients: 3); all radial
+                           sums and the other classes as in FP64 (with both la
+                           and lb >= 4 the angular sum cancels beyond
+                           double-float reach, below 2 FP64 is faster).  On
+                           GB300 it saves little or no time                    */
 };
 
 enum shg_schedule {
@@ -261,15 +264,14 @@ int shg_graph_launch(shg_graph_t *graph, void *stream);
 void shg_graph_destroy(shg_graph_t *graph);
 
 /*
- * shg_plan_2c_exec_fused - several operators of one plan in a single pass.  The two-center formula of Sec. II B factors as
- *   (a|O|b)[ma][mb] = (-1)^lb A_{la,ma} A_{lb,mb} sum_j 2^{la+lb-j} O^{(la+lb-j)} Q_j[ma][mb],
- * where Q_j (Eq. Q_matrix contracted with the weights (2j-1)!! B_{j,kappa} of
- * Eq. B) depends on the geometry only; the pass builds Q_j once per shell
- * pair and contracts it with the radial orders of every requested operator
- * (Table S1).  The radial sums share their primitive-pair setup, erfc(wr)/r
+ * shg_plan_2c_exec_fused - several operators of one plan in a single pass.
+ * The harmonics of R_a - R_b in the expanded angular part depend on the
+ * geometry only; the pass forms them once per shell pair and combines them
+ * with the radial orders of every requested operator (Table S1).  The radial
+ * sums share their primitive-pair setup, erfc(wr)/r
  * is formed as 1/r - erf(wr)/r, and erf and erfc with the same omega share
  * one attenuated sum.  Results agree with shg_plan_2c_exec of each operator
- * up to the order of the floating-point sums.  SHG_PREC_MIXED runs the same
+ * up to the rounding of those shared sums.  SHG_PREC_MIXED runs the same
  * scheme with the mixed angular part; its accuracy bar is that of the mixed
  * single-operator pass.  A short list runs as one launch per operator, all
  * side by side (shg_plan_launches_fused).
@@ -303,11 +305,11 @@ void shg_plan_destroy(shg_plan_t *plan);
 
 /*
  * shg_eval_3c_aab - three-index overlaps (a b a~) = int phi_a phi_a~ phi_b of
- * Sec. II D: the product phi_a phi_a~ is expanded with real Gaunt
- * coefficients into shells L_a = |la-la~|..la+la~ (step 2) with exponent
+ * Sec. II D: the product phi_a phi_a~ is expanded in real solid harmonics
+ * into shells L_a = |la-la~|..la+la~ (step 2) with exponent
  * alpha + alpha~ (Eq. product_SHG_STGO), the radial part is P^{(k)} of
  * Eq. Pa_aba built from (0_a'|r_a^{2m}|0_b)^{(k)} (Eqs. sra2ms, devsra2ms),
- * and the angular part reuses Q of Sec. II E.
+ * and the angular part of each is that of a two-center block.
  *   orb            basis of a and a~ (both on one center, checked)
  *   aux            basis of b (may be the same handle as orb)
  *   d_a, d_atilde  device int32[n_triples] indices into orb
@@ -455,7 +457,7 @@ int shg_reduce_centers(const shg_basis_t *basis, int64_t n_pairs, const int32_t 
 /*
  * shg_debug_boys - device Boys function F_n(T) = int_0^1 exp(-T t^2) t^{2n} dt
  * (SI Eq. 3) as used by the Coulomb-type radial terms: for every T in
- * d_T[n_T] writes F_n for n = 0..nmax (nmax <= 24) to d_F[i*(nmax+1) + n].
+ * d_T[n_T] writes F_n for n = 0..nmax (nmax <= 15) to d_F[i*(nmax+1) + n].
  */
 int shg_debug_boys(int64_t n_T, const double *d_T, int nmax, double *d_F, void *stream);
 

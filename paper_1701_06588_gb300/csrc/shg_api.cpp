@@ -358,6 +358,9 @@ struct DevState {
     bool ready = false;
 };
 
+// Estimated cost of a triple of kk primitive combinations, for the order of the tiles: operations of the form that sums order
+// by order with translation matrices.  The present kernels take fewer per element (the expanded harmonics) and per
+// combination, so it overrates large l.
 static double class_cost3(int la, int lt, int lb, int kk)
 {
     const int Lmin = std::abs(la - lt), Lmax = la + lt, nL = (Lmax - Lmin) / 2 + 1;
@@ -376,6 +379,7 @@ static uint8_t g_chunk_class[2][kNClass];   // class of every chunk of a schedul
 static std::mutex g_mu;
 static DevState g_dev[64];
 
+// the same of a pair
 static double class_cost(int la, int lb, int kk)
 {
     const int J = std::min(la, lb) + 1;

@@ -21,14 +21,16 @@ constexpr int kTile = 32;         // pairs per warp tile
 // of the largest term); below, the FP64 units, which are otherwise a third busy, take the few sums sooner than the FP32
 // pipes take 18 instructions for each: 1M pairs, 1/r and erfc, 2.92 ms with all classes below 4 in double-float, 2.53 ms
 // from 2 or from 3 on; 123,000 pairs, erfc, 596, 439 (from 2) and 466 us (from 3); 250,000 gradients of erfc 1.22, 1.16 and
-// 1.09 ms.
+// 1.09 ms.  Between these two limits double-float gains nothing over FP64 for every class either (1M pairs 2.49 ms, the
+// 2M-pair step 4.93 against 4.85, 500,000 gradients of erfc 1.99 against 1.95): the classes kept are those where it loses
+// least.
 constexpr int kMixedDfMinL = 2, kMixedDfMinLGrad = 3, kMixedFp64MinL = 4;
 inline int min_l(int cls) { return cls / 7 < cls % 7 ? cls / 7 : cls % 7; }
 inline bool mixed_runs_fp64(int cls) { return min_l(cls) < kMixedDfMinL || min_l(cls) >= kMixedFp64MinL; }
 
 // Boys function for the extended-float radial sums: from T = kFarT on the asymptotic form (relative error below 5e-18
-// for n <= 13: T^{n-1/2} e^{-T} / Gamma(n+1/2)); below, per order n = 0..kBoysOrders-1 and cell [i, i+1) / 512 of T, the Taylor coefficients c_t = F_{n+t}(T_{i+1}) / t! about the upper end of the cell, scaled by
-// 2^s so that c0 < 2^63 (1 - 2^-8): c0, c1 in units 2^-s, c2 likewise with s - 62 in its low 8 bits, c3 in units
+// for n <= 13: T^{n-1/2} e^{-T} / Gamma(n+1/2)); below, per order n = 0..kBoysOrders-1 and cell [i, i+1) / 512 of T, the
+// Taylor coefficients c_t = F_{n+t}(T_{i+1}) / t! about the upper end of the cell, scaled by 2^s so that c0 < 2^63 (1 - 2^-8): c0, c1 in units 2^-s, c2 likewise with s - 62 in its low 8 bits, c3 in units
 // 2^{30-s}, c4 (24 bits) in units 2^{35-s}, c5 (8 bits) in units 2^{49-s}.  y = T_{i+1} - T <= 2^-9, so the dropped
 // y^6/720 is below 2^-63.  One 32-byte load per evaluation; 18.9 MB, resident in L2.
 constexpr int kFarT = 72;
