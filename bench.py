@@ -35,7 +35,6 @@ METRIC = "shell-pair integrals/s on 1 GB300 at 1e-12 rel (FP64) vs mixed; % of r
 UNIT = "shell-pair integrals/s"
 WORKLOAD = "c3_2m_l6_k20"
 OPS = [("coulomb", 1, 0.0), ("erfc", 2, 0.11)]
-DF_FMA_FP32_INSTR = 18.0       # FP32 instructions of one double-float multiply-add
 FP64_NOMINAL_TFLOPS = 1.25   # 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (nominal, context)
 PROFILES = {"fp64_fused": os.path.join(ROOT, "profiles", "k_2c_fp64_fused_c3_2m.txt"),
             "mixed_fused": os.path.join(ROOT, "profiles", "k_2c_mixed_fused_c3_2m.txt"),
@@ -219,9 +218,7 @@ def run_reference(args, rank, world):
 # --------------------------------------------------------------------------- #
 # GPU arm                                                                     #
 # --------------------------------------------------------------------------- #
-# the sources that build the two-center kernels the profiles describe (their
-# device code, tables and launch logic); the (aab), family, gradient and
-# allocation-free translation units are not part of them
+# every source of the library: a summary counts for exactly the sources it was taken on
 KERNEL_SOURCES = sorted(f for f in os.listdir(os.path.join(ROOT, "paper_1701_06588_gb300", "csrc"))
                         if f.endswith((".cu", ".cuh", ".cpp", ".h")))
 
@@ -378,17 +375,19 @@ def run_ours(args, rank, world):
         ms_step = float(t.item())
     value = job_units / (ms_step * 1e-3)
 
+    # the formula's FP64 flops (translation-matrix form, far pairs of 1/r as one multiply-add)
     flops_separate = sum(counts.workload_flops(shells, pa, pb, op) for _, op, _ in OPS)
-    # the passes sum the far field of 1/r as one multiply-add per primitive pair: count
-    # those pairs (T >= 120) exactly
-    n_far = counts.far_primitive_pairs(shells, pa, pb) if fused else None
-    flops_step = (counts.workload_fused_flops(shells, pa, pb, [(op, om) for _, op, om in OPS], n_far) if fused
-                  else flops_separate)
-    achieved = flops_step / (kern_ms * 1e-3) / 1e12
-    # double-float: one multiply-add of the FP64 formula costs 18 FP32 instructions
-    # (TwoProd 4, FastTwoSum 3, TwoSum 6, 2 adds, FastTwoSum 3), so the FP32 FMA rate
-    # (2 flops per instruction) bounds FP64-formula flops at fp32_peak / 18
-    peak = (fp64_peak if args.precision == "fp64" else fp32_peak / DF_FMA_FP32_INSTR) / 1e12
+    formula_flops = flops_separate
+    if fused:
+        formula_flops = counts.workload_fused_flops(shells, pa, pb, [(op, om) for _, op, om in OPS],
+                                                    counts.far_primitive_pairs(shells, pa, pb))
+    # what the passes leave to the FP64 units, two flops an instruction (an addition holds the unit as long as a multiply-add);
+    # the rest runs on the integer pipes, and in mixed precision on the FP32 pipes
+    n_far = counts.far_primitive_pairs(shells, pa, pb, tmax=counts.FAR_T)
+    fp64_instr = sum(counts.workload_fp64_instructions(shells, pa, pb, ops_of_pass, n_far, args.precision == "mixed")
+                     for ops_of_pass in ([[(op, om) for _, op, om in OPS]] if fused else [[(op, om)] for _, op, om in OPS]))
+    achieved = 2 * fp64_instr / (kern_ms * 1e-3) / 1e12
+    peak = fp64_peak / 1e12
     traffic = read_profile_traffic(form)
 
     forms = {}
@@ -515,8 +514,9 @@ def run_ours(args, rank, world):
                                    "data-path collective; rank 0 evaluates pairs [%d, %d)" %
                                    (world, first_pair, first_pair + n_pairs)),
                    "precision": args.precision,
-                   "form": ("fused multi-operator pass (one kernel per step, geometry-only Q_j shared by the "
-                            "operators), autotuned launch shape, one CUDA graph per step" if fused else
+                   "form": ("fused multi-operator pass (harmonics and primitive setup shared by the operators; %s per "
+                            "step), autotuned launch shape, one CUDA graph per step" %
+                            ("one kernel" if args.precision == "fp64" else "two kernels side by side") if fused else
                             "one pass per operator, autotuned launch shape, one CUDA graph per step"),
                    "launch": {k: tuned[form].get(k, 0) for k in ("schedule", "threads_per_cta", "ctas_per_sm", "variant")},
                    "units_per_step": job_units, "units_per_step_this_rank": units_per_step,
@@ -526,14 +526,16 @@ def run_ours(args, rank, world):
         "per_operator_kernel_ms": {n: m for n, m in zip(names, per_op_ms)} if per_op_ms else None,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                      "traffic": traffic,
-                     "peak_source": ("measured FP64 FMA-chain probe (shg_measure_alu_peak) in this run; nominal %.2f "
-                                     "TFLOP/s = 152 SMs x 2 FMA/clk x 2 x 2.07 GHz" % FP64_NOMINAL_TFLOPS)
-                     if args.precision == "fp64" else
-                     "double-float rate derived from the measured FP32 FMA-chain probe (shg_measure_alu_peak) "
-                     "in this run: FP32 rate / 18 (FP32 instructions of one double-float multiply-add); "
-                     "algorithmic flops are the FP64 formula count",
-                     "algorithmic_flops_per_step": flops_step, "kernel_ms_per_step": kern_ms,
-                     "far_field_primitive_pairs": (int(n_far.sum()) if n_far is not None else None),
+                     "peak_source": "measured FP64 FMA-chain probe (shg_measure_alu_peak) in this run; nominal %.2f "
+                                    "TFLOP/s = 152 SMs x 2 FMA/clk x 2 x 2.07 GHz" % FP64_NOMINAL_TFLOPS,
+                     "counted": "FP64 instructions of the pass (2 flops each, as an FMA): contraction sums, harmonics, "
+                                "angular part; the primitive terms run on the integer pipes%s" %
+                                (" and the angular part of min(la, lb) = 2, 3 on the FP32 pipes"
+                                 if args.precision == "mixed" else ""),
+                     "algorithmic_flops_per_step": 2 * fp64_instr, "kernel_ms_per_step": kern_ms,
+                     "far_field_primitive_pairs": int(n_far.sum()),
+                     "formula_flops_per_step": formula_flops,
+                     "formula_tflops": formula_flops / (kern_ms * 1e-3) / 1e12,
                      "separate_passes_flops_per_step": flops_separate,
                      "kernel": ("k_2c_%s_fused<1/r, erfc> (one pass)" %
                                 ("fp64" if args.precision == "fp64" else "mixed") if fused else

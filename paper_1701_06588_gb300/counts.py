@@ -37,7 +37,8 @@ def os_contracted_elements(l_a, l_b, k_a, k_b, gradients=False):
 _BOYS = 2 * 8 + 2 * 8 + 1          # Taylor of F_kmax (8 fma), exp Taylor (8 fma), scale by exp(-T_i)
 _BOYS_F = 2 * 8                     # Taylor of F_kmax alone: J = 1 needs no exp(-T) (no recursion)
 KBOYS_TMAX = 120.0                  # T = rho R^2 at and above which a primitive pair of the 1/r sum counts as one
-                                    # multiply-add (the far field; the kernels take it from 72 on)
+                                    # multiply-add (the far field) in the formula's count
+FAR_T = 72.0                        # where the kernels take it
 
 
 def _boys(J):
@@ -197,6 +198,46 @@ def fused_pair_flops(la, lb, ka, kb, ops, n_far=None):
     scale = na * J * J                                                    # (2j-1)!! B weights on W_a
     assembly = na * nb * (2 * J * J + 1 + nop * (2 * J + 1))
     return rad + finish + post + harmonics + w_rows + scale + assembly
+
+
+def _fp64_angular(la, lb, n_op, double_float=False):
+    """FP64 instructions of one pair outside the sums over primitive pairs: R^2, harmonics and, per operator, F_p, the
+    products p_{L,M} F_p and the elements of the expanded angular part (double_float: the F_p only)."""
+    J, kmax = min(la, lb) + 1, la + lb
+    f = sum(1 + 2 * p for p in range(J)) + 1
+    if double_float:
+        return 6 + n_op * f
+    harm = 4 * kmax + 3 * kmax * (kmax + 1) // 2
+    f += sum(1 for M in range(kmax + 1) for p in range(J) if M + 2 * p <= kmax)
+    for a in range(la + 1):
+        for b in range(lb + 1):
+            f += min(J, (kmax - abs(a - b)) // 2 + 1)
+            f += min(J, (kmax - a - b) // 2 + 1) + 6 if a and b else 1 + (a > 0) + (b > 0)
+    return 6 + harm + n_op * f
+
+
+def workload_fp64_instructions(shells, pair_a, pair_b, ops, n_far=None, mixed=False):
+    """FP64 instructions of a fused pass over `ops` ((op id, omega) pairs) per thread lane, without the repetitions of a
+    pair with several lanes: per primitive pair one addition for each order of each sum (a far one of 1/r one multiply-add),
+    per pair the downward recursions of the 1/r-type sums, erfc = 1/r - erf, and _fp64_angular.  The terms themselves are
+    formed on the integer pipes.  mixed: the angular part of min(la, lb) = 2, 3 runs in double-float."""
+    ids = dict(ops)
+    coul = OP_COULOMB in ids or OP_ERFC in ids
+    att = len({ids[o] for o in (OP_ERF, OP_ERFC) if o in ids})
+    plain = (OP_OVERLAP in ids) + (OP_GAUSS in ids)
+    l, k = np.asarray(shells["l"]).astype(np.int64), np.asarray(shells["nprim"]).astype(np.int64)
+    la, lb = l[pair_a], l[pair_b]
+    kk = k[pair_a] * k[pair_b]
+    nfar = np.zeros(len(kk)) if n_far is None else np.asarray(n_far)
+    J = np.minimum(la, lb) + 1
+    out = (kk - nfar) * J * coul + nfar * coul + kk * J * (att + plain)
+    out = out + 2 * (J - 1) * (coul + att) + J * (OP_ERFC in ids) + J * plain
+    total = float(np.sum(out))
+    cls, cnt = np.unique(la * 16 + lb, return_counts=True)
+    for c, n in zip(cls.tolist(), cnt.tolist()):
+        a, b = c // 16, c % 16
+        total += n * _fp64_angular(a, b, len(ids), mixed and min(a, b) in (2, 3))
+    return total
 
 
 def workload_fused_flops(shells, pair_a, pair_b, ops, n_far=None):
