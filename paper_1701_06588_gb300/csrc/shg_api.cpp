@@ -603,12 +603,17 @@ const Consts &consts()
     return k;
 }
 
-static void fill_kappa_mix(KappaMix &k)
+static const KappaMix &kappa_mix()
 {
-    for (int n = 0; n < 32; ++n) k.inv[n] = n ? split2(1.0L / n) : make_float2(0, 0);
-    for (int l = 0; l < 16; ++l)
-        for (int m = 0; m < 16; ++m)
-            k.v[l][m] = l && m <= l ? split2((long double)(l * l - m * m) / (4 * l * l - 1)) : make_float2(0, 0);
+    static KappaMix k;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        for (int n = 0; n < 32; ++n) k.inv[n] = n ? split2(1.0L / n) : make_float2(0, 0);
+        for (int l = 0; l < 16; ++l)
+            for (int m = 0; m < 16; ++m)
+                k.v[l][m] = l && m <= l ? split2((long double)(l * l - m * m) / (4 * l * l - 1)) : make_float2(0, 0);
+    });
+    return k;
 }
 
 static bool is_finite_d(double x) { return std::isfinite(x); }
@@ -1305,7 +1310,7 @@ static int exec_short(shg_plan_t *p, const ArgsFused &f, bool mixed, cudaStream_
     for (int op = 0; op < 6; ++op) ops |= f.out[op] ? 1u << op : 0u;
     const bool split = pass_parts(p->d, ops) > 1;
     ArgsMixFused m;
-    if (mixed) fill_kappa_mix(m.kappa);
+    if (mixed) m.kappa = kappa_mix();
     bool beside = false;
     for (int op = 0; op < 6; ++op) {
         if (!f.out[op] || (pair && op == SHG_OP_ERFC)) continue;
@@ -1376,7 +1381,7 @@ static int exec_mixed(shg_plan_t *p, const ArgsFused &f, cudaStream_t s)
 {
     ArgsMixFused m;
     m.f = f;
-    fill_kappa_mix(m.kappa);
+    m.kappa = kappa_mix();
     ArgsFused a = f;
     if (p->d.schedule == SHG_SCHED_PERSISTENT) {
         if (p->d.n_tiles <= kStaticTiles) return exec_short(p, f, true, s);
@@ -1633,7 +1638,7 @@ int shg_eval_2c_grad(const shg_basis_t *basis, int64_t n, const int32_t *pa, con
     // fused_ops reads the wanted sums off the outputs
     a.f.r.want = want_of(op);
     fused_plan(a.f, basis->d, p->d, *t, w_off);
-    fill_kappa_mix(a.kappa);
+    a.kappa = kappa_mix();
     a.w = w;
     a.grad_a = grad_a;
     a.grad_b = grad_b;
