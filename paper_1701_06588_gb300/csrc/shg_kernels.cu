@@ -1,13 +1,14 @@
 // CUDA kernels of the SHG integral library (sm_103a): FP64 two-center passes of (a|r_a^{2n}|b) and of
-// precomputed radial terms (the other operators: shg_pair2c.cuh), planning kernels, Boys debug kernel and the ALU throughput probe.
+// precomputed radial terms (the other operators: shg_pair2c.cuh), planning kernels, Boys debug kernel and the ALU
+// throughput probe.
 //
-// Two-center integrals follow Sec. II B of Golze et al. (arXiv:1701.06588):
+// The (a|r_a^{2n}|b) blocks follow Sec. II B of Golze et al. (arXiv:1701.06588):
 //   (a|O|b) = (-1)^lb A_{la,ma} A_{lb,mb} sum_j 2^{la+lb-j} O^{(la+lb-j)}
 //             (2j-1)!! sum_kappa B_{j,kappa} Q^{c/s,c/s}_{la,|ma|,lb,|mb|,j,kappa}
 // with Q = W_a W_b^T (Eq. Q_matrix), W built from the regular scaled solid
 // harmonics R^{c/s}_{l,m} of the vector R_a - R_b (Sec. II E), and
 // O^{(k)} = sum_{alpha,beta} w_alpha w_beta (d/dR^2)^k (0_a|O|0_b)  (Eq. O_rab2_deriv,
-// Table S1).
+// with T^{(k)} of Eq. T_rab2_deriv in place of Table S1); precomputed radial terms take the angular part of shg_cg.cuh.
 //
 // Work mapping: one thread evaluates one shell pair (radial terms of every
 // primitive pair in registers, then the (2la+1)(2lb+1) block); a warp owns a
@@ -75,7 +76,7 @@ __device__ __forceinline__ ddv rsd_get(const ddv *Rs, int L, int m)
     return (m < 0 && !(am & 1)) ? dd_neg(v) : v;
 }
 
-// scaled_harmonics with double-double arithmetic and constants
+// regular scaled solid harmonics R^{c/s}_{l,m} (Sec. II E) in double-double
 __device__ void scaled_harmonics_dd(ddv x, ddv y, ddv z, int lmax, const Consts &k, ddv *Rc, ddv *Rs)
 {
     const ddv r2 = dd_add(dd_add(dd_mul(x, x), dd_mul(y, y)), dd_mul(z, z));
@@ -132,7 +133,7 @@ __device__ __forceinline__ void w_row_dd(const ddv *Rc, const ddv *Rs, int l, in
 }
 
 // Radial orders of one primitive pair, accumulated in double-double into
-// O[j] = O^{(kmax-j)} (the FP64 radial_acc_fp64<OP_RA2N> with the Horner
+// O[j] = O^{(kmax-j)} (radial_acc_ra2n with the Horner
 // variable R^2 and the accumulation kept in double-double).
 template <int J>
 __device__ __forceinline__ void radial_ra2n_dd(const PrimRec &pa, const PrimRec &pb, ddv R2d, int kmax, int la,
