@@ -21,8 +21,8 @@ constexpr int kTile = 32;         // pairs per warp tile
 // of the largest term); below, the FP64 units, which are otherwise a third busy, take the few sums sooner than the FP32
 // pipes take 18 instructions for each: 1M pairs, 1/r and erfc, 2.92 ms with all classes below 4 in double-float, 2.53 ms
 // from 2 or from 3 on; 123,000 pairs, erfc, 596, 439 (from 2) and 466 us (from 3); 250,000 gradients of erfc 1.22, 1.16 and
-// 1.09 ms.  Between these two limits double-float gains nothing over FP64 for every class either (1M pairs 2.49 ms, the
-// 2M-pair step 4.93 against 4.85, 500,000 gradients of erfc 1.99 against 1.95): the classes kept are those where it loses
+// 1.09 ms.  Between these two limits double-float gains nothing over FP64 for every class either (1M pairs 2.48 ms, the
+// 2M-pair step 4.92 against 4.84, 500,000 gradients of erfc 1.97 against 1.93): the classes kept are those where it loses
 // least.
 constexpr int kMixedDfMinL = 2, kMixedDfMinLGrad = 3, kMixedFp64MinL = 4;
 inline int min_l(int cls) { return cls / 7 < cls % 7 ? cls / 7 : cls % 7; }
